@@ -15,6 +15,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/stokes_mg.h"
+#include "cluster_cycle.cuh"
 #include "coef.h"
 #include "elements.h"
 #include "kernels.cuh"
@@ -181,7 +182,9 @@ struct stokes_handle_t {
     double* hscal = nullptr;                // pinned host mirror
     MassCoef<double> mass{};
     OpCoef<float> chi{}, clo{};             // MIXED: finest float64 coefficients split hi + lo
-    bool coarse_kernel = true;              // float32 levels <= 4 in one shared-memory kernel
+    int cl_top = -1;                        // levels clev+1..cl_top: one thread-block cluster per visit
+    ClusterTables<float>* cl_tab32 = nullptr;   // device: what its threads sum (MIXED, FP64)
+    ClusterTables<double>* cl_tab64 = nullptr;
     bool launch_failed = false;             // a step variant refused to launch (reported by the next call)
     bool has_planar = false;                // some float32 level is planar
     int small_top = -1;                     // float32 levels clev+1..small_top: one cooperative launch per visit
@@ -294,10 +297,74 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
     return sw;
 }
 
-// Sec. 3: one multigrid iteration on level l of hierarchy H (x = (u, p), F = (f, g) of the level);
-// the iterate is in (u, p) on entry and on exit.
+// The operations of one iteration on level l (cluster_cycle.cuh); an exact coarsest solve repeated with
+// the same right-hand side (W-cycle) would return the same values, so it is listed once.
+void cluster_list(const stokes_handle* h, int l, bool zero, std::vector<unsigned char>& ops) {
+    if (l == h->clev) {
+        ops.push_back(cluster_op(kOpCoarse, l));
+        return;
+    }
+    if (zero && h->prm.nu_pre == 0) ops.push_back(cluster_op(kOpClear, l));
+    ops.push_back(cluster_op(zero ? kOpPreZero : kOpPre, l));
+    ops.push_back(cluster_op(kOpRestrict, l));
+    for (int r = 0; r < (l - 1 == h->clev ? 1 : h->prm.gamma); ++r) cluster_list(h, l - 1, r == 0, ops);
+    ops.push_back(cluster_op(kOpProlong, l));
+    ops.push_back(cluster_op(kOpPost, l));
+}
+
+// One iteration on level l <= cl_top from its (u, p) (from zero, whatever they hold, when `zero`), by the
+// cluster kernel: one launch, or, when the coarsest level's dense inverse is too large for one cluster,
+// one launch up to each coarsest solve and between two of them.
 template <typename T>
-void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l) {
+void cluster_visit(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero) {
+    ClusterHost<T> c{};
+    for (int k = h->clev; k <= l; ++k) {
+        Level<T>& L = H[k];
+        c.u[k] = L.u;
+        c.p[k] = L.p;
+        c.f[k] = L.f;
+        c.g[k] = L.g;
+        c.sinv[k] = L.sinv;
+    }
+    if constexpr (sizeof(T) == 4) c.tab = h->cl_tab32;
+    else c.tab = h->cl_tab64;
+    c.inv0 = h->inv;
+    c.cinv = h->cinv;
+    c.cnb = h->cnb;
+    c.sigma = (T)h->prm.sigma;
+    c.nu_pre = h->prm.nu_pre;
+    c.nu_post = h->prm.nu_post;
+    c.top = l;
+    c.lo = h->clev;
+    c.dom = h->dom;
+    std::vector<unsigned char> ops;
+    cluster_list(h, l, zero, ops);
+    const bool split = h->cnb - 1 > kClusterMaxNb;
+    const unsigned top = 1u << l, all = (2u << l) - (1u << h->clev), held = all & ~(1u << h->clev);
+    unsigned ld_x = zero ? 0u : top, ld_f = top;
+    std::vector<unsigned char> part;
+    auto launch = [&](unsigned st_x, unsigned st_f) {
+        if (launch_cluster_ops<T>(h->st, c, part, ld_x, ld_f, st_x, st_f) != cudaSuccess) h->launch_failed = true;
+        part.clear();
+    };
+    for (unsigned char o : ops) {
+        if (split && (o & 15) == kOpCoarse) {
+            launch(held, all & ~top);
+            Level<T>& C = H[h->clev];
+            launch_dense_solve<T>(h->st, C.n, h->cinv, h->cnb, C.f, C.g, C.u, C.p);
+            ld_x = all;
+            ld_f = held;
+        } else {
+            part.push_back(o);
+        }
+    }
+    launch(top, 0u);
+}
+
+// Sec. 3: one multigrid iteration on level l of hierarchy H (x = (u, p), F = (f, g) of the level);
+// the iterate is in (u, p) on entry and on exit; `zero`: it is zero on entry.
+template <typename T>
+void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = false) {
     Level<T>& lv = H[l];
     if (l == h->clev) {   // the coarsest level of the iteration: exact solve (Sec. 3)
         if (l == 0) launch_coarse_solve<T>(h->st, h->inv, lv.f, lv.g, lv.u, lv.p);
@@ -334,27 +401,10 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l) {
             if (launch_small_cycle(h->st, sh) != cudaSuccess) h->launch_failed = true;
             return;
         }
-        // small levels: the whole V-cycle from level l down in one CTA (shared memory)
-        if (l <= kCoarseCycleTop && h->prm.gamma == 1 && h->prm.smoother == STOKES_UZAWA && h->coarse_kernel &&
-            h->clev == 0) {
-            CoarseCycleArgs a;
-            for (int k = 1; k <= l; ++k) {
-                a.c[k - 1] = H[k].c;
-                a.sinv[k - 1] = H[k].sinv;
-            }
-            a.inv = h->inv;
-            a.u = lv.u;
-            a.p = lv.p;
-            a.f = lv.f;
-            a.g = lv.g;
-            a.tau = (float)h->prm.tau;
-            a.sigma = (float)h->prm.sigma;
-            a.nu_pre = h->prm.nu_pre;
-            a.nu_post = h->prm.nu_post;
-            a.top = l;
-            launch_coarse_cycle(h->st, a);
-            return;
-        }
+    }
+    if (l <= h->cl_top && !lv.planar) {
+        cluster_visit<T>(h, H, l, zero);
+        return;
     }
     const bool top = l == (int)H.size() - 1;
     bool sw = smooth_level(h, lv, h->prm.nu_pre, top, false);
@@ -364,6 +414,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l) {
     T* ru = sw ? lv.u : lv.tu;
     T* rp = sw ? lv.p : lv.tp;
     Level<T>& cl = H[l - 1];
+    const int visits = l - 1 == h->clev ? 1 : h->prm.gamma;   // a second exact solve would return the same values
     if constexpr (sizeof(T) == 4) {
         if (lv.planar) {
             // the defect and its restriction in one kernel on the staged tiles (the defect stays on chip)
@@ -371,7 +422,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l) {
                 launch_residual_planar(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp);
                 launch_restrict_planar(h->st, cl.n, cl.planar, ru, rp, cl.f, cl.g, cl.u, cl.p);
             }
-            for (int r = 0; r < h->prm.gamma; ++r) mg_cycle(h, H, l - 1);
+            for (int r = 0; r < visits; ++r) mg_cycle(h, H, l - 1, r == 0);
             if (h->fuse_prolong && h->prm.nu_post > 0) fused_coarse = &cl;
             else launch_prolong_add_planar(h->st, cl.n, cl.planar, cl.u, cl.p, xu, xp);
         }
@@ -379,7 +430,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l) {
     if (!lv.planar) {
         launch_residual<T, T>(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp, nullptr, nullptr, nullptr, h->dom);
         launch_restrict<T>(h->st, cl.n, ru, rp, cl.f, cl.g, cl.u, cl.p, h->dom);   // and the coarse iterate := 0
-        for (int r = 0; r < h->prm.gamma; ++r) mg_cycle(h, H, l - 1);
+        for (int r = 0; r < visits; ++r) mg_cycle(h, H, l - 1, r == 0);
         launch_prolong_add<T>(h->st, cl.n, cl.u, cl.p, xu, xp, h->dom);
     }
     sw = smooth_level(h, lv, h->prm.nu_post, top, sw, fused_coarse);
@@ -415,7 +466,7 @@ void record_step(stokes_handle* h) {
         Level<float>& E = h->h32.back();
         cudaMemsetAsync(E.u, 0, 2 * E.n2 * sizeof(float), h->st);
         cudaMemsetAsync(E.p, 0, E.n1 * sizeof(float), h->st);
-        for (int c = 0; c < h->prm.inner_cycles; ++c) mg_cycle<float>(h, h->h32, h->L - 1);
+        for (int c = 0; c < h->prm.inner_cycles; ++c) mg_cycle<float>(h, h->h32, h->L - 1, c == 0);
         // x += e, r -= A e (two-float residual, error-free float32 products), r32 = float(r)
         const int k = ev_begin(h, kEvResid);
         if (k >= 0) h->ev_resid++;
@@ -537,6 +588,18 @@ void collect_timing(stokes_handle* h) {
     }
 }
 
+// The cluster cycle's lists for the levels' current operators.
+template <typename T>
+stokes_status upload_cluster_tables(stokes_handle* h, const std::vector<Level<T>>& H, ClusterTables<T>* dst) {
+    std::vector<ClusterTables<T>> t(1);   // on the heap
+    bool ok = fill_cluster_xfer(t[0].x);
+    for (int k = 1; k <= h->cl_top && ok; ++k) ok = fill_cluster_level(t[0].L[k], H[k].n, H[k].c, (T)h->prm.tau);
+    if (!ok) return STOKES_ERR_BAD_ARG;
+    CK(cudaMemcpyAsync(dst, t.data(), sizeof(ClusterTables<T>), cudaMemcpyHostToDevice, h->st));
+    CK(cudaStreamSynchronize(h->st));
+    return STOKES_OK;
+}
+
 stokes_status rebuild_beta(stokes_handle* h) {
     const double beta = h->prm.beta;
     for (auto& lv : h->h64) {
@@ -552,6 +615,11 @@ stokes_status rebuild_beta(stokes_handle* h) {
         if (lv.planar && !reg_tables_match(lv.c)) return STOKES_ERR_BAD_ARG;
         launch_schur_diag<float>(h->st, lv.n, make_coef<double>(lv.n, beta), lv.sinv, h->dom,
                                  lv.planar ? pl_vpitch(lv.n) : 0);
+    }
+    if (h->cl_top > 0) {
+        const stokes_status s = h->mixed() ? upload_cluster_tables(h, h->h32, h->cl_tab32)
+                                           : upload_cluster_tables(h, h->h64, h->cl_tab64);
+        if (s != STOKES_OK) return s;
     }
     if (h->mixed()) {
         const OpCoef<double>& c = h->fin().c;
@@ -693,7 +761,7 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
     stokes_status s = ensure_weights();
     if (s != STOKES_OK) return s;
     if (prepare_uzawa_fused<float>() != cudaSuccess || prepare_uzawa_fused<double>() != cudaSuccess ||
-        prepare_coarse_cycle() != cudaSuccess || prepare_uzawa_pair() != cudaSuccess ||
+        prepare_uzawa_pair() != cudaSuccess ||
         prepare_uzawa_reg() != cudaSuccess || prepare_dense_solve(bordered_size(1 << (kMaxCoarseLevel + 1))) != cudaSuccess)
         return STOKES_ERR_CUDA;
     stokes_handle* h = new stokes_handle_t();
@@ -741,6 +809,19 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
                     cudaGetLastError();
                     return bail(STOKES_ERR_OOM);
                 }
+            }
+        }
+    }
+    // the cluster cycle of the small levels: Uzawa smoother, at least one level above the coarsest
+    if (P.smoother == STOKES_UZAWA) {
+        const bool f32 = P.precision == STOKES_MIXED;
+        const int ctop = std::min(P.levels - 1, f32 ? cluster_top<float>() : cluster_top<double>());
+        if (ctop > P.coarse_level && (f32 ? prepare_cluster_cycle<float>() : prepare_cluster_cycle<double>())) {
+            h->cl_top = ctop;
+            if ((f32 ? h->mem.get(&h->cl_tab32, sizeof(ClusterTables<float>))
+                     : h->mem.get(&h->cl_tab64, sizeof(ClusterTables<double>))) != cudaSuccess) {
+                cudaGetLastError();
+                return bail(STOKES_ERR_OOM);
             }
         }
     }

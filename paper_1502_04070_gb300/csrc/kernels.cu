@@ -316,17 +316,10 @@ __device__ __forceinline__ void restrict_rows(const T (&v)[2][4][4], T (&acc)[2]
     }
 }
 
-// global arrays go through the read-only path; shared-memory arrays (the coarse sub-cycle) do not
-template <bool LDG, typename T>
-__device__ __forceinline__ T ldv(const T* p) {
-    if constexpr (LDG) return __ldg(p);
-    else return *p;
-}
-
-// Strides of the arrays a transfer reads and writes, each pointer at the array's (0, 0) entry:
-// the dense level arrays (dense_layout), the padded shared-memory arrays of the coarse cycle, or
-// float32 levels in the planar layout (template flags PF / PC of the fine / coarse level; there the
-// row stride is in floats, the component stride is 1 and psf / psc is the parity-plane stride).
+// Strides of the arrays a transfer reads and writes, each pointer at the array's (0, 0) entry: the dense
+// level arrays (dense_layout), or float32 levels in the planar layout (template flags PF / PC of the
+// fine / coarse level; there the row stride is in floats, the component stride is 1 and psf / psc is the
+// parity-plane stride).
 struct XferLayout {
     int ldf, n2f;   // fine velocity: row stride, component stride
     int ldpf;       // fine vertex array: row stride
@@ -362,7 +355,7 @@ __host__ __device__ __forceinline__ int lat_at(int X, int Y, int ld, int ps) {
     else return Y * ld + X;
 }
 
-template <int SQ, bool LDG, bool PF, typename T>
+template <int SQ, bool PF, typename T>
 __device__ __forceinline__ void restrict_visit(int I, int J, int nc, const T* __restrict__ ru, T (&acc)[2][4],
                                                const XferLayout& lay) {
     const int SI = I - (SQ & 1), SJ = J - (SQ >> 1);
@@ -373,25 +366,25 @@ __device__ __forceinline__ void restrict_visit(int I, int J, int nc, const T* __
 #pragma unroll
         for (int fa = 0; fa < 4; ++fa) {
             const int k = lat_at<PF>(4 * SI + fa, 4 * SJ + fb, lay.ldf, lay.psf);
-            v[0][fb][fa] = ldv<LDG>(ru + k);
-            v[1][fb][fa] = ldv<LDG>(ru + lay.n2f + k);
+            v[0][fb][fa] = __ldg(ru + k);
+            v[1][fb][fa] = __ldg(ru + lay.n2f + k);
         }
     if (orient(SI, SJ, nc)) restrict_rows<1, SQ, 0>(v, acc);
     else restrict_rows<0, SQ, 0>(v, acc);
 }
 
 // coarse cell (i, j) of level nc: its owned coarse velocity nodes and vertex
-template <bool LDG, typename T, bool PF = false, bool PC = false>
+template <typename T, bool PF, bool PC>
 __device__ __forceinline__ void restrict_cell(int i, int j, int nc, const T* __restrict__ ru, const T* __restrict__ rp,
                                               T* __restrict__ fc, T* __restrict__ gc, const XferLayout& lay,
                                               int dom = kDomSquare) {
     T acc[2][4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) acc[0][s] = acc[1][s] = T(0);
-    restrict_visit<0, LDG, PF>(i, j, nc, ru, acc, lay);
-    restrict_visit<1, LDG, PF>(i, j, nc, ru, acc, lay);
-    restrict_visit<2, LDG, PF>(i, j, nc, ru, acc, lay);
-    restrict_visit<3, LDG, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<0, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<1, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<2, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<3, PF>(i, j, nc, ru, acc, lay);
     const CellNodes cn = cell_nodes_dom(i, j, nc, dom);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -434,7 +427,7 @@ __global__ void __launch_bounds__(NT) k_restrict(int nc, const T* __restrict__ r
     CELL_INDEX
     if (!active) return;
     const XferLayout lay = xfer_layout(nc, PF, PC);
-    restrict_cell<true, T, PF, PC>(i, j, nc, ru, rp, fc, gc, lay, dom);
+    restrict_cell<T, PF, PC>(i, j, nc, ru, rp, fc, gc, lay, dom);
     if (uc) {
         const CellNodes cn = cell_nodes(i, j, nc);
 #pragma unroll
@@ -469,7 +462,7 @@ void launch_restrict_planar(cudaStream_t s, int nc, bool pc_planar, const float*
 // Prolongation (Sec. 3, canonical embedding): every fine point owned by coarse square (I, J) is
 // the coarse P2 function of that square evaluated there; P1 values are vertex injection and
 // averages along coarse edges.
-template <bool LDG, typename T, bool PF = false, bool PC = false>
+template <typename T, bool PF, bool PC>
 __device__ __forceinline__ void prolong_cell(int i, int j, int nc, const T* __restrict__ uc, const T* __restrict__ pc,
                                              T* __restrict__ u, T* __restrict__ p, const XferLayout& lay,
                                              int dom = kDomSquare) {
@@ -479,8 +472,8 @@ __device__ __forceinline__ void prolong_cell(int i, int j, int nc, const T* __re
 #pragma unroll
         for (int m = 0; m < 9; ++m) {
             const int k = lat_at<PC>(2 * i + m % 3, 2 * j + m / 3, lay.ldc, lay.psc);
-            z[0][m] = ldv<LDG>(uc + k);
-            z[1][m] = ldv<LDG>(uc + lay.n2c + k);
+            z[0][m] = __ldg(uc + k);
+            z[1][m] = __ldg(uc + lay.n2c + k);
         }
         const int o = orient(i, j, nc);
 #pragma unroll
@@ -502,7 +495,7 @@ __device__ __forceinline__ void prolong_cell(int i, int j, int nc, const T* __re
             }
     }
     const int ldp = lay.ldpc, ldpf = lay.ldpf;
-    auto P = [&](int a, int b) { return ldv<LDG>(pc + (b * ldp + a)); };
+    auto P = [&](int a, int b) { return __ldg(pc + (b * ldp + a)); };
     const T p00 = P(i, j);
     // on the L, fine vertices strictly inside the removed quadrant keep their zero
     auto live = [&](int x, int y) { return !(dom == kDomL && l_masked_vertex(x, y, nf)); };
@@ -522,7 +515,7 @@ __global__ void __launch_bounds__(NT) k_prolong(int nc, const T* __restrict__ uc
     const int n = nc;
     CELL_INDEX
     if (!active) return;
-    prolong_cell<true, T, PF, PC>(i, j, nc, uc, pc, u, p, xfer_layout(nc, PF, PC), dom);
+    prolong_cell<T, PF, PC>(i, j, nc, uc, pc, u, p, xfer_layout(nc, PF, PC), dom);
     pdl_trigger();
 }
 
@@ -939,8 +932,6 @@ void launch_mask_l(cudaStream_t s, int n, double* u, double* p) {
     const int blocks = std::min((ld * ld + 255) / 256, 4096);
     k_mask_l<<<blocks, 256, 0, s>>>(n, u, p);
 }
-
-#include "coarse_cycle.cuh"
 
 // ------------------------------------------------------------------------------------------
 #define INST(T)                                                                                         \

@@ -13,8 +13,8 @@
 // the vertex row of B^T vanishes, and every entry of B and B^T is +-b or +-b/2 for one b ~ h.  The
 // kernel therefore keeps the eight A values as (a, a) pairs in sixteen registers, applies each A
 // term with one packed FP32x2 FMA on the (u_x, u_y) pair, and forms B u and B^T p as sums with the
-// literal weights +-1, +-1/2, scaled once by b.  The structure is a compile-time table (below),
-// checked against the level's assembled coefficients on the host before every launch
+// literal weights +-1, +-1/2, scaled once by b.  The structure is a compile-time table
+// (stencil_tables.cuh), checked against the level's assembled coefficients on the host before every launch
 // (make_reg_coef).
 //
 // Data movement: a CTA owns a 28 x ty tile of cells and stages, with asynchronous 4-byte copies
@@ -32,53 +32,10 @@
 #include "cellops.cuh"
 #include "elements.h"
 #include "kernels.cuh"
+#include "stencil_tables.cuh"
 #include "tiles.cuh"
 
 namespace smg {
-namespace {
-
-// ---------------------------------------------------------------------------------------------
-// Structure of the merged stencils of the orientation classes 0 and 1 (common.cuh), by window
-// point w = (dy + 2) * 5 + dx + 2 of the 5 x 5 lattice window around the cell's vertex (2i, 2j)
-// and owned node s (0 V, 1 H, 2 E, 3 C):
-//   kGid[cls][s][w]  group of the A coefficient (-1: zero); every group holds one value
-//   kBx / kBy[cls][w]  the vertex's B row in units of b/2 (values 0, +-1, +-2)
-//   kBTx / kBTy[cls][s][v]  the B^T rows over the 3 x 3 vertex window v = (dj + 1) * 3 + di + 1,
-//                           in units of b/2
-constexpr int kGroups = 8;
-constexpr int kGidDiagV = 4, kGidDiagE = 7;   // groups of the diagonal of the V row and of the H, E, C rows
-constexpr signed char kGid[2][4][25] = {
-    {{0, 1, 2, -1, -1, 1, -1, 3, 1, -1, 2, 3, 4, 3, 2, -1, 1, 3, -1, 1, -1, -1, 2, 1, 0},
-     {-1, -1, 1, -1, -1, -1, -1, 5, 6, -1, -1, -1, 3, 7, 3, -1, -1, -1, 6, 5, -1, -1, -1, -1, 1},
-     {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 1, 5, 3, -1, -1, -1, 6, 7, 6, -1, -1, -1, 3, 5, 1},
-     {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 6, 1, -1, -1, 6, 7, 6, -1, -1, 1, 6, -1}},
-    {{-1, -1, 0, 1, 2, -1, 1, 3, -1, 1, 0, 3, 4, 3, 0, 1, -1, 3, 1, -1, 2, 1, 0, -1, -1},
-     {-1, -1, -1, -1, 1, -1, -1, -1, 5, 6, -1, -1, 3, 7, 3, -1, -1, 6, 5, -1, -1, -1, 1, -1, -1},
-     {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 3, 6, 1, -1, 5, 7, 5, -1, 1, 6, 3, -1, -1},
-     {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 1, 5, -1, -1, -1, 5, 7, 5, -1, -1, -1, 5, 1}}};
-constexpr signed char kBx[2][25] = {
-    {0, 0, 0, 0, 0, -1, -1, 1, 1, 0, 0, -2, 0, 2, 0, 0, -1, -1, 1, 1, 0, 0, 0, 0, 0},
-    {0, 0, 0, 0, 0, 0, -1, -1, 1, 1, 0, -2, 0, 2, 0, -1, -1, 1, 1, 0, 0, 0, 0, 0, 0}};
-constexpr signed char kBy[2][25] = {
-    {0, -1, 0, 0, 0, 0, -1, -2, -1, 0, 0, 1, 0, -1, 0, 0, 1, 2, 1, 0, 0, 0, 0, 1, 0},
-    {0, 0, 0, -1, 0, 0, -1, -2, -1, 0, 0, -1, 0, 1, 0, 0, 1, 2, 1, 0, 0, 1, 0, 0, 0}};
-constexpr signed char kBTx[2][4][9] = {
-    {{0, 0, 0, 0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 2, -2, 0, 0, 0}, {0, 0, 0, 1, -1, 0, 0, 1, -1}, {0, 0, 0, 0, 1, -1, 0, 1, -1}},
-    {{0, 0, 0, 0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 2, -2, 0, 0, 0}, {0, 0, 0, 0, 1, -1, 1, -1, 0}, {0, 0, 0, 0, 1, -1, 0, 1, -1}}};
-constexpr signed char kBTy[2][4][9] = {
-    {{0, 0, 0, 0, 0, 0, 0, 0, 0}, {0, 1, 0, 0, -1, 1, 0, 0, -1}, {0, 0, 0, 0, 2, 0, 0, -2, 0}, {0, 0, 0, 0, 1, 1, 0, -1, -1}},
-    {{0, 0, 0, 0, 0, 0, 0, 0, 0}, {0, 0, 1, 0, 1, -1, 0, -1, 0}, {0, 0, 0, 0, 2, 0, 0, -2, 0}, {0, 0, 0, 0, 1, 1, 0, -1, -1}}};
-
-__host__ __device__ constexpr bool a_win(int C, int w) {
-    return kGid[C][0][w] >= 0 || kGid[C][1][w] >= 0 || kGid[C][2][w] >= 0 || kGid[C][3][w] >= 0;
-}
-__host__ __device__ constexpr bool bt_vwin(int C, int v) {
-    for (int s = 0; s < 4; ++s)
-        if (kBTx[C][s][v] != 0 || kBTy[C][s][v] != 0) return true;
-    return false;
-}
-
-}  // namespace
 
 // Values of the structure above for one level (host-built by make_reg_coef)
 struct RegCoef {
@@ -87,54 +44,16 @@ struct RegCoef {
     float b;                // B = (b / 2) x (the integer tables)
 };
 
-// Fills q from the level's merged stencils and checks that they have exactly the compile-time
-// structure (zeros, equal groups, B entries +-b, +-b/2); false if not (the caller then uses
-// another step variant).
+// false if the level's stencils lack the structure (the caller then uses another step variant)
 static bool make_reg_coef(const OpCoef<float>& c, float tau, RegCoef& q) {
-    double amax = 0.0, bmax = 0.0;
+    RegVals<float> v;
+    if (!make_reg_vals(c, tau, v)) return false;
     for (int C = 0; C < 2; ++C) {
-        for (int s = 0; s < 4; ++s)
-            for (int w = 0; w < 25; ++w) amax = std::max(amax, std::fabs((double)c.MA[C][s][w]));
-        for (int w = 0; w < 25; ++w) bmax = std::max({bmax, std::fabs((double)c.MBx[C][w]), std::fabs((double)c.MBy[C][w])});
+        for (int g = 0; g < kGroups; ++g) q.a[C][g] = make_float2(v.a[C][g], v.a[C][g]);
+        q.ti[C][0] = v.ti[C][0];
+        q.ti[C][1] = v.ti[C][1];
     }
-    if (!(amax > 0.0) || !(bmax > 0.0)) return false;
-    const double b = bmax;
-    for (int C = 0; C < 2; ++C) {
-        bool set[kGroups] = {};
-        for (int s = 0; s < 4; ++s)
-            for (int w = 0; w < 25; ++w) {
-                const double v = c.MA[C][s][w];
-                const int gid = kGid[C][s][w];
-                if (gid < 0) {
-                    if (std::fabs(v) > 1e-6 * amax) return false;
-                    continue;
-                }
-                if (!set[gid]) {
-                    q.a[C][gid] = make_float2((float)v, (float)v);
-                    set[gid] = true;
-                } else if (std::fabs(v - (double)q.a[C][gid].x) > 1e-6 * std::fabs(v) + 1e-7 * amax) {
-                    return false;
-                }
-            }
-        for (int g = 0; g < kGroups; ++g)
-            if (!set[g]) return false;
-        for (int w = 0; w < 25; ++w)
-            if (std::fabs(c.MBx[C][w] - 0.5 * b * kBx[C][w]) > 1e-6 * b ||
-                std::fabs(c.MBy[C][w] - 0.5 * b * kBy[C][w]) > 1e-6 * b)
-                return false;
-        for (int s = 0; s < 4; ++s)
-            for (int v = 0; v < 9; ++v)
-                if (std::fabs(c.MBTx[C][s][v] - 0.5 * b * kBTx[C][s][v]) > 1e-6 * b ||
-                    std::fabs(c.MBTy[C][s][v] - 0.5 * b * kBTy[C][s][v]) > 1e-6 * b)
-                    return false;
-        // the diagonal groups are the stored inverse diagonals
-        if (std::fabs(1.0 / q.a[C][kGidDiagV].x - c.MIdg[C][0]) > 1e-6 * std::fabs(c.MIdg[C][0])) return false;
-        for (int s = 1; s < 4; ++s)
-            if (std::fabs(1.0 / q.a[C][kGidDiagE].x - c.MIdg[C][s]) > 1e-6 * std::fabs(c.MIdg[C][s])) return false;
-        q.ti[C][0] = tau * c.MIdg[C][0];
-        q.ti[C][1] = tau * c.MIdg[C][1];
-    }
-    q.b = (float)b;
+    q.b = v.b;
     return true;
 }
 
@@ -243,15 +162,6 @@ struct ULat {
         return ycomp ? e.y : e.x;
     }
 };
-
-// acc += (k / 2) v with a compile-time k in {0, +-1, +-2}
-template <int K>
-__device__ __forceinline__ void addk(float& acc, float v) {
-    if constexpr (K == 2) acc += v;
-    else if constexpr (K == -2) acc -= v;
-    else if constexpr (K == 1) acc = fmaf(0.5f, v, acc);
-    else if constexpr (K == -1) acc = fmaf(-0.5f, v, acc);
-}
 
 // ---- phase 1, fast path: A rows over the u window, B^T rows over the p window
 template <int C, int UWH, int W>
@@ -921,57 +831,6 @@ __device__ __forceinline__ void tma_prefetch_tile(int TY, int i0, int j0, const 
 // p tiles of the first post-smoothing step: every fine lattice point of the u tile and every fine
 // vertex of the p tile gets the coarse P2 / P1 function of the coarse square that owns it, added in
 // shared memory, so the corrected state is never written to global memory and read back.
-
-// the two triangles of a coarse square of orientation o (the split of tri_mask), vertices in coarse
-// lattice units (0 or 2)
-struct EmbedTri {
-    int x[3], y[3];
-};
-__host__ __device__ constexpr EmbedTri embed_tri(int o, int t) {
-    return o == 0 ? (t == 0 ? EmbedTri{{0, 2, 2}, {0, 0, 2}} : EmbedTri{{0, 2, 0}, {0, 2, 2}})
-                  : (t == 0 ? EmbedTri{{0, 2, 0}, {0, 0, 2}} : EmbedTri{{2, 2, 0}, {0, 2, 2}});
-}
-// Value at the fine lattice point (fa / 2, fb / 2), fa, fb in [0, 4), of the coarse P2 basis
-// function of local node L (lattice offset (L % 3, L / 3)): in the triangle that holds the point,
-// with barycentric coordinates l, l_i (2 l_i - 1) at vertex i and 4 l_j l_k at the midpoint of the
-// edge (j, k); zero where L is no node of that triangle.  Evaluated at compile time.
-__host__ __device__ constexpr double embed_weight(int o, int L, int fa, int fb) {
-    const double px = 0.5 * fa, py = 0.5 * fb;
-    const int lx = L % 3, ly = L / 3;
-    for (int t = 0; t < 2; ++t) {
-        const EmbedTri T = embed_tri(o, t);
-        const double twoA = (T.x[1] - T.x[0]) * (T.y[2] - T.y[0]) - (T.x[2] - T.x[0]) * (T.y[1] - T.y[0]);
-        double l[3] = {0.0, 0.0, 0.0};
-        bool inside = true;
-        for (int i = 0; i < 3; ++i) {
-            const int j = (i + 1) % 3, k = (i + 2) % 3;
-            l[i] = ((T.x[j] - px) * (T.y[k] - py) - (T.x[k] - px) * (T.y[j] - py)) / twoA;
-            if (l[i] < 0.0) inside = false;
-        }
-        if (!inside) continue;
-        for (int i = 0; i < 3; ++i)
-            if (T.x[i] == lx && T.y[i] == ly) return l[i] * (2.0 * l[i] - 1.0);
-        for (int i = 0; i < 3; ++i) {
-            const int j = (i + 1) % 3, k = (i + 2) % 3;
-            if (T.x[j] + T.x[k] == 2 * lx && T.y[j] + T.y[k] == 2 * ly) return 4.0 * l[j] * l[k];
-        }
-        return 0.0;
-    }
-    return 0.0;
-}
-__host__ __device__ constexpr bool embed_partition_of_unity() {
-    for (int o = 0; o < 2; ++o)
-        for (int f = 0; f < 16; ++f) {
-            double s = 0.0;
-            for (int L = 0; L < 9; ++L) s += embed_weight(o, L, f % 4, f / 4);
-            if (s != 1.0) return false;
-        }
-    return true;
-}
-static_assert(embed_partition_of_unity(), "the coarse basis functions sum to one at every fine point");
-static_assert(embed_weight(0, 0, 1, 0) == 0.375 && embed_weight(0, 1, 1, 0) == 0.75 && embed_weight(0, 2, 1, 0) == -0.125,
-              "on a coarse edge the embedding is the quadratic through its three nodes");
-static_assert(embed_weight(1, 4, 2, 2) == 1.0 && embed_weight(0, 3, 2, 2) == 0.0, "a coarse node keeps its value");
 
 template <int O, int FA, int FB, int L>
 __device__ __forceinline__ void embed_term(const float2 (&z)[9], float2& acc) {
