@@ -118,6 +118,7 @@ struct Level {
     bool planar = false;     // float32 level in the planar layout (common.cuh), smoothed by the TMA step
     T *u = nullptr, *p = nullptr, *f = nullptr, *g = nullptr;
     T *tu = nullptr, *tp = nullptr, *sinv = nullptr;
+    MidLists* mid = nullptr;   // planar: the lists of the tiles on the mid-lines
     void* slab = nullptr;
     OpCoef<T> c{};
 };
@@ -130,7 +131,7 @@ stokes_status alloc_level(Level<T>& L, int k, DevMem& mem, bool planar = false) 
     L.n1 = planar ? pl_pcount(L.n) : (size_t)(L.n + 1) * (L.n + 1);
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t bu = al(2 * L.n2 * sizeof(T)), bp = al(L.n1 * sizeof(T));
-    const size_t total = 3 * bu + 4 * bp;
+    const size_t total = 3 * bu + 4 * bp + (planar ? al(sizeof(MidLists)) : 0);
     CK(mem.get(&L.slab, total));
     char* q = (char*)L.slab;
     L.u = (T*)q; q += bu;
@@ -139,7 +140,8 @@ stokes_status alloc_level(Level<T>& L, int k, DevMem& mem, bool planar = false) 
     L.p = (T*)q; q += bp;
     L.g = (T*)q; q += bp;
     L.tp = (T*)q; q += bp;
-    L.sinv = (T*)q;
+    L.sinv = (T*)q; q += bp;
+    if (planar) L.mid = (MidLists*)q;
     CK(cudaMemsetAsync(L.slab, 0, total, mem.st));
     return STOKES_OK;
 }
@@ -187,6 +189,7 @@ struct stokes_handle_t {
     ClusterTables<double>* cl_tab64 = nullptr;
     bool launch_failed = false;             // a step variant refused to launch (reported by the next call)
     bool has_planar = false;                // some float32 level is planar
+    bool shared = false;                    // one of a batch: its kernels run beside those of other solves
     int small_top = -1;                     // float32 levels clev+1..small_top: one cooperative launch per visit
     bool fuse_prolong = false;              // planar levels: x += P x_c inside the first post-smoothing step
     OpCoef<float>* dcoef = nullptr;         // device copies of the float32 operators of levels 0..small_top
@@ -280,7 +283,7 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
             } else if (lv.planar) {
                 CoarseCorrection cc;
                 if (coarse && s == 0) cc = CoarseCorrection{coarse->u, coarse->p, coarse->planar};
-                if (launch_uzawa_tma(h->st, lv.n, lv.c, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou,
+                if (launch_uzawa_tma(h->st, lv.n, lv.c, PlanarLevel{lv.mid, h->shared}, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou,
                                      op, cc))
                     sw = !sw;
                 else
@@ -418,7 +421,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
     if constexpr (sizeof(T) == 4) {
         if (lv.planar) {
             // the defect and its restriction in one kernel on the staged tiles (the defect stays on chip)
-            if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, xu, xp, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p)) {
+            if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, PlanarLevel{lv.mid, h->shared}, xu, xp, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p)) {
                 launch_residual_planar(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp);
                 launch_restrict_planar(h->st, cl.n, cl.planar, ru, rp, cl.f, cl.g, cl.u, cl.p);
             }
@@ -612,7 +615,11 @@ stokes_status rebuild_beta(stokes_handle* h) {
         if (k <= h->small_top)   // the cooperative cycle's copy (the host structure stays in the handle)
             CK(cudaMemcpyAsync(h->dcoef + k, &lv.c, sizeof(OpCoef<float>), cudaMemcpyHostToDevice, h->st));
         // planar levels run only the register-tile step, which needs its coefficient structure
-        if (lv.planar && !reg_tables_match(lv.c)) return STOKES_ERR_BAD_ARG;
+        if (lv.planar) {
+            MidLists ml;
+            if (!reg_tables_match(lv.c) || !fill_mid_lists(ml, lv.c, (float)h->prm.tau)) return STOKES_ERR_BAD_ARG;
+            CK(cudaMemcpyAsync(lv.mid, &ml, sizeof ml, cudaMemcpyHostToDevice, h->st));   // pageable: copied on return
+        }
         launch_schur_diag<float>(h->st, lv.n, make_coef<double>(lv.n, beta), lv.sinv, h->dom,
                                  lv.planar ? pl_vpitch(lv.n) : 0);
     }
@@ -1103,7 +1110,7 @@ stokes_status stokes_residual_restrict_f32(stokes_handle* h, const float* u, con
     if (lv.planar) {
         launch_to_planar(h->st, lv.n, u, p, lv.u, lv.p);
         launch_to_planar(h->st, lv.n, f, g, lv.f, lv.g);
-        if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, lv.u, lv.p, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p))
+        if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, PlanarLevel{lv.mid, h->shared}, lv.u, lv.p, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p))
             return STOKES_ERR_CUDA;
         if (cl.planar) {
             launch_from_planar(h->st, cl.n, cl.f, cl.g, fc, gc);
@@ -1270,7 +1277,7 @@ static stokes_status autotune_levels(stokes_handle* h, cudaStream_t st) {
     for (int l = 1; l < (int)h->h32.size(); ++l) {
         Level<float>& lv = h->h32[l];
         if (lv.planar ? tma_tuned(lv.n) : uzawa_tuned(lv.n)) continue;
-        cudaError_t e = lv.planar ? autotune_uzawa_tma(st, lv.n, lv.c, (float)h->prm.tau, (float)h->prm.sigma, lv.u, lv.p,
+        cudaError_t e = lv.planar ? autotune_uzawa_tma(st, lv.n, lv.c, PlanarLevel{lv.mid, h->shared}, (float)h->prm.tau, (float)h->prm.sigma, lv.u, lv.p,
                                                        lv.f, lv.g, lv.sinv, lv.tu, lv.tp)
                                   : autotune_uzawa_fused(st, lv.n, lv.c, (float)h->prm.tau, (float)h->prm.sigma, lv.u,
                                                          lv.p, lv.f, lv.g, lv.sinv, lv.tu, lv.tp, nullptr, nullptr);
@@ -1352,6 +1359,7 @@ stokes_status stokes_batch_setup(int count, const int* levels, const double* bet
             stokes_batch_destroy(b);
             return s;
         }
+        h->shared = count > 1;
         b->inst.push_back(h);
     }
     init_mem(b->mem, b->st);

@@ -40,7 +40,6 @@
 
 #include "cellops.cuh"
 #include "cluster_cycle.cuh"
-#include "coef.h"
 #include "elements.h"
 #include "kernels.cuh"
 
@@ -772,18 +771,8 @@ bool prepare_cluster_cycle() {
 template <typename T>
 bool fill_cluster_level(LevelLists<T>& q, int n, const OpCoef<T>& c, T tau) {
     const int WH = n + 3, RS = 2 * WH, VW = n + 3;   // as in place()
+    const ListStructure& S = list_structure();
     q = LevelLists<T>{};
-    // Which entries there are is read off the float64 stencils at beta h^2 = 1, where stiffness and mass are of one
-    // size: at small beta h^2 the entries that only the mass has are tiny, and yet they count (dropping them below
-    // 1e-6 of the largest made float32 W-cycles a hundred times less accurate).
-    const OpCoef<double> ref = make_coef<double>(n, (double)n * n);
-    const double tol = 1e-12;
-    double amax = 0.0, bmax = 0.0;
-    for (int k = 0; k < kStencilClasses; ++k)
-        for (int w = 0; w < 25; ++w) {
-            for (int s = 0; s < 4; ++s) amax = std::max(amax, std::fabs(ref.MA[k][s][w]));
-            bmax = std::max({bmax, std::fabs(ref.MBx[k][w]), std::fabs(ref.MBy[k][w])});
-        }
     auto off = [&](int w) {
         const int dx = w % 5 - 2, dy = w / 5 - 2;
         return dy * RS + (dx & 1) * WH + (dx >> 1);
@@ -791,29 +780,16 @@ bool fill_cluster_level(LevelLists<T>& q, int n, const OpCoef<T>& c, T tau) {
     for (int k = 0; k < kStencilClasses; ++k) {
         for (int s = 0; s < 4; ++s) {
             q.ti[k][s] = tau * c.MIdg[k][s];
-            int m = 0;
-            const int cap = s == 0 ? (k == 6 ? 27 : 18) : 9;
-            for (int w = 0; w < 25; ++w)
-                if (std::fabs(ref.MA[k][s][w]) > tol * amax) {
-                    if (m == cap) return false;
-                    q.A[k][list_start(s) + m++] = E1<T>{c.MA[k][s][w], off(w)};
-                }
-            m = 0;
-            for (int v = 0; v < 9; ++v)
-                if (std::fabs(ref.MBTx[k][s][v]) > tol * bmax || std::fabs(ref.MBTy[k][s][v]) > tol * bmax) {
-                    if (s == 0 || m == 4) return false;
-                    q.BT[k][4 * (s - 1) + m++] = E2<T>{c.MBTx[k][s][v], c.MBTy[k][s][v], (v / 3 - 1) * VW + v % 3 - 1};
-                }
+            for (int m = list_start(s); m < (s < 3 ? list_start(s + 1) : kListA); ++m)
+                if (const int w = S.A[k][m]; w >= 0) q.A[k][m] = E1<T>{c.MA[k][s][w], off(w)};
+            for (int m = 4 * (s - 1); s > 0 && m < 4 * s; ++m)
+                if (const int v = S.BT[k][m]; v >= 0)
+                    q.BT[k][m] = E2<T>{c.MBTx[k][s][v], c.MBTy[k][s][v], (v / 3 - 1) * VW + v % 3 - 1};
         }
-        int m = 0;
-        const int cap = k == 6 ? 16 : 12;
-        for (int w = 0; w < 25; ++w)
-            if (std::fabs(ref.MBx[k][w]) > tol * bmax || std::fabs(ref.MBy[k][w]) > tol * bmax) {
-                if (m == cap) return false;
-                q.B[k][m++] = E2<T>{c.MBx[k][w], c.MBy[k][w], off(w)};
-            }
+        for (int m = 0; m < kListB; ++m)
+            if (const int w = S.B[k][m]; w >= 0) q.B[k][m] = E2<T>{c.MBx[k][w], c.MBy[k][w], off(w)};
     }
-    return true;
+    return S.ok;
 }
 
 template <typename T>

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "stencil_tables.cuh"
 
 namespace smg {
 
@@ -21,24 +22,13 @@ constexpr int cluster_top() { return sizeof(T) == 4 ? 5 : 4; }
 enum : unsigned char { kOpPreZero = 0, kOpPre = 1, kOpPost = 2, kOpRestrict = 3, kOpCoarse = 4, kOpProlong = 5, kOpClear = 6 };
 inline unsigned char cluster_op(int op, int level) { return (unsigned char)(op | level << 4); }
 
-// What the kernel's threads sum: lists of (coefficient, offset of the value from the cell's own), per
-// stencil class and, for velocity, node s (0 V, 1 H, 2 E, 3 C); unused entries are zero.
-template <typename T>
-struct alignas(2 * sizeof(T)) E1 {
-    T c;
-    int o;
-};
-template <typename T>
-struct alignas(16) E2 {
-    T cx, cy;                            // the x and the y coefficient
-    int o;
-};
-__host__ __device__ constexpr int list_start(int s) { return s == 0 ? 0 : 18 + 9 * s; }
+// What the kernel's threads sum (stencil_tables.cuh): offsets are those of the value from the cell's own in
+// the level's arrays; unused entries are zero.
 template <typename T>
 struct alignas(16) LevelLists {
-    E1<T> A[kStencilClasses][54];        // from list_start(s): 18 entries of V (27 at the centre), 9 of H, E, C
-    E2<T> BT[kStencilClasses][12];       // 4 of H, E, C (the V rows of B^T vanish)
-    E2<T> B[kStencilClasses][16];        // 12 (16 at the centre)
+    E1<T> A[kStencilClasses][kListA];    // from list_start(s): 18 entries of V (21 at the centre), 9 of H, E, C
+    E2<T> BT[kStencilClasses][kListBT];  // 4 of H, E, C (the V rows of B^T vanish)
+    E2<T> B[kStencilClasses][kListB];    // 12 (16 at the centre)
     T ti[kStencilClasses][4];            // tau / diag A
 };
 template <typename T>

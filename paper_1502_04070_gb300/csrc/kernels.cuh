@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "stencil_tables.cuh"
 
 namespace smg {
 
@@ -81,8 +82,23 @@ struct CoarseCorrection {
     const float* p = nullptr;
     bool planar = false;
 };
-bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma, const float* u,
-                      const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
+// What the tiles on the mid-lines sum (device copy per planar level): the lists of stencil_tables.cuh with
+// offsets in the staged tiles; A over the u tile, B^T over the p or dp tile, B over the u^{m-1/2} tile, BU the
+// same rows over the u tile.
+struct alignas(16) MidLists {
+    E1<float> A[kStencilClasses][kListA];
+    E2<float> BT[kStencilClasses][kListBT], B[kStencilClasses][kListB], BU[kStencilClasses][kListB];
+    float ti[kStencilClasses][4];        // tau / diag A
+};
+// what the kernels of a planar level take beside its arrays and operator: its lists (device), and whether
+// other solves share the GPU (a batch), which favours tall tiles
+struct PlanarLevel {
+    const MidLists* lists = nullptr;
+    bool shared = false;
+};
+bool fill_mid_lists(MidLists& q, const OpCoef<float>& c, float tau);   // host; false: a stencil has more entries
+bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau, float sigma,
+                      const float* u, const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
                       const CoarseCorrection& cc = CoarseCorrection{});
 bool uzawa_tma_available();
 // the fused correction can be used: the tensor-map encoder is there and the kernel's compile-time
@@ -100,15 +116,15 @@ bool fuse_prolong_enabled();
 // launch_uzawa_tma runs the variant chosen for level size n (0 until autotune_uzawa_tma or
 // set_tma_choice).
 constexpr int kTmaVariants = 6;
-bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma,
-                              const float* u, const float* p, const float* f, const float* g, const float* sinv,
+bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
+                              float sigma, const float* u, const float* p, const float* f, const float* g, const float* sinv,
                               float* u_out, float* p_out, const CoarseCorrection& cc = CoarseCorrection{});
 // r = F - A x on a planar level (N = n) and its restriction (fc, gc) = I^T r to the coarse level
 // (planar or not: pc_planar), with the coarse iterate (uc, pc) set to zero, in one kernel on the
 // tiles of the planar step; the fine defect stays in shared memory.  False (nothing launched) as
 // for launch_uzawa_tma.
-bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const float* u, const float* p,
-                         const float* f, const float* g, float* fc, float* gc, float* uc, float* pc);
+bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& ml,
+                         const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc, float* pc);
 // The float32 V- or W-cycle from level `top` (compact layout, top <= kSmallCycleTop) down to the
 // coarsest level clev of the iteration, with its exact solve, in ONE cooperative launch (uzawa_reg.cu):
 // every CTA resident, phases separated by grid barriers whose waits are bounded (about a second; a
@@ -136,8 +152,8 @@ int tma_choice(int n);
 bool tma_tuned(int n);
 bool set_tma_choice(int n, int v);
 // times every planar variant on these planar buffers (contents overwritten) and keeps the fastest
-cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma, float* u,
-                               float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out);
+cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
+                               float sigma, float* u, float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out);
 unsigned uzawa_tma_timeouts();
 // Does the compile-time structure of the register tile match these coefficients?
 bool reg_tables_match(const OpCoef<float>& c);

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "coef.h"
 #include "common.cuh"
 
 namespace smg {
@@ -171,5 +172,69 @@ static_assert(embed_partition_of_unity(), "the coarse basis functions sum to one
 static_assert(embed_weight(0, 0, 1, 0) == 0.375 && embed_weight(0, 1, 1, 0) == 0.75 && embed_weight(0, 2, 1, 0) == -0.125,
               "on a coarse edge the embedding is the quadratic through its three nodes");
 static_assert(embed_weight(1, 4, 2, 2) == 1.0 && embed_weight(0, 3, 2, 2) == 0.0, "a coarse node keeps its value");
+
+// ---- the merged stencils of every class as lists (for kernels that sum them entry by entry)
+template <typename T>
+struct alignas(2 * sizeof(T)) E1 {   // coefficient and an offset
+    T c;
+    int o;
+};
+template <typename T>
+struct alignas(16) E2 {              // the x and the y coefficient and an offset
+    T cx, cy;
+    int o;
+};
+// In every class, mid-lines included, the nodes V, H, E, C of a cell have 17 + 9 + 9 + 7 entries of A and 0 + 4 + 4 + 4
+// of B^T, its vertex has 12 of B; the one cell at the centre (class 6) has 21 of A at V and 16 of B.
+__host__ __device__ constexpr int list_start(int s) { return s == 0 ? 0 : 18 + 9 * s; }
+constexpr int kListA = 54, kListBT = 12, kListB = 16;   // per class: 27 + 9 + 9 + 9, 4 + 4 + 4, 16
+
+// Which entries there are, read once off the float64 stencils at beta h^2 = 1, where stiffness and mass are of
+// one size (at small beta h^2 the entries that only the mass has are tiny, and yet they count: leaving them
+// out below 1e-6 of the largest made float32 W-cycles a hundred times less accurate).
+struct ListStructure {
+    signed char A[kStencilClasses][kListA], BT[kStencilClasses][kListBT], B[kStencilClasses][kListB];   // window points, -1: none
+    bool ok = true;
+};
+inline const ListStructure& list_structure() {
+    static const ListStructure S = [] {
+        ListStructure r;
+        const OpCoef<double> c = make_coef<double>(4, 16.0);
+        double amax = 0.0, bmax = 0.0;
+        for (int k = 0; k < kStencilClasses; ++k)
+            for (int w = 0; w < 25; ++w) {
+                for (int s = 0; s < 4; ++s) amax = std::max(amax, std::fabs(c.MA[k][s][w]));
+                bmax = std::max({bmax, std::fabs(c.MBx[k][w]), std::fabs(c.MBy[k][w])});
+            }
+        const double ta = 1e-12 * amax, tb = 1e-12 * bmax;
+        for (int k = 0; k < kStencilClasses; ++k) {
+            for (auto& v : r.A[k]) v = -1;
+            for (auto& v : r.BT[k]) v = -1;
+            for (auto& v : r.B[k]) v = -1;
+            for (int s = 0; s < 4; ++s) {
+                int m = 0;
+                for (int w = 0; w < 25; ++w)
+                    if (std::fabs(c.MA[k][s][w]) > ta) {
+                        if (m == (s == 0 ? (k == 6 ? 21 : 18) : 9)) r.ok = false;
+                        else r.A[k][list_start(s) + m++] = (signed char)w;
+                    }
+                m = 0;
+                for (int v = 0; v < 9; ++v)
+                    if (std::fabs(c.MBTx[k][s][v]) > tb || std::fabs(c.MBTy[k][s][v]) > tb) {
+                        if (s == 0 || m == 4) r.ok = false;
+                        else r.BT[k][4 * (s - 1) + m++] = (signed char)v;
+                    }
+            }
+            int m = 0;
+            for (int w = 0; w < 25; ++w)
+                if (std::fabs(c.MBx[k][w]) > tb || std::fabs(c.MBy[k][w]) > tb) {
+                    if (m == (k == 6 ? 16 : 12)) r.ok = false;
+                    else r.B[k][m++] = (signed char)w;
+                }
+        }
+        return r;
+    }();
+    return S;
+}
 
 }  // namespace smg

@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include <cuda.h>
 
@@ -163,6 +164,134 @@ struct ULat {
     }
 };
 
+// Where a cell's new values go: the compact float32 lattice (PLO false) or the planar layout
+template <bool PLO>
+__device__ __forceinline__ void store_node(float* __restrict__ u_out, int n, int X, int Y, float2 v) {
+    if constexpr (PLO) {
+        *reinterpret_cast<float2*>(u_out + pl_u(n, X, Y)) = v;
+    } else {
+        const int ld = 2 * n + 1, k = Y * ld + X;
+        u_out[k] = v.x;
+        u_out[ld * ld + k] = v.y;
+    }
+}
+template <bool PLO>
+__device__ __forceinline__ int vert_at(int n, int i, int j) {
+    return j * (PLO ? pl_vpitch(n) : n + 1) + i;
+}
+
+// ---- cells on a mid-line: sums over the lists of the cell's class (MidLists, through the read-only path: a few
+// kilobytes that stay in L1), which have the same length in every class, so that the lanes of a warp run
+// together.  The classes' own code, one class after the other in each row, made a tile on the mid-lines two to three
+// times as long as the others, and that is the time of a launch on levels with few waves of tiles: N = 128, 256, 512,
+// 2048 took 7.4, 11.1, 15.2, 99.9 us a step, with the lists 5.9, 8.7, 12.9, 96.3 (and 5.5, 6.8, 11.1 at the tile
+// heights that suit them, tile_rows).
+__device__ __forceinline__ E1<float> ld_e1(const E1<float>* e) {
+    const float2 v = __ldg(reinterpret_cast<const float2*>(e));
+    return E1<float>{v.x, __float_as_int(v.y)};
+}
+__device__ __forceinline__ E2<float> ld_e2(const E2<float>* e) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(e));
+    return E2<float>{v.x, v.y, __float_as_int(v.z)};
+}
+// acc + N entries over a velocity tile in two (row pairs whole) or four planes: offset = (o >> 2) + (o & 3) x plane
+template <int N>
+__device__ __forceinline__ float2 mid_sum(const E1<float>* e, const float2* c, int plane, float2 acc) {
+    E1<float> t[N];
+#pragma unroll
+    for (int w = 0; w < N; ++w) t[w] = ld_e1(e + w);
+#pragma unroll
+    for (int w = 0; w < N; ++w)
+        acc = __ffma2_rn(f2(t[w].c, t[w].c), c[(t[w].o >> 2) + (t[w].o & 3) * plane], acc);
+    return acc;
+}
+template <int N>
+__device__ __forceinline__ float mid_sum_b(const E2<float>* e, const float2* c, int plane, float acc) {
+#pragma unroll
+    for (int w = 0; w < N; ++w) {
+        const E2<float> t = ld_e2(e + w);
+        const float2 v = c[(t.o >> 2) + (t.o & 3) * plane];
+        acc = fmaf(t.cx, v.x, fmaf(t.cy, v.y, acc));
+    }
+    return acc;
+}
+__device__ __forceinline__ float2 mid_sum_bt(const E2<float>* e, const float* p) {
+    float2 acc = f2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        const E2<float> t = ld_e2(e + w);
+        acc = __ffma2_rn(f2(t.cx, t.cy), f2(p[t.o], p[t.o]), acc);
+    }
+    return acc;
+}
+__device__ __forceinline__ int mid_class(int i, int j, int n) {   // any class for cells outside the level
+    return stencil_class(min(max(i, 0), n), min(max(j, 0), n), n);
+}
+__device__ __forceinline__ float mid_bu(const E2<float>* e, int k, const float2* c, int plane) {
+    float t = mid_sum_b<6>(e, c, plane, 0.f);
+    t = mid_sum_b<6>(e + 6, c, plane, t);
+    if (k == 6) t = mid_sum_b<4>(e + 12, c, plane, t);
+    return t;
+}
+// Node s of cell `x` of row r of the u^{m-1/2} region (STEP), or of the defect (r_u over f)
+template <class G, bool STEP>
+__device__ __forceinline__ void mid_node(const MidLists& ml, int k, int s, const float2* sU, int UPL, const float* sP,
+                                         float2* sF, int FPL, int r, int x, int i0, int j0, int n) {
+    const int X = 2 * (i0 - 2 + x) + (s & 1), Y = 2 * (j0 - 2 + r) + (s >> 1);
+    const float2* t0 = sU + 2 * (r + 1) * G::UWH + x + G::UX - 2;
+    float2* fr = sF + r * G::FW + x + s * FPL;
+    const E1<float>* e = ml.A[k] + list_start(s);
+    float2 t = mid_sum<9>(e, t0, UPL, f2(0.f, 0.f));
+    if (s == 0) {
+        t = mid_sum<9>(e + 9, t0, UPL, t);
+        if (k == 6) t = mid_sum<3>(e + 18, t0, UPL, t);
+    } else {
+        const float2 b = mid_sum_bt(ml.BT[k] + 4 * (s - 1), sP + (r + 1) * G::PW + x + G::PX - 2);
+        t = f2(t.x + b.x, t.y + b.y);
+    }
+    const float2 fs = *fr;
+    t = f2(fs.x - t.x, fs.y - t.y);
+    if constexpr (STEP) {
+        const float ti = __ldg(&ml.ti[k][s]);
+        t = __ffma2_rn(f2(ti, ti), t, t0[(s >> 1) * G::UWH + (s & 1) * UPL]);
+    }
+    *fr = interior2(X, Y, n) ? t : f2(0.f, 0.f);
+}
+// r_p = g - B u at vertex `x` of row r (over g; that tile starts two rows below the CTA's)
+template <class G>
+__device__ __forceinline__ void mid_defect_p(const MidLists& ml, int k, const float2* sU, int UPL, float* sG, int r, int x,
+                                             int i0, int j0, int n) {
+    const int ci = i0 - 2 + x, cj = j0 - 2 + r, q = r * G::DW + x + G::DX - 2;
+    const bool live = ci >= 0 && cj >= 0 && ci <= n && cj <= n;
+    sG[q] = live ? sG[q] - mid_bu(ml.BU[k], k, sU + 2 * (r + 1) * G::UWH + x + G::UX - 2, UPL) : 0.f;
+}
+// dp at vertex `x` of row r (Shat^{-1} is zero off the domain)
+template <class G>
+__device__ __forceinline__ void mid_dp(const MidLists& ml, const float2* sF, int FPL, float* sG, const float* sS, float sigma,
+                                       int r, int x, int i0, int j0, int n) {
+    const int k = mid_class(i0 - 1 + x, j0 - 1 + r, n), q = r * G::DW + x + G::DX - 1;
+    sG[q] = sigma * sS[q] * (mid_bu(ml.B[k], k, sF + (r + 1) * G::FW + x + 1, FPL) - sG[q]);
+}
+// the new u at node s (and p, with node 0) of cell `x` of row r
+template <class G, bool PLO>
+__device__ __forceinline__ void mid_out(const MidLists& ml, int s, const float2* sF, int FPL, const float* sG, const float* sP,
+                                        int r, int x, int i0, int j0, int n, float* __restrict__ u_out,
+                                        float* __restrict__ p_out) {
+    const int ci = i0 + x, cj = j0 + r;
+    if (ci > n || cj > n) return;
+    const int k = stencil_class(ci, cj, n), X = 2 * ci + (s & 1), Y = 2 * cj + (s >> 1);
+    const float* dp = sG + (r + 1) * G::DW + x + G::DX;
+    if (X <= 2 * n && Y <= 2 * n) {
+        float2 o = sF[(r + 2) * G::FW + x + 2 + s * FPL];
+        if (s > 0) {
+            const float ti = __ldg(&ml.ti[k][s]);
+            o = __ffma2_rn(f2(-ti, -ti), mid_sum_bt(ml.BT[k] + 4 * (s - 1), dp), o);
+        }
+        store_node<PLO>(u_out, n, X, Y, interior2(X, Y, n) ? o : f2(0.f, 0.f));
+    }
+    if (s == 0) p_out[vert_at<PLO>(n, ci, cj)] = sP[(r + 3) * G::PW + x + G::PX] + dp[0];
+}
+
 // ---- phase 1, fast path: A rows over the u window, B^T rows over the p window
 template <int C, int UWH, int W>
 __device__ __forceinline__ void a_term(const float2 (&a)[kGroups], const float2* t0, const float2* t1, float2 (&au)[4],
@@ -233,12 +362,12 @@ __device__ __forceinline__ void load_coef(const RegCoef& q, float2 (&a)[kGroups]
 
 template <class G, int C, bool INNER>
 __device__ __forceinline__ void phase1_fast(const RegCoef& q, const float2* sU, int UPL, const float* sP, float2* sF,
-                                           int FPL, int TY, int NW, int warp, int lane, int i0, int j0, int n) {
+                                           int FPL, int r0, int rb, int rs, int lane, int i0, int j0, int n) {
     float2 a[kGroups];
     load_coef<C>(q, a);
     const float ti0 = q.ti[C][0], ti1 = q.ti[C][1];
     const float2 mb = f2(-q.b, -q.b);
-    for (int r = warp; r < TY + 4; r += NW) {
+    for (int r = r0; r < rb; r += rs) {
         const float2* t0 = sU + 2 * (r + 1) * G::UWH + lane + G::UX - 2;
         const float2* t1 = t0 + UPL;
         float2 au[4], ctr[4], bt[4];
@@ -274,9 +403,9 @@ __device__ __forceinline__ void phase1_fast(const RegCoef& q, const float2* sU, 
 
 template <class G, int C>
 __device__ __forceinline__ void phase2_fast(const RegCoef& q, const float2* sF, int FPL, float* sG, const float* sS,
-                                            float sigma, int TY, int NW, int warp, int lane) {
+                                            float sigma, int r0, int rb, int rs, int lane) {
     const float b = q.b;
-    for (int r = warp; r < TY + 2; r += NW) {
+    for (int r = r0; r < rb; r += rs) {
         if (lane >= G::DN) break;
         const float2* f0 = sF + (r + 1) * G::FW + lane + 1;
         const float acc = b_row<C, G::FW>(f0, FPL, std::make_integer_sequence<int, 25>{});
@@ -286,28 +415,12 @@ __device__ __forceinline__ void phase2_fast(const RegCoef& q, const float2* sF, 
     }
 }
 
-// Where a cell's new values go: the compact float32 lattice (PLO false) or the planar layout
-template <bool PLO>
-__device__ __forceinline__ void store_node(float* __restrict__ u_out, int n, int X, int Y, float2 v) {
-    if constexpr (PLO) {
-        *reinterpret_cast<float2*>(u_out + pl_u(n, X, Y)) = v;
-    } else {
-        const int ld = 2 * n + 1, k = Y * ld + X;
-        u_out[k] = v.x;
-        u_out[ld * ld + k] = v.y;
-    }
-}
-template <bool PLO>
-__device__ __forceinline__ int vert_at(int n, int i, int j) {
-    return j * (PLO ? pl_vpitch(n) : n + 1) + i;
-}
-
 template <class G, bool PLO, int C, bool INNER>
 __device__ __forceinline__ void phase3_fast(const RegCoef& q, const float2* sF, int FPL, const float* sG,
-                                            const float* sP, int TY, int NW, int warp, int lane, int i0, int j0,
-                                            int n, float* __restrict__ u_out, float* __restrict__ p_out) {
+                                            const float* sP, int r0, int rb, int rs, int lane, int i0,
+                                            int j0, int n, float* __restrict__ u_out, float* __restrict__ p_out) {
     const float nb1 = -q.ti[C][1] * q.b;
-    for (int r = warp; r < TY; r += NW) {
+    for (int r = r0; r < rb; r += rs) {
         if (lane >= G::TX) break;
         const int ci = i0 + lane, cj = j0 + r;
         if (!INNER && (ci > n || cj > n)) continue;
@@ -532,11 +645,65 @@ __device__ __forceinline__ void phase3_pair(const RegCoef& q, const float2* sF, 
     }
 }
 
+// A tile on a mid-line: every row by the lists if the tile meets x = 1/2, else the register rows of one class below
+// y = 1/2 and of the other above, and the row on it by the lists.  (Splitting a row at x = 1/2 into its two classes
+// and the one cell between was slower: two passes a row, or packed passes that leave a warp with the lists.)
+// rect(class, r, end, step): rows r, r + step, .. < end; row(r); first_j: the cell row of r = 0; count rows.
+template <class Rect, class Row>
+__device__ __forceinline__ void mid_cover(bool col, bool right, int h, int first_j, int count, int NW, Rect&& rect, Row&& row) {
+    const int warp = threadIdx.x >> 5;
+    const int m = col ? 0 : min(max(h - first_j, 0), count), e = col ? count : min(max(h - first_j + 1, 0), count);
+    // row r goes to warp r modulo NW throughout
+#pragma unroll 1
+    for (int t = 0; t < 2 && !col; ++t) {   // one copy of each class's rows in the code
+        const int ra = t ? e : 0;
+        rect((int)right ^ t, ra + (((warp - ra) % NW) + NW) % NW, t ? count : m, NW);
+    }
+    for (int r = m + (((warp - m) % NW) + NW) % NW; r < e; r += NW) row(r);
+}
+template <class G, bool PLO, int NW>
+__device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const RegCoef& q, const MidLists& ml, float sigma,
+                                           const float2* sU, float2* sF, const float* sP, float* sG, const float* sS,
+                                           float* __restrict__ u_out, float* __restrict__ p_out) {
+    const int UPL = G::upl(TY), FPL = G::fpl(TY), lane = threadIdx.x & 31, h = n >> 1;
+    const bool col = h >= i0 - 2 && h < i0 + G::TX + 2, right = i0 >= h;
+    mid_cover(col, right, h, j0 - 2, TY + 4, NW,
+              [&](int cls, int r, int end, int step) {
+                  if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n);
+                  else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n);
+              },
+              [&](int r) {
+                  const int k = mid_class(i0 - 2 + lane, j0 - 2 + r, n);
+#pragma unroll
+                  for (int s = 0; s < 4; ++s) mid_node<G, true>(ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n);
+              });
+    __syncthreads();
+    mid_cover(col, right, h, j0 - 1, TY + 2, NW,
+              [&](int cls, int r, int end, int step) {
+                  if (cls == 0) phase2_fast<G, 0>(q, sF, FPL, sG, sS, sigma, r, end, step, lane);
+                  else phase2_fast<G, 1>(q, sF, FPL, sG, sS, sigma, r, end, step, lane);
+              },
+              [&](int r) {
+                  if (lane < G::DN) mid_dp<G>(ml, sF, FPL, sG, sS, sigma, r, lane, i0, j0, n);
+              });
+    __syncthreads();
+    mid_cover(col, right, h, j0, TY, NW,
+              [&](int cls, int r, int end, int step) {
+                  if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, r, end, step, lane, i0, j0, n, u_out, p_out);
+                  else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, r, end, step, lane, i0, j0, n, u_out, p_out);
+              },
+              [&](int r) {
+                  if (lane < G::TX)
+#pragma unroll
+                      for (int s = 0; s < 4; ++s) mid_out<G, PLO>(ml, s, sF, FPL, sG, sP, r, lane, i0, j0, n, u_out, p_out);
+              });
+}
+
 // The three phases of the step on the staged tiles (sU, sP, sF = f, sG = g, sS = Shat^{-1}); writes
 // the new state of the CTA's cells to (u_out, p_out).
-template <class G, bool PLO, int NW, bool PAIR = false>
-__device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const OpCoef<float>& c, const RegCoef& q,
-                                           float tau, float sigma, const float2* sU, float2* sF, const float* sP,
+template <class G, bool PLO, int NW, bool PAIR = false, bool LISTS = false>
+__device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
+                                           const MidLists* ml, float tau, float sigma, const float2* sU, float2* sF, const float* sP,
                                            float* sG, const float* sS, float* __restrict__ u_out,
                                            float* __restrict__ p_out) {
     constexpr int TX = G::TX;
@@ -547,6 +714,12 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
     const bool inner = fast && i0 >= 4 && j0 >= 4 && i0 + TX + 3 <= n && j0 + TY + 3 <= n;
     const int cls = orient(i0, j0, n);
 
+    if constexpr (LISTS) {
+        if (!fast) {
+            mid_phases<G, PLO, NW>(n, TY, i0, j0, q, *ml, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+            return;
+        }
+    }
     const ULat<G> vux{sU, UPL, i0 - G::UX, 2 * (j0 - 3), false};
     const ULat<G> vuy{sU, UPL, i0 - G::UX, 2 * (j0 - 3), true};
     const SVert<float, G::PW> vp{sP, i0 - G::PX, j0 - 3};
@@ -564,13 +737,13 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
         }
     } else if (fast) {
         if (inner) {
-            if (cls == 0) phase1_fast<G, 0, true>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
-            else phase1_fast<G, 1, true>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
+            if (cls == 0) phase1_fast<G, 0, true>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
+            else phase1_fast<G, 1, true>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
         } else {
-            if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
-            else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
+            if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
+            else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
         }
-    } else {
+    } else if constexpr (!LISTS) {
         for (int r = warp; r < TY + 4; r += NW) {
             const int ci = i0 - 2 + lane, cj = j0 - 2 + r;
             float2 hv[4];
@@ -579,7 +752,7 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
             float2* fr = sF + r * G::FW + lane;
             if (ci >= 0 && cj >= 0 && ci <= n && cj <= n) {
                 Acc<float> a;
-                cell_apply_auto<true, true, false, true, false>(ci, cj, n, c, vux, vuy, vp, a);
+                cell_apply_auto<true, true, false, true, false>(ci, cj, n, *c, vux, vuy, vp, a);
                 const CellNodes cn = cell_nodes(ci, cj, n);
 #pragma unroll
                 for (int s = 0; s < 4; ++s) {
@@ -601,9 +774,9 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
         if (cls == 0) phase2_pair<G, 0>(q, sF, FPL, sG, sS, sigma, TY, NW, warp, lane);
         else phase2_pair<G, 1>(q, sF, FPL, sG, sS, sigma, TY, NW, warp, lane);
     } else if (fast) {
-        if (cls == 0) phase2_fast<G, 0>(q, sF, FPL, sG, sS, sigma, TY, NW, warp, lane);
-        else phase2_fast<G, 1>(q, sF, FPL, sG, sS, sigma, TY, NW, warp, lane);
-    } else {
+        if (cls == 0) phase2_fast<G, 0>(q, sF, FPL, sG, sS, sigma, warp, TY + 2, NW, lane);
+        else phase2_fast<G, 1>(q, sF, FPL, sG, sS, sigma, warp, TY + 2, NW, lane);
+    } else if constexpr (!LISTS) {
         for (int r = warp; r < TY + 2; r += NW) {
             if (lane >= G::DN) break;
             const int vi = i0 - 1 + lane, vj = j0 - 1 + r;
@@ -611,7 +784,7 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
             float d = 0.f;
             if (vi >= 0 && vj >= 0 && vi <= n && vj <= n) {
                 Acc<float> a;
-                cell_apply_auto<false, false, true, false, false>(vi, vj, n, c, vhx, vhy, vp, a);
+                cell_apply_auto<false, false, true, false, false>(vi, vj, n, *c, vhx, vhy, vp, a);
                 d = sigma * sS[k] * (a.bu - sG[k]);
             }
             sG[k] = d;
@@ -630,20 +803,20 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
         }
     } else if (fast) {
         if (inner) {
-            if (cls == 0) phase3_fast<G, PLO, 0, true>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
-            else phase3_fast<G, PLO, 1, true>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
+            if (cls == 0) phase3_fast<G, PLO, 0, true>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
+            else phase3_fast<G, PLO, 1, true>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
         } else {
-            if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
-            else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
+            if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
+            else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
         }
-    } else {
+    } else if constexpr (!LISTS) {
         const SVert<float, G::DW> vd{sG, i0 - G::DX, j0 - 1};
         for (int r = warp; r < TY; r += NW) {
             if (lane >= TX) break;
             const int ci = i0 + lane, cj = j0 + r;
             if (ci > n || cj > n) continue;
             Acc<float> a;
-            cell_apply_auto<false, true, false, true, false>(ci, cj, n, c, vhx, vhy, vd, a);
+            cell_apply_auto<false, true, false, true, false>(ci, cj, n, *c, vhx, vhy, vd, a);
             const CellNodes cn = cell_nodes(ci, cj, n);
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
@@ -758,7 +931,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
     __syncthreads();
 
 
-    reg_phases<G, false, NW>(n, TY, i0, j0, c, q, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, false, NW>(n, TY, i0, j0, &c, q, nullptr, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -1000,8 +1173,8 @@ __device__ __forceinline__ void embed_apply(const EmbedJob& jb, int n, int TY, i
 // ahead), so that the CTA that takes it finds its tiles in L2
 template <int NW, int MINB, bool PAIR = false>
 __global__ void __launch_bounds__(32 * NW, MINB)
-    k_uzawa_tma(int n, int TY, TileOrder ord, const __grid_constant__ OpCoef<float> c, const __grid_constant__ RegCoef q,
-                float tau, float sigma, const __grid_constant__ TmaMaps maps, float* __restrict__ u_out,
+    k_uzawa_tma(int n, int TY, TileOrder ord, const __grid_constant__ RegCoef q, const MidLists* __restrict__ ml,
+                float sigma, const __grid_constant__ TmaMaps maps, float* __restrict__ u_out,
                 float* __restrict__ p_out, int pf, const float* __restrict__ uc, const float* __restrict__ pc, int pcp) {
     using G = TmaTile;
     extern __shared__ unsigned char smem_raw[];
@@ -1059,7 +1232,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         }
         __syncthreads();
     }
-    reg_phases<G, true, NW, PAIR>(n, TY, i0, j0, c, q, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, true, NW, PAIR, true>(n, TY, i0, j0, nullptr, q, ml, 0.f, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -1098,13 +1271,13 @@ __device__ __forceinline__ float bu_row(const float2* t0, const float2* t1, std:
 // the defect on cells and vertices (i0 - 2 + lane, j0 - 2 + r), r < TY + 2, fast path (class C)
 template <class G, int C>
 __device__ __forceinline__ void defect_fast(const RegCoef& q, const float2* sU, int UPL, const float* sP, float2* sF,
-                                           int FPL, float* sG, int TY, int NW, int warp, int lane, int i0, int j0,
-                                           int n) {
+                                           int FPL, float* sG, int r0, int rb, int rs, int lane, int i0,
+                                           int j0, int n) {
     float2 a[kGroups];
     load_coef<C>(q, a);
     const float2 mb = f2(-q.b, -q.b);
     const float hb = q.b;
-    for (int r = warp; r < TY + 2; r += NW) {
+    for (int r = r0; r < rb; r += rs) {
         const float2* t0 = sU + 2 * (r + 1) * G::UWH + lane + G::UX - 2;
         const float2* t1 = t0 + UPL;
         float2 au[4], ctr[4], bt[4];
@@ -1165,8 +1338,9 @@ __device__ __forceinline__ void restrict_sq(const RestrictWeights& wt, int I, in
 // (r_u over sF, r_p over sG, whose tile starts at vertex row j0 - 2) and its restriction to the
 // coarse cells [i0 / 2, i0 / 2 + TX / 2) x [j0 / 2, j0 / 2 + TY / 2) of level n / 2 (planar: PC), with
 // the coarse iterate of those cells set to zero.  All threads of the CTA take part.
-template <class G, int NW, bool PC>
-__device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, const OpCoef<float>& c, const RegCoef& q,
+template <class G, int NW, bool PC, bool LISTS = false>
+__device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
+                                                const MidLists* ml,
                                                 const RestrictWeights& wt, const float2* sU, float2* sF,
                                                 const float* sP, float* sG, float* __restrict__ fc,
                                                 float* __restrict__ gc, float* __restrict__ uc,
@@ -1178,8 +1352,20 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
     const int h = n >> 1;
     const bool fast = (h < i0 - 2 || h >= i0 + TX) && (h < j0 - 2 || h >= j0 + TY);
     if (fast) {
-        if (orient(i0, j0, n) == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, TY, NW, warp, lane, i0, j0, n);
-        else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, TY, NW, warp, lane, i0, j0, n);
+        if (orient(i0, j0, n) == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, warp, TY + 2, NW, lane, i0, j0, n);
+        else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, warp, TY + 2, NW, lane, i0, j0, n);
+    } else if constexpr (LISTS) {
+        mid_cover(h >= i0 - 2 && h < i0 + TX, i0 >= h, h, j0 - 2, TY + 2, NW,
+                  [&](int cls, int r, int end, int step) {
+                      if (cls == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, r, end, step, lane, i0, j0, n);
+                      else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, r, end, step, lane, i0, j0, n);
+                  },
+                  [&](int r) {
+                      const int k = mid_class(i0 - 2 + lane, j0 - 2 + r, n);
+#pragma unroll
+                      for (int s = 0; s < 4; ++s) mid_node<G, false>(*ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n);
+                      if (lane < G::DN) mid_defect_p<G>(*ml, k, sU, UPL, sG, r, lane, i0, j0, n);
+                  });
     } else {
         const ULat<G> vux{sU, UPL, i0 - G::UX, 2 * (j0 - 3), false};
         const ULat<G> vuy{sU, UPL, i0 - G::UX, 2 * (j0 - 3), true};
@@ -1195,7 +1381,7 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
             const int k = r * G::DW + lane + G::DX - 2;
             if (live) {
                 Acc<float> a;
-                cell_apply_auto<true, true, true, false, false>(ci, cj, n, c, vux, vuy, vp, a);
+                cell_apply_auto<true, true, true, false, false>(ci, cj, n, *c, vux, vuy, vp, a);
                 const CellNodes cn = cell_nodes(ci, cj, n);
 #pragma unroll
                 for (int s = 0; s < 4; ++s) {
@@ -1264,8 +1450,7 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
 
 template <int NW, int MINB, bool PC>
 __global__ void __launch_bounds__(32 * NW, MINB)
-    k_restrict_tma(int n, int TY, TileOrder ord, const __grid_constant__ OpCoef<float> c,
-                   const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
+    k_restrict_tma(int n, int TY, TileOrder ord, const MidLists* __restrict__ ml, const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
                    const __grid_constant__ TmaMaps maps, float* __restrict__ fc, float* __restrict__ gc,
                    float* __restrict__ uc, float* __restrict__ pc) {
     using G = TmaTile;
@@ -1305,7 +1490,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         }
         return;
     }
-    defect_restrict<G, NW, PC>(n, TY, i0, j0, c, q, wt, sU, sF, sP, sG, fc, gc, uc, pc);
+    defect_restrict<G, NW, PC, true>(n, TY, i0, j0, nullptr, q, ml, wt, sU, sF, sP, sG, fc, gc, uc, pc);
     pdl_trigger();
 }
 
@@ -1569,7 +1754,7 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
             const int i0 = (t % cols) * G::TX, j0 = (t / cols) * TY;
             stage_compact(n, TY, i0, j0, j0 - 1, xu, xp, L.f, L.g, L.sinv, sU, sF, sP, sG, sS);
             __syncthreads();
-            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, sc[lv - A.clev - 1], A.q[lv], A.tau, A.sigma, sU, sF, sP, sG,
+            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, A.tau, A.sigma, sU, sF, sP, sG,
                                            sS, ou, op);
             __syncthreads();
         }
@@ -1598,7 +1783,7 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
                     stage_compact(n, TY, i0, j0, j0 - 2, sw[l] ? L.tu : L.u, sw[l] ? L.tp : L.p, L.f, L.g, nullptr, sU,
                                   sF, sP, sG, sS);
                     __syncthreads();
-                    defect_restrict<G, kSmallNW, false>(n, TY, i0, j0, sc[l - A.clev - 1], A.q[l], A.wt, sU, sF, sP, sG,
+                    defect_restrict<G, kSmallNW, false>(n, TY, i0, j0, &sc[l - A.clev - 1], A.q[l], nullptr, A.wt, sU, sF, sP, sG,
                                                         C.f, C.g, C.u, C.p);
                     __syncthreads();
                 }
@@ -1657,11 +1842,17 @@ cudaError_t tma_smem_attr() {
                                 (int)TmaTile::bytes(kRegMaxRows));
 }
 
-// Rows per tile for level size n: the least work on the busiest SM, (tiles per SM, rounded up) x
-// (work of one tile, about ty + 4 rows of the u^{m-1/2} region), among the tile heights that keep
-// at least MINB CTAs of kernel k (dynamic shared memory G::bytes(ty)) resident per SM.
+// Rows per tile for level size n, among the tile heights that keep at least MINB CTAs of kernel k (dynamic
+// shared memory G::bytes(ty)) resident per SM.  The planar step (TmaTile): a model of its measured time, the longer of
+// two terms plus a third of the shorter.  The first is the longest CTA, a tile on a mid-line: one unit per pass
+// of its 8 warps over the rows of a phase, ceil((ty + 4) / 8) + ceil((ty + 2) / 8) + ceil(ty / 8), and three for the launch and the
+// tile's arrival; the second the whole GPU's work, tiles x (ty + 7.3) / (9.4 per SM) (the unit is 0.87 us on a GB300).  It
+// picks 4, 4, 12 and 20 or more rows at N = 128, 256, 512 and from 1024 on: 5.5, 6.8, 11.1 us a step, where
+// balancing the tiles over the SMs alone took 5.9, 8.7, 12.9.  `shared` (the solves of a batch, which fill the GPU
+// together): the work plus a third of the longest CTA (24 uneven solves 33.5 against 37.8 ms).  The compact step (RegTile): the least work on the busiest
+// SM, (tiles per SM, rounded up) x (ty + 4).
 template <class G, class K>
-int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false) {
+int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false, bool shared = false) {
     const int lv = 31 - __builtin_clz((unsigned)n);
     int& r = cache[lv & 31];
     if (r) return r;
@@ -1678,7 +1869,11 @@ int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false)
             per_sm < minb)
             continue;
         const long tiles = (long)cols * ((n + 1 + ty - 1) / ty);
-        const double cost = (double)((tiles + sms - 1) / sms) * (ty + 4);
+        double cost = (double)((tiles + sms - 1) / sms) * (ty + 4);
+        if (std::is_same<G, TmaTile>::value) {
+            const double lat = 3.0 + (ty + 11) / 8 + (ty + 9) / 8 + (ty + 7) / 8, thr = (double)tiles * (ty + 7.3) / (9.4 * sms);
+            cost = shared ? thr + 0.35 * lat : std::max(lat, thr) + 0.35 * std::min(lat, thr);
+        }
         if (cost < best) {
             best = cost;
             best_ty = ty;
@@ -1701,9 +1896,9 @@ int reg_rows(int n) {
     return tile_rows<RegTile>(n, k_uzawa_reg<NW, MINB>, 32 * NW, MINB, cache);
 }
 template <int NW, int MINB, bool PAIR = false>
-int tma_rows(int n) {
-    static int cache[32] = {};
-    return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR>, 32 * NW, MINB, cache, PAIR);
+int tma_rows(int n, bool shared) {
+    static int cache[2][32] = {};
+    return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR>, 32 * NW, MINB, cache[shared], PAIR, shared);
 }
 template <class G>
 TileOrder tile_order(int n, int ty) {
@@ -1772,12 +1967,12 @@ bool make_tma_maps(int n, int ty, const float* u, const float* p, const float* f
 }
 
 template <int NW, int MINB, bool PAIR = false>
-bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma, const float* u, const float* p,
+bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau, float sigma, const float* u, const float* p,
                   const float* f, const float* g, const float* sinv, float* u_out, float* p_out, bool prefetch,
                   const CoarseCorrection& cc) {
     RegCoef q;
     if (!make_reg_coef(c, tau, q)) return false;
-    int ty = tma_rows<NW, MINB, PAIR>(n);
+    int ty = tma_rows<NW, MINB, PAIR>(n, ml.shared);
     if (cc.u) ty = std::min(ty, kEmbedMaxRows);
     TmaMaps m;
     if (!make_tma_maps(n, ty, u, p, f, g, sinv, m)) return false;
@@ -1793,8 +1988,8 @@ bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, float tau, floa
         cudaGetLastError();
         pf = std::max(1, sms) * std::max(1, per_sm);
     }
-    launch_pdl(k_uzawa_tma<NW, MINB, PAIR>, dim3(ord.cols * ord.rows), dim3(32 * NW), TmaTile::bytes(ty), s, n, ty, ord, c,
-               q, tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
+    launch_pdl(k_uzawa_tma<NW, MINB, PAIR>, dim3(ord.cols * ord.rows), dim3(32 * NW), TmaTile::bytes(ty), s, n, ty, ord, q,
+               ml.lists, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
     return true;
 }
 
@@ -1826,15 +2021,15 @@ const RestrictWeights& restrict_weights() {
 }
 
 template <bool PC>
-bool launch_rt(cudaStream_t s, int n, const OpCoef<float>& c, const float* u, const float* p, const float* f,
+bool launch_rt(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, const float* u, const float* p, const float* f,
                const float* g, float* fc, float* gc, float* uc, float* pc) {
     RegCoef q;
     if (!make_reg_coef(c, 1.0f, q)) return false;
-    const int ty = std::max(4, tma_rows<8, 3>(n) & ~1);   // even: whole coarse cells per tile
+    const int ty = std::max(4, tma_rows<8, 3>(n, ml.shared) & ~1);   // even: whole coarse cells per tile
     TmaMaps m;
     if (!make_tma_maps(n, ty, u, p, f, g, g, m)) return false;   // no Shat^{-1} tile (its map is unused)
     const TileOrder ord = tile_order<TmaTile>(n, ty);
-    launch_pdl(k_restrict_tma<8, 3, PC>, dim3(ord.cols * ord.rows), dim3(256), TmaTile::bytes(ty), s, n, ty, ord, c, q,
+    launch_pdl(k_restrict_tma<8, 3, PC>, dim3(ord.cols * ord.rows), dim3(256), TmaTile::bytes(ty), s, n, ty, ord, ml.lists, q,
                restrict_weights(), m, fc, gc, uc, pc);
     return true;
 }
@@ -1888,10 +2083,10 @@ cudaError_t launch_small_cycle(cudaStream_t s, const SmallCycleHost& h) {
     return cudaLaunchKernelEx(&cfg, k_small_cycle, A);
 }
 
-bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const float* u, const float* p,
-                         const float* f, const float* g, float* fc, float* gc, float* uc, float* pc) {
-    return pc_planar ? launch_rt<true>(s, n, c, u, p, f, g, fc, gc, uc, pc)
-                     : launch_rt<false>(s, n, c, u, p, f, g, fc, gc, uc, pc);
+bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& ml,
+                         const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc, float* pc) {
+    return pc_planar ? launch_rt<true>(s, n, c, ml, u, p, f, g, fc, gc, uc, pc)
+                     : launch_rt<false>(s, n, c, ml, u, p, f, g, fc, gc, uc, pc);
 }
 
 cudaError_t prepare_uzawa_reg() {
@@ -1920,24 +2115,24 @@ bool g_tma_tuned[32] = {};
 int lvl(int n) { return (31 - __builtin_clz((unsigned)n)) & 31; }
 }  // namespace
 
-bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma,
-                              const float* u, const float* p, const float* f, const float* g, const float* sinv,
+bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
+                              float sigma, const float* u, const float* p, const float* f, const float* g, const float* sinv,
                               float* u_out, float* p_out, const CoarseCorrection& cc) {
     if (cc.u && (!cc.p || !embed_table_matches())) return false;
     switch (variant) {
-        case 1: return launch_tma_v<8, 3>(s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        case 2: return launch_tma_v<8, 4>(s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
-        case 3: return launch_tma_v<8, 4>(s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        case 4: return launch_tma_v<8, 2, true>(s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        case 5: return launch_tma_v<8, 3, true>(s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        default: return launch_tma_v<8, 3>(s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
+        case 1: return launch_tma_v<8, 3>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        case 2: return launch_tma_v<8, 4>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
+        case 3: return launch_tma_v<8, 4>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        case 4: return launch_tma_v<8, 2, true>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        case 5: return launch_tma_v<8, 3, true>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        default: return launch_tma_v<8, 3>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
     }
 }
 
-bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma, const float* u,
-                      const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
+bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau, float sigma,
+                      const float* u, const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
                       const CoarseCorrection& cc) {
-    return launch_uzawa_tma_variant(g_tma_choice[lvl(n)], s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
+    return launch_uzawa_tma_variant(g_tma_choice[lvl(n)], s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
 }
 
 bool uzawa_tma_embed_available() { return uzawa_tma_available() && embed_table_matches(); }
@@ -1958,8 +2153,8 @@ bool set_tma_choice(int n, int v) {
     return true;
 }
 
-cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, float tau, float sigma, float* u,
-                               float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out) {
+cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
+                               float sigma, float* u, float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return cudaErrorUnknown;
     if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -1971,11 +2166,11 @@ cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, fl
     float bms = 1e30f;
     cudaError_t err = cudaSuccess;
     for (int v = 0; v < kTmaVariants && err == cudaSuccess; ++v) {
-        if (!launch_uzawa_tma_variant(v, s, n, c, tau, sigma, u, p, f, g, sinv, u_out, p_out)) continue;   // warm-up
+        if (!launch_uzawa_tma_variant(v, s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out)) continue;   // warm-up
         bool sw = true;
         cudaEventRecord(e0, s);
         for (int r = 0; r < reps; ++r) {
-            launch_uzawa_tma_variant(v, s, n, c, tau, sigma, sw ? u_out : u, sw ? p_out : p, f, g, sinv, sw ? u : u_out,
+            launch_uzawa_tma_variant(v, s, n, c, ml, tau, sigma, sw ? u_out : u, sw ? p_out : p, f, g, sinv, sw ? u : u_out,
                                      sw ? p : p_out);
             sw = !sw;
         }
@@ -1994,6 +2189,38 @@ cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, fl
     g_tma_choice[lvl(n)] = best;
     g_tma_tuned[lvl(n)] = true;
     return cudaGetLastError();
+}
+
+bool fill_mid_lists(MidLists& q, const OpCoef<float>& c, float tau) {
+    using G = TmaTile;
+    const ListStructure& S = list_structure();
+    q = MidLists{};
+    // over the u tile (planes by column parity), the f tile (planes by node type), the vertex tiles
+    auto ou = [](int w) {
+        const int dx = w % 5 - 2, dy = w / 5 - 2;
+        return 4 * (dy * G::UWH + (dx >> 1)) + (dx & 1);
+    };
+    auto of = [](int w) {
+        const int dx = w % 5 - 2, dy = w / 5 - 2;
+        return 4 * ((dy >> 1) * G::FW + (dx >> 1)) + (dx & 1) + 2 * (dy & 1);
+    };
+    static_assert(G::PW == G::DW, "one list of vertex offsets");
+    for (int k = 0; k < kStencilClasses; ++k) {
+        for (int s = 0; s < 4; ++s) {
+            q.ti[k][s] = tau * c.MIdg[k][s];
+            for (int m = list_start(s); m < (s < 3 ? list_start(s + 1) : kListA); ++m)
+                if (const int w = S.A[k][m]; w >= 0) q.A[k][m] = E1<float>{c.MA[k][s][w], ou(w)};
+            for (int m = 4 * (s - 1); s > 0 && m < 4 * s; ++m)
+                if (const int v = S.BT[k][m]; v >= 0)
+                    q.BT[k][m] = E2<float>{c.MBTx[k][s][v], c.MBTy[k][s][v], (v / 3 - 1) * G::PW + v % 3 - 1};
+        }
+        for (int m = 0; m < kListB; ++m)
+            if (const int w = S.B[k][m]; w >= 0) {
+                q.B[k][m] = E2<float>{c.MBx[k][w], c.MBy[k][w], of(w)};
+                q.BU[k][m] = E2<float>{c.MBx[k][w], c.MBy[k][w], ou(w)};
+            }
+    }
+    return S.ok;
 }
 
 bool uzawa_tma_available() { return encode_tiled() != nullptr; }
