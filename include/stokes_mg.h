@@ -169,7 +169,9 @@ stokes_status stokes_sizes(const stokes_handle* h, int* N, size_t* n_vel, size_t
 
 /* One multigrid iteration on the finest level (Sec. 3; V or W by params.gamma), in place on
  * (u, p), followed by the zero-mean projection of p.  Under STOKES_MIXED it is one refinement
- * step: float64 residual, params.inner_cycles float32 cycles on the correction, float64 update. */
+ * step: float64 residual, params.inner_cycles float32 cycles on the correction, float64 update; it keeps
+ * the float32 order of operations of one launch per phase or step (and of the one-CTA cycle below N = 64),
+ * whose rounding its result carries, where the steps of a solve run the faster cluster cycle. */
 stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double* f, const double* g);
 
 /* Iterates stokes_cycle from the given (u, p) until ||F - A x||_2 <= tol ||F||_2 or max_cycles.

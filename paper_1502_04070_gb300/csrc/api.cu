@@ -146,20 +146,6 @@ stokes_status alloc_level(Level<T>& L, int k, DevMem& mem, bool planar = false) 
     return STOKES_OK;
 }
 
-std::mutex g_dev_mu;
-unsigned long long g_dev_weights = 0;   // devices whose constant transfer table is set
-
-stokes_status ensure_weights() {
-    int dev = 0;
-    CK(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lk(g_dev_mu);
-    if (dev < 64 && (g_dev_weights >> dev) & 1ull) return STOKES_OK;
-    static TransferWeights W = transfer_weights();
-    CK(upload_transfer_weights(&W.P2[0][0][0][0]));
-    if (dev < 64) g_dev_weights |= 1ull << dev;
-    return STOKES_OK;
-}
-
 }  // namespace
 
 struct stokes_handle_t {
@@ -189,13 +175,15 @@ struct stokes_handle_t {
     ClusterTables<double>* cl_tab64 = nullptr;
     bool launch_failed = false;             // a step variant refused to launch (reported by the next call)
     bool has_planar = false;                // some float32 level is planar
+    bool plain = false;                     // recording stokes_cycle of a MIXED handle (see there)
     bool shared = false;                    // one of a batch: its kernels run beside those of other solves
     int small_top = -1;                     // float32 levels clev+1..small_top: one cooperative launch per visit
     bool fuse_prolong = false;              // planar levels: x += P x_c inside the first post-smoothing step
     OpCoef<float>* dcoef = nullptr;         // device copies of the float32 operators of levels 0..small_top
     unsigned* dbar = nullptr;               // grid-barrier counter of that launch
     cudaGraphExec_t step = nullptr;         // one cycle + projection + residual norm
-    int step_kernels = 0;                   // kernel nodes in `step`
+    cudaGraphExec_t plain_step = nullptr;   // MIXED: the same for stokes_cycle
+    int step_kernels = 0, plain_kernels = 0;   // kernel nodes in them
     cudaGraphExec_t loop = nullptr;         // WHILE(not converged) { step; device-side test }
     int loop_kernels = 0;                   // kernels per loop iteration
     double* dctl = nullptr;                 // loop control (see k_solve_check), device
@@ -257,6 +245,11 @@ stokes_status take_launch_failure(stokes_handle* h, stokes_status st = STOKES_OK
     return st;
 }
 
+template <typename T>
+PlanarLevel planar_level(const stokes_handle* h, const Level<T>& lv) {
+    return PlanarLevel{h->plain ? nullptr : lv.mid, h->shared};
+}
+
 // nu smoothing steps on level lv.  The state is in (u, p) when `sw` is false and in (tu, tp)
 // when true; returns where it is afterwards.  The fused float32 Uzawa kernel writes the other
 // buffer pair (ping-pong); the float64 and normal-equation steps work in place and use the other
@@ -279,11 +272,11 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
         } else if constexpr (sizeof(T) == 4) {
             if (h->dom == kDomL) {   // the L: the per-phase kernels (in place), the removed quadrant kept zero
                 launch_uzawa<float>(h->st, lv.n, lv.c, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op,
-                                    32, 8, h->dom);
+                                    0, 0, h->dom);
             } else if (lv.planar) {
                 CoarseCorrection cc;
                 if (coarse && s == 0) cc = CoarseCorrection{coarse->u, coarse->p, coarse->planar};
-                if (launch_uzawa_tma(h->st, lv.n, lv.c, PlanarLevel{lv.mid, h->shared}, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou,
+                if (launch_uzawa_tma(h->st, lv.n, lv.c, planar_level(h, lv), (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou,
                                      op, cc))
                     sw = !sw;
                 else
@@ -293,7 +286,7 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
                 sw = !sw;
             }
         } else {
-            launch_uzawa<T>(h->st, lv.n, lv.c, (T)P.tau, (T)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op, 32, 8, h->dom);
+            launch_uzawa<T>(h->st, lv.n, lv.c, (T)P.tau, (T)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op, 0, 0, h->dom);
         }
         ev_end(h, k);
     }
@@ -405,7 +398,29 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
             return;
         }
     }
-    if (l <= h->cl_top && !lv.planar) {
+    if constexpr (sizeof(T) == 4) {
+        if (h->plain && l <= kCoarseCycleTop && h->prm.gamma == 1 && h->prm.smoother == STOKES_UZAWA && h->clev == 0 &&
+            h->dom == kDomSquare) {
+            CoarseCycleArgs a;
+            for (int k = 1; k <= l; ++k) {
+                a.c[k - 1] = H[k].c;
+                a.sinv[k - 1] = H[k].sinv;
+            }
+            a.inv = h->inv;
+            a.u = lv.u;
+            a.p = lv.p;
+            a.f = lv.f;
+            a.g = lv.g;
+            a.tau = (float)h->prm.tau;
+            a.sigma = (float)h->prm.sigma;
+            a.nu_pre = h->prm.nu_pre;
+            a.nu_post = h->prm.nu_post;
+            a.top = l;
+            launch_coarse_cycle(h->st, a);
+            return;
+        }
+    }
+    if (l <= h->cl_top && !lv.planar && !h->plain) {
         cluster_visit<T>(h, H, l, zero);
         return;
     }
@@ -421,7 +436,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
     if constexpr (sizeof(T) == 4) {
         if (lv.planar) {
             // the defect and its restriction in one kernel on the staged tiles (the defect stays on chip)
-            if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, PlanarLevel{lv.mid, h->shared}, xu, xp, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p)) {
+            if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, planar_level(h, lv), xu, xp, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p)) {
                 launch_residual_planar(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp);
                 launch_restrict_planar(h->st, cl.n, cl.planar, ru, rp, cl.f, cl.g, cl.u, cl.p);
             }
@@ -488,8 +503,8 @@ void record_step(stokes_handle* h) {
     }
 }
 
-stokes_status build_graph(stokes_handle* h) {
-    if (h->step) return STOKES_OK;
+stokes_status capture_step(stokes_handle* h, cudaGraphExec_t* exec, int* kernels) {
+    if (*exec) return STOKES_OK;
     cudaGraph_t g = nullptr;
     h->ev_cursor = h->ev_smooth = h->ev_resid = 0;
     CK(cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
@@ -500,18 +515,33 @@ stokes_status build_graph(stokes_handle* h) {
     cudaGraphGetNodes(g, nullptr, &nn);
     std::vector<cudaGraphNode_t> nodes(nn);
     cudaGraphGetNodes(g, nodes.data(), &nn);
-    h->step_kernels = 0;
+    *kernels = 0;
     for (auto nd : nodes) {
         cudaGraphNodeType ty;
-        if (cudaGraphNodeGetType(nd, &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel) h->step_kernels++;
+        if (cudaGraphNodeGetType(nd, &ty) == cudaSuccess && ty == cudaGraphNodeTypeKernel) ++*kernels;
     }
-    e = cudaGraphInstantiate(&h->step, g, 0);
+    e = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-        h->step = nullptr;
+        *exec = nullptr;
         return fail(e);
     }
     return STOKES_OK;
+}
+
+stokes_status build_graph(stokes_handle* h) { return capture_step(h, &h->step, &h->step_kernels); }
+
+// stokes_cycle on a MIXED handle: its result is one float32 cycle's, rounding included, and nothing after it removes
+// that rounding; it keeps the order of float32 operations it has always had (the one-CTA coarse cycle, per-cell
+// rows on the mid-lines), so that it returns the same values, about half as fast as a step inside a solve.
+stokes_status build_plain_graph(stokes_handle* h) {
+    const bool timing = h->timing;
+    h->timing = false;
+    h->plain = true;
+    const stokes_status s = capture_step(h, &h->plain_step, &h->plain_kernels);
+    h->plain = false;
+    h->timing = timing;
+    return s;
 }
 
 // The solve loop on the device: one conditional WHILE node whose body is one step followed by
@@ -607,6 +637,7 @@ stokes_status rebuild_beta(stokes_handle* h) {
     const double beta = h->prm.beta;
     for (auto& lv : h->h64) {
         lv.c = make_coef<double>(lv.n, beta);
+        if (!stencil_masks_cover(lv.c)) return STOKES_ERR_BAD_ARG;   // no beta does
         launch_schur_diag<double>(h->st, lv.n, lv.c, lv.sinv, h->dom);
     }
     for (auto& lv : h->h32) {
@@ -659,6 +690,10 @@ stokes_status rebuild_beta(stokes_handle* h) {
     if (h->step) {
         cudaGraphExecDestroy(h->step);
         h->step = nullptr;
+    }
+    if (h->plain_step) {
+        cudaGraphExecDestroy(h->plain_step);
+        h->plain_step = nullptr;
     }
     if (h->loop) {
         cudaGraphExecDestroy(h->loop);
@@ -737,6 +772,7 @@ void stokes_destroy(stokes_handle* h) {
     if (!h) return;
     if (h->st) cudaStreamSynchronize(h->st);
     if (h->step) cudaGraphExecDestroy(h->step);
+    if (h->plain_step) cudaGraphExecDestroy(h->plain_step);
     if (h->loop) cudaGraphExecDestroy(h->loop);
     if (h->euler) cudaGraphExecDestroy(h->euler);
     if (h->hhist) cudaFreeHost(h->hhist);
@@ -765,10 +801,9 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
     // level 1 (the L's level 0)
     if (P.domain == STOKES_L_SHAPE && (P.smoother != STOKES_UZAWA || P.coarse_level != 1 || P.levels < 2))
         return STOKES_ERR_BAD_ARG;
-    stokes_status s = ensure_weights();
-    if (s != STOKES_OK) return s;
+    stokes_status s = STOKES_OK;
     if (prepare_uzawa_fused<float>() != cudaSuccess || prepare_uzawa_fused<double>() != cudaSuccess ||
-        prepare_uzawa_pair() != cudaSuccess ||
+        prepare_coarse_cycle() != cudaSuccess || prepare_uzawa_pair() != cudaSuccess ||
         prepare_uzawa_reg() != cudaSuccess || prepare_dense_solve(bordered_size(1 << (kMaxCoarseLevel + 1))) != cudaSuccess)
         return STOKES_ERR_CUDA;
     stokes_handle* h = new stokes_handle_t();
@@ -870,6 +905,10 @@ stokes_status stokes_autotune(stokes_handle* h) {
         cudaGraphExecDestroy(h->step);
         h->step = nullptr;
     }
+    if (s == STOKES_OK && h->plain_step) {
+        cudaGraphExecDestroy(h->plain_step);
+        h->plain_step = nullptr;
+    }
     if (s == STOKES_OK && h->loop) {
         cudaGraphExecDestroy(h->loop);
         h->loop = nullptr;
@@ -915,10 +954,12 @@ stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double*
     if (h->mixed()) {
         residual_norm_fin(h);   // float64 residual and the float32 right-hand side of the correction
         h->launches += 2;
+        if ((s = build_plain_graph(h)) != STOKES_OK) return s;
+        CK(cudaGraphLaunch(h->plain_step, h->st));
+        h->launches += h->plain_kernels;
+    } else {
+        if ((s = build_graph(h)) != STOKES_OK || (s = launch_step(h)) != STOKES_OK) return s;
     }
-    if ((s = build_graph(h)) != STOKES_OK) return s;
-    stokes_status s2 = launch_step(h);
-    if (s2 != STOKES_OK) return s2;
     return take_launch_failure(h, copy_out(h, u, p));
 }
 
@@ -1110,7 +1151,7 @@ stokes_status stokes_residual_restrict_f32(stokes_handle* h, const float* u, con
     if (lv.planar) {
         launch_to_planar(h->st, lv.n, u, p, lv.u, lv.p);
         launch_to_planar(h->st, lv.n, f, g, lv.f, lv.g);
-        if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, PlanarLevel{lv.mid, h->shared}, lv.u, lv.p, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p))
+        if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, planar_level(h, lv), lv.u, lv.p, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p))
             return STOKES_ERR_CUDA;
         if (cl.planar) {
             launch_from_planar(h->st, cl.n, cl.f, cl.g, fc, gc);
@@ -1178,7 +1219,9 @@ stokes_status stokes_stencil_rows(int levels, double beta, int cls, double* ma, 
 
 stokes_status stokes_step_tables_match(int levels, double beta) {
     if (levels < 1 || levels > 13 || !(beta >= 0.0) || !std::isfinite(beta)) return STOKES_ERR_BAD_ARG;
-    return reg_tables_match(make_coef<float>(1 << levels, beta)) ? STOKES_OK : STOKES_ERR_BAD_ARG;
+    return reg_tables_match(make_coef<float>(1 << levels, beta)) && stencil_masks_cover(make_coef<double>(1 << levels, beta))
+               ? STOKES_OK
+               : STOKES_ERR_BAD_ARG;
 }
 
 stokes_status stokes_transfer_weights(double* w) {
@@ -1277,10 +1320,17 @@ static stokes_status autotune_levels(stokes_handle* h, cudaStream_t st) {
     for (int l = 1; l < (int)h->h32.size(); ++l) {
         Level<float>& lv = h->h32[l];
         if (lv.planar ? tma_tuned(lv.n) : uzawa_tuned(lv.n)) continue;
-        cudaError_t e = lv.planar ? autotune_uzawa_tma(st, lv.n, lv.c, PlanarLevel{lv.mid, h->shared}, (float)h->prm.tau, (float)h->prm.sigma, lv.u, lv.p,
-                                                       lv.f, lv.g, lv.sinv, lv.tu, lv.tp)
-                                  : autotune_uzawa_fused(st, lv.n, lv.c, (float)h->prm.tau, (float)h->prm.sigma, lv.u,
-                                                         lv.p, lv.f, lv.g, lv.sinv, lv.tu, lv.tp, nullptr, nullptr);
+        auto planar = [&](const PlanarLevel& pl) {
+            return autotune_uzawa_tma(st, lv.n, lv.c, pl, (float)h->prm.tau, (float)h->prm.sigma, lv.u, lv.p, lv.f, lv.g, lv.sinv,
+                                      lv.tu, lv.tp);
+        };
+        cudaError_t e = cudaSuccess;
+        if (lv.planar) {
+            if ((e = planar(PlanarLevel{lv.mid, h->shared})) == cudaSuccess) e = planar(PlanarLevel{});   // and stokes_cycle's
+        } else {
+            e = autotune_uzawa_fused(st, lv.n, lv.c, (float)h->prm.tau, (float)h->prm.sigma, lv.u, lv.p, lv.f, lv.g, lv.sinv, lv.tu,
+                                     lv.tp, nullptr, nullptr);
+        }
         if (e != cudaSuccess) return fail(e);
         cudaMemsetAsync(lv.u, 0, 2 * lv.n2 * sizeof(float), st);
         cudaMemsetAsync(lv.p, 0, lv.n1 * sizeof(float), st);

@@ -3,16 +3,22 @@
 // A "view" maps P2-lattice coordinates (X, Y) (or vertex coordinates for pressure) to values; the
 // same row code reads global memory through the read-only path or a shared-memory tile.
 #pragma once
+#include <type_traits>
 #include <utility>
 
 #include "common.cuh"
 
 namespace smg {
 
-constexpr int BX = 32, BY = 8, NT = BX * BY;
+constexpr int BX = 32, BY = 8, NT = BX * BY;   // threads of a block at most
 
+// One thread per cell, in blocks of BX x BY cells, lower ones on levels with few cells so that their warps reach all
+// SMs: a float64 warp instruction occupies its pipe for 64 clocks, so eight warps on one SM and none on the next
+// is eight times the time.  N <= 128: one warp a block (645 blocks at N = 128), N = 256: four (585).
+__host__ __device__ constexpr int cells_by(int n) { return n <= 128 ? 1 : n <= 256 ? 4 : BY; }
 int cells_blocks(int n);
-inline dim3 cells_grid(int n) { return dim3((n + 1 + BX - 1) / BX, (n + 1 + BY - 1) / BY); }
+inline dim3 cells_block(int n) { return dim3(BX, cells_by(n)); }
+inline dim3 cells_grid(int n) { return dim3((n + 1 + BX - 1) / BX, (n + 1 + cells_by(n) - 1) / cells_by(n)); }
 
 // ------------------------------------------------------------------------------------------
 // rows of the square at position SQ relative to the cell: SQ 0 = (i, j), 1 = (i-1, j),
@@ -274,90 +280,89 @@ __device__ __forceinline__ void vwin_load(int i, int j, int n, const VP& p, T (&
     (vwin_load1<C, V>(i, j, n, p, pw), ...);
 }
 
-template <int C, int S, int K, typename T>
-__device__ __forceinline__ void ma_term(const OpCoef<T>& c, const T (&w)[25], T& s) {
-    if constexpr (nz_MA(C, S, K)) s = fma(c.MA[C][S][K], w[K], s);
-}
-template <int C, int S, typename T, int... K>
-__device__ __forceinline__ T ma_row_i(const OpCoef<T>& c, const T (&w)[25], std::integer_sequence<int, K...>) {
-    T s = T(0);
-    (ma_term<C, S, K>(c, w, s), ...);
-    return s;
-}
-template <int C, int S, typename T>
-__device__ __forceinline__ T ma_row(const OpCoef<T>& c, const T (&w)[25]) {
-    return ma_row_i<C, S>(c, w, std::make_integer_sequence<int, 25>{});
-}
-
-template <int C, int S, int K, typename T>
-__device__ __forceinline__ void mbt_term(const T (&B)[kStencilClasses][4][9], const T (&pw)[9], T& s) {
-    if constexpr (nz_MBT(C, S, K)) s = fma(B[C][S][K], pw[K], s);
-}
-template <int C, int S, typename T, int... K>
-__device__ __forceinline__ T mbt_row_i(const T (&B)[kStencilClasses][4][9], const T (&pw)[9],
+// SUB: the products are subtracted from what the accumulator holds
+template <bool SUB, typename T>
+__device__ __forceinline__ void acc_fma(T c, T v, T& s) { s = SUB ? fma(-c, v, s) : fma(c, v, s); }
+template <bool SUB, int C, int S, typename T, int... K>
+__device__ __forceinline__ void ma_row(const T (&m)[kStencilClasses][4][25], const T (&wx)[25], const T (&wy)[25], T& sx, T& sy,
                                        std::integer_sequence<int, K...>) {
-    T s = T(0);
-    (mbt_term<C, S, K>(B, pw, s), ...);
-    return s;
+    auto term = [&](auto kk) {
+        constexpr int k = decltype(kk)::value;
+        if constexpr (nz_MA(C, S, k)) {
+            acc_fma<SUB>(m[C][S][k], wx[k], sx);
+            acc_fma<SUB>(m[C][S][k], wy[k], sy);
+        }
+    };
+    (term(std::integral_constant<int, K>{}), ...);
 }
-template <int C, int S, typename T>
-__device__ __forceinline__ T mbt_row(const T (&B)[kStencilClasses][4][9], const T (&pw)[9]) {
-    return mbt_row_i<C, S>(B, pw, std::make_integer_sequence<int, 9>{});
+template <bool SUB, int C, int S, typename T, int... V>
+__device__ __forceinline__ void mbt_row(const OpCoef<T>& c, const T (&pw)[9], T& sx, T& sy, std::integer_sequence<int, V...>) {
+    auto term = [&](auto vv) {
+        constexpr int v = decltype(vv)::value;
+        if constexpr (nz_MBTx(C, S, v)) acc_fma<SUB>(c.MBTx[C][S][v], pw[v], sx);
+        if constexpr (nz_MBTy(C, S, v)) acc_fma<SUB>(c.MBTy[C][S][v], pw[v], sy);
+    };
+    (term(std::integral_constant<int, V>{}), ...);
+}
+template <bool SUB, int C, typename T, int... K>
+__device__ __forceinline__ void mb_row(const OpCoef<T>& c, const T (&wx)[25], const T (&wy)[25], T& s,
+                                       std::integer_sequence<int, K...>) {
+    auto term = [&](auto kk) {
+        constexpr int k = decltype(kk)::value;
+        if constexpr (nz_MBy(C, k)) acc_fma<SUB>(c.MBy[C][k], wy[k], s);
+        if constexpr (nz_MBx(C, k)) acc_fma<SUB>(c.MBx[C][k], wx[k], s);
+    };
+    (term(std::integral_constant<int, K>{}), ...);
 }
 
-template <int C, int K, typename T>
-__device__ __forceinline__ void mb_term(const OpCoef<T>& c, const T (&wx)[25], const T (&wy)[25], T& s) {
-    if constexpr (nz_MB(C, K)) s = fma(c.MBx[C][K], wx[K], fma(c.MBy[C][K], wy[K], s));
-}
-template <int C, typename T, int... K>
-__device__ __forceinline__ T mb_row_i(const OpCoef<T>& c, const T (&wx)[25], const T (&wy)[25],
-                                      std::integer_sequence<int, K...>) {
-    T s = T(0);
-    (mb_term<C, K>(c, wx, wy, s), ...);
-    return s;
-}
-
-template <bool DA, bool DBT, bool DB, bool DD, bool MASK, int C, typename T, typename VU, typename VP>
+// SUB false: a.au = A u, a.bt = B^T p, a.bu = B u.  SUB true: a.au, a.bu come in as f, g and go out as f - A u - B^T p and
+// g - B u (a.bt is not used): no separate subtractions.
+template <bool DA, bool DBT, bool DB, bool DD, bool MASK, int C, bool SUB, typename T, typename VU, typename VP>
 __device__ __forceinline__ void cell_apply_merged(int i, int j, int n, const OpCoef<T>& c, const VU& ux, const VU& uy,
                                                   const VP& p, Acc<T>& a) {
+    constexpr auto K25 = std::make_integer_sequence<int, 25>{};
+    constexpr auto V9 = std::make_integer_sequence<int, 9>{};
     T wx[25], wy[25], pw[9];
-    if constexpr (DA || DB) win_load<C, DA, DB, MASK>(i, j, n, ux, uy, wx, wy, std::make_integer_sequence<int, 25>{});
-    if constexpr (DBT) vwin_load<C>(i, j, n, p, pw, std::make_integer_sequence<int, 9>{});
+    if constexpr (DA || DB) win_load<C, DA, DB, MASK>(i, j, n, ux, uy, wx, wy, K25);
+    if constexpr (DBT) vwin_load<C>(i, j, n, p, pw, V9);
+    if constexpr (!SUB) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) a.au[0][s] = a.au[1][s] = a.bt[0][s] = a.bt[1][s] = a.idg[s] = T(0);
-    a.bu = T(0);
+        for (int s = 0; s < 4; ++s) a.au[0][s] = a.au[1][s] = a.bt[0][s] = a.bt[1][s] = a.idg[s] = T(0);
+        a.bu = T(0);
+    }
     if constexpr (DA) {
-        a.au[0][0] = ma_row<C, 0>(c, wx); a.au[1][0] = ma_row<C, 0>(c, wy);
-        a.au[0][1] = ma_row<C, 1>(c, wx); a.au[1][1] = ma_row<C, 1>(c, wy);
-        a.au[0][2] = ma_row<C, 2>(c, wx); a.au[1][2] = ma_row<C, 2>(c, wy);
-        a.au[0][3] = ma_row<C, 3>(c, wx); a.au[1][3] = ma_row<C, 3>(c, wy);
+        ma_row<SUB, C, 0>(c.MA, wx, wy, a.au[0][0], a.au[1][0], K25);
+        ma_row<SUB, C, 1>(c.MA, wx, wy, a.au[0][1], a.au[1][1], K25);
+        ma_row<SUB, C, 2>(c.MA, wx, wy, a.au[0][2], a.au[1][2], K25);
+        ma_row<SUB, C, 3>(c.MA, wx, wy, a.au[0][3], a.au[1][3], K25);
     }
     if constexpr (DBT) {
-        a.bt[0][0] = mbt_row<C, 0>(c.MBTx, pw); a.bt[1][0] = mbt_row<C, 0>(c.MBTy, pw);
-        a.bt[0][1] = mbt_row<C, 1>(c.MBTx, pw); a.bt[1][1] = mbt_row<C, 1>(c.MBTy, pw);
-        a.bt[0][2] = mbt_row<C, 2>(c.MBTx, pw); a.bt[1][2] = mbt_row<C, 2>(c.MBTy, pw);
-        a.bt[0][3] = mbt_row<C, 3>(c.MBTx, pw); a.bt[1][3] = mbt_row<C, 3>(c.MBTy, pw);
+        auto& r = SUB ? a.au : a.bt;
+        mbt_row<SUB, C, 0>(c, pw, r[0][0], r[1][0], V9);
+        mbt_row<SUB, C, 1>(c, pw, r[0][1], r[1][1], V9);
+        mbt_row<SUB, C, 2>(c, pw, r[0][2], r[1][2], V9);
+        mbt_row<SUB, C, 3>(c, pw, r[0][3], r[1][3], V9);
     }
     if constexpr (DD) {
 #pragma unroll
         for (int s = 0; s < 4; ++s) a.idg[s] = c.MIdg[C][s];
     }
-    if constexpr (DB) a.bu = mb_row_i<C>(c, wx, wy, std::make_integer_sequence<int, 25>{});
+    if constexpr (DB) mb_row<SUB, C>(c, wx, wy, a.bu, K25);
 }
 
 // Operator rows of cell (i, j) from the merged stencils of its class (branch uniform across a warp
 // except where the warp meets a mid-line).
-template <bool DA, bool DBT, bool DB, bool DD, bool MASK, typename T, typename VU, typename VP>
+template <bool DA, bool DBT, bool DB, bool DD, bool MASK, bool SUB = false, typename T, typename VU, typename VP>
 __device__ __forceinline__ void cell_apply_auto(int i, int j, int n, const OpCoef<T>& c, const VU& ux, const VU& uy,
                                                 const VP& p, Acc<T>& a) {
     switch (stencil_class(i, j, n)) {
-        case 0: cell_apply_merged<DA, DBT, DB, DD, MASK, 0>(i, j, n, c, ux, uy, p, a); break;
-        case 1: cell_apply_merged<DA, DBT, DB, DD, MASK, 1>(i, j, n, c, ux, uy, p, a); break;
-        case 2: cell_apply_merged<DA, DBT, DB, DD, MASK, 2>(i, j, n, c, ux, uy, p, a); break;
-        case 3: cell_apply_merged<DA, DBT, DB, DD, MASK, 3>(i, j, n, c, ux, uy, p, a); break;
-        case 4: cell_apply_merged<DA, DBT, DB, DD, MASK, 4>(i, j, n, c, ux, uy, p, a); break;
-        case 5: cell_apply_merged<DA, DBT, DB, DD, MASK, 5>(i, j, n, c, ux, uy, p, a); break;
-        default: cell_apply_merged<DA, DBT, DB, DD, MASK, 6>(i, j, n, c, ux, uy, p, a); break;
+        case 0: cell_apply_merged<DA, DBT, DB, DD, MASK, 0, SUB>(i, j, n, c, ux, uy, p, a); break;
+        case 1: cell_apply_merged<DA, DBT, DB, DD, MASK, 1, SUB>(i, j, n, c, ux, uy, p, a); break;
+        case 2: cell_apply_merged<DA, DBT, DB, DD, MASK, 2, SUB>(i, j, n, c, ux, uy, p, a); break;
+        case 3: cell_apply_merged<DA, DBT, DB, DD, MASK, 3, SUB>(i, j, n, c, ux, uy, p, a); break;
+        case 4: cell_apply_merged<DA, DBT, DB, DD, MASK, 4, SUB>(i, j, n, c, ux, uy, p, a); break;
+        case 5: cell_apply_merged<DA, DBT, DB, DD, MASK, 5, SUB>(i, j, n, c, ux, uy, p, a); break;
+        default: cell_apply_merged<DA, DBT, DB, DD, MASK, 6, SUB>(i, j, n, c, ux, uy, p, a); break;
     }
 }
 
@@ -373,7 +378,7 @@ __device__ __forceinline__ bool slot_unknown(const CellNodes& cn, int s) {
     return s == 0 ? cn.v : s == 1 ? cn.h : s == 2 ? cn.e : cn.c;
 }
 
-// (kernels that reduce over the block with block_sum2d are launched with BX x BY threads)
+// (blocks of whole warps, at most NT threads: the block sums below)
 #define CELL_INDEX                                          \
     const int i = blockIdx.x * blockDim.x + threadIdx.x;    \
     const int j = blockIdx.y * blockDim.y + threadIdx.y;    \
@@ -393,7 +398,7 @@ __device__ __forceinline__ double2 block_sum2d_pair(double a, double b, int tid)
     __syncthreads();
     double2 s = make_double2(0.0, 0.0);
     if (tid < 32) {
-        s = tid < NT / 32 ? red2[tid] : make_double2(0.0, 0.0);
+        s = tid < (int)(blockDim.x * blockDim.y) / 32 ? red2[tid] : make_double2(0.0, 0.0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             s.x += __shfl_down_sync(0xffffffffu, s.x, o);
@@ -421,8 +426,8 @@ __device__ __forceinline__ double2 block_sum2_fd(float a, double b, int tid) {
     float sa = 0.f;
     double sb = 0.0;
     if (tid < 32) {
-        sa = tid < NT / 32 ? redf[tid] : 0.f;
-        sb = tid < NT / 32 ? redd[tid] : 0.0;
+        sa = tid < (int)(blockDim.x * blockDim.y) / 32 ? redf[tid] : 0.f;
+        sb = tid < (int)(blockDim.x * blockDim.y) / 32 ? redd[tid] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             sa += __shfl_down_sync(0xffffffffu, sa, o);
@@ -441,7 +446,7 @@ __device__ __forceinline__ double block_sum2d(double v, int tid) {
     __syncthreads();
     double s = 0.0;
     if (tid < 32) {
-        s = tid < NT / 32 ? red[tid] : 0.0;
+        s = tid < (int)(blockDim.x * blockDim.y) / 32 ? red[tid] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     }

@@ -58,6 +58,11 @@ template <typename T>
 struct MassCoef {          // mass matrices of one level (load vectors, adjoint)
     T M[2][9][9];
     T MP[2][4][4];
+    // node and vertex stencils per class, as OpCoef's: rows of the velocity mass at the four owned nodes, of the
+    // pressure mass at the owned vertex (all four squares inside the domain) and that row's sum
+    T MM[kStencilClasses][4][25];
+    T MMP[kStencilClasses][9];
+    T MW[kStencilClasses];
 };
 
 // triangle membership of local P2 nodes, per orientation (bit m set if node m lies in the triangle)
@@ -86,30 +91,67 @@ __host__ __device__ constexpr int sq_win(int SQ, int m) { return (m / 3 - 2 * (S
 // vertex offset (from (i, j)) of corner q of square SQ, as a 3 x 3 window index
 __host__ __device__ constexpr int sq_vwin(int SQ, int q) { return (q / 2 - (SQ >> 1) + 1) * 3 + (q % 2 - (SQ & 1) + 1); }
 
-// structural nonzeros of the merged stencils of class k (compile-time)
+// Nonzeros of the merged stencils of class k (compile-time), one bit per window point.  Fewer than the
+// couplings of the triangles: the P2 stiffness has zeros on right isosceles triangles, the P2 mass others, and
+// contributions of neighbouring triangles cancel.  The same for every beta and h (stencil_masks_cover checks
+// a level's coefficients against them): 17 + 9 + 9 + 7 entries of A in every class but the centre's (21), 10 of each
+// component of B^T and 10 of B (14 at the centre) - the float64 kernels' time is their count of float64
+// instructions.
 __host__ __device__ constexpr bool nz_MA(int k, int s, int w) {
-    for (int SQ = 0; SQ < 4; ++SQ) {
-        const int L = sq_local(SQ, s);
-        if (L < 0) continue;
-        for (int m = 0; m < 9; ++m)
-            if (sq_win(SQ, m) == w && couple(sq_orient(k, SQ), L, m)) return true;
-    }
-    return false;
+    constexpr unsigned m[kStencilClasses][4] = {
+        {0x1cb7da7, 0x10c7184, 0x1c71c00, 0x0ce6000}, {0x076fedc, 0x0467310, 0x0777000, 0x18e3000},
+        {0x0477ebf, 0x0467310, 0x0477c00, 0x18e3000}, {0x1fafdc4, 0x10c7184, 0x1f71000, 0x0ce6000},
+        {0x076fda7, 0x0467184, 0x0777000, 0x18e3000}, {0x1cb7edc, 0x10c7310, 0x1c71c00, 0x0ce6000},
+        {0x1fafebf, 0x10c7310, 0x1f71000, 0x0ce6000}};
+    return (m[k][s] >> w) & 1u;
 }
-__host__ __device__ constexpr bool nz_MBT(int k, int s, int v) {
-    for (int SQ = 0; SQ < 4; ++SQ) {
-        const int L = sq_local(SQ, s);
-        if (L < 0) continue;
-        for (int q = 0; q < 4; ++q)
-            if (sq_vwin(SQ, q) == v && couple(sq_orient(k, SQ), corner_node(q), L)) return true;
-    }
-    return false;
+__host__ __device__ constexpr bool nz_MBTx(int k, int s, int v) {
+    constexpr unsigned m[kStencilClasses][4] = {{0, 0x030, 0x198, 0x1b0}, {0, 0x030, 0x0f0, 0x1b0}, {0, 0x030, 0x028, 0x1b0},
+                                                {0, 0x030, 0x140, 0x1b0}, {0, 0x030, 0x0f0, 0x1b0}, {0, 0x030, 0x198, 0x1b0},
+                                                {0, 0x030, 0x140, 0x1b0}};
+    return (m[k][s] >> v) & 1u;
 }
-__host__ __device__ constexpr bool nz_MB(int k, int w) {
-    for (int SQ = 0; SQ < 4; ++SQ)
-        for (int m = 0; m < 9; ++m)
-            if (sq_win(SQ, m) == w && couple(sq_orient(k, SQ), corner_node(SQ), m)) return true;
-    return false;
+__host__ __device__ constexpr bool nz_MBTy(int k, int s, int v) {
+    constexpr unsigned m[kStencilClasses][4] = {{0, 0x132, 0x090, 0x1b0}, {0, 0x0b4, 0x090, 0x1b0}, {0, 0x0b4, 0x090, 0x1b0},
+                                                {0, 0x132, 0x090, 0x1b0}, {0, 0x082, 0x090, 0x1b0}, {0, 0x104, 0x090, 0x1b0},
+                                                {0, 0x104, 0x090, 0x1b0}};
+    return (m[k][s] >> v) & 1u;
+}
+__host__ __device__ constexpr bool nz_MBx(int k, int w) {
+    constexpr unsigned m[kStencilClasses] = {0x00f29e0, 0x007abc0, 0x0052b60, 0x00da940, 0x007a9e0, 0x00f2bc0, 0x00dab60};
+    return (m[k] >> w) & 1u;
+}
+__host__ __device__ constexpr bool nz_MBy(int k, int w) {
+    constexpr unsigned m[kStencilClasses] = {0x08729c2, 0x02729c8, 0x00729ca, 0x0a729c0, 0x02701c2, 0x08701c8, 0x0a701ca};
+    return (m[k] >> w) & 1u;
+}
+__host__ __device__ constexpr bool nz_MBT(int k, int s, int v) { return nz_MBTx(k, s, v) || nz_MBTy(k, s, v); }
+__host__ __device__ constexpr bool nz_MB(int k, int w) { return nz_MBx(k, w) || nz_MBy(k, w); }
+// host: every entry of the level's merged stencils off these masks is zero up to rounding
+template <typename T>
+inline bool stencil_masks_cover(const OpCoef<T>& c) {
+    const double tol = sizeof(T) == 4 ? 1e-6 : 1e-14;
+    auto abs = [](double v) { return v < 0.0 ? -v : v; };
+    double amax = 0.0, bmax = 0.0, a = 0.0, b = 0.0;   // largest entry, largest off the masks
+    auto see = [&](bool on, double v, double& all, double& off) {
+        v = abs(v);
+        if (v > all) all = v;
+        if (!on && v > off) off = v;
+    };
+    for (int k = 0; k < kStencilClasses; ++k) {
+        for (int s = 0; s < 4; ++s) {
+            for (int w = 0; w < 25; ++w) see(nz_MA(k, s, w), c.MA[k][s][w], amax, a);
+            for (int v = 0; v < 9; ++v) {
+                see(nz_MBTx(k, s, v), c.MBTx[k][s][v], bmax, b);
+                see(nz_MBTy(k, s, v), c.MBTy[k][s][v], bmax, b);
+            }
+        }
+        for (int w = 0; w < 25; ++w) {
+            see(nz_MBx(k, w), c.MBx[k][w], bmax, b);
+            see(nz_MBy(k, w), c.MBy[k][w], bmax, b);
+        }
+    }
+    return amax > 0.0 && bmax > 0.0 && a <= tol * amax && b <= tol * bmax;
 }
 
 // host: merged stencils from the square-local matrices (sums over the squares that share a node)
@@ -152,6 +194,27 @@ inline void fill_merged(OpCoef<T>& c) {
     }
 }
 
+template <typename T>
+inline void fill_merged(MassCoef<T>& m) {
+    for (int k = 0; k < kStencilClasses; ++k) {
+        double p[9] = {}, w = 0.0;
+        for (int s = 0; s < 4; ++s) {
+            double a[25] = {};
+            for (int SQ = 0; SQ < 4; ++SQ)
+                if (const int L = sq_local(SQ, s); L >= 0)
+                    for (int q = 0; q < 9; ++q) a[sq_win(SQ, q)] += (double)m.M[sq_orient(k, SQ)][L][q];
+            for (int q = 0; q < 25; ++q) m.MM[k][s][q] = (T)a[q];
+        }
+        for (int SQ = 0; SQ < 4; ++SQ)
+            for (int q = 0; q < 4; ++q) {
+                p[sq_vwin(SQ, q)] += (double)m.MP[sq_orient(k, SQ)][SQ][q];
+                w += (double)m.MP[sq_orient(k, SQ)][SQ][q];
+            }
+        for (int q = 0; q < 9; ++q) m.MMP[k][q] = (T)p[q];
+        m.MW[k] = (T)w;
+    }
+}
+
 __host__ __device__ __forceinline__ int orient(int si, int sj, int n) {
     const int h = n >> 1;
     return (si < h) != (sj < h);
@@ -170,7 +233,8 @@ __device__ __forceinline__ int vertex_triangles(int i, int j, int n) {
     return cnt;
 }
 
-// w_i = int psi_i = (number of triangles at vertex i) h^2 / 6: the pressure-mean weight (M_P 1)_i
+// w_i = int psi_i = (number of triangles at vertex i) h^2 / 6: the pressure-mean weight (M_P 1)_i (two float64
+// divisions: kernels that sum over all vertices count triangles and scale their sums)
 __device__ __forceinline__ double vertex_weight(int i, int j, int n) {
     const double h = 1.0 / n;
     return vertex_triangles(i, j, n) * h * h / 6.0;

@@ -11,10 +11,14 @@
 
 #include "cellops.cuh"
 #include "kernels.cuh"
+#include "stencil_tables.cuh"
 
 namespace smg {
 
-int cells_blocks(int n) { return ((n + 1 + BX - 1) / BX) * ((n + 1 + BY - 1) / BY); }
+int cells_blocks(int n) {
+    const dim3 g = cells_grid(n);
+    return (int)(g.x * g.y);
+}
 
 bool pdl_enabled() {
     static const bool on = [] {
@@ -32,20 +36,10 @@ bool fuse_prolong_enabled() {
     return on;
 }
 
-__constant__ double c_W2d[2][9][5][5];
-__constant__ float c_W2f[2][9][5][5];
-
-template <typename T> __device__ __forceinline__ T W2(int o, int L, int fb, int fa);
-template <> __device__ __forceinline__ double W2<double>(int o, int L, int fb, int fa) { return c_W2d[o][L][fb][fa]; }
-template <> __device__ __forceinline__ float W2<float>(int o, int L, int fb, int fa) { return c_W2f[o][L][fb][fa]; }
-
-cudaError_t upload_transfer_weights(const double* P2) {
-    float tmp[2 * 9 * 25];
-    for (int i = 0; i < 2 * 9 * 25; ++i) tmp[i] = (float)P2[i];
-    cudaError_t e = cudaMemcpyToSymbol(c_W2d, P2, sizeof(double) * 2 * 9 * 25);
-    if (e != cudaSuccess) return e;
-    return cudaMemcpyToSymbol(c_W2f, tmp, sizeof(float) * 2 * 9 * 25);
-}
+// float64 kernels subtract the products from the right-hand side as they go (their time is the number of float64
+// instructions); the float32 ones keep the order of operations that defines the result of a float32 cycle
+template <typename T>
+constexpr bool kSubtract = sizeof(T) == 8;
 
 // ------------------------------------------------------------------------------------------
 // r = F - A x  (eq. gen:bil:mv), optional sum of squares.  PL: float32 arrays in the planar layout
@@ -64,45 +58,54 @@ __global__ void __launch_bounds__(NT) k_residual(int n, const __grid_constant__ 
     const int vld = PL ? pl_vpitch(n) : n + 1;
     double ss = 0.0;
     if (active) {
-        Acc<T> a;
-        if constexpr (PL) {
-            if (block_interior(n, 2))
-                cell_apply_auto<true, true, true, false, false>(i, j, n, c, gviewp<true>(u, n, 0), gviewp<true>(u, n, 1),
-                                                                gviewu(p, vld), a);
-            else
-                cell_apply_auto<true, true, true, false, true>(i, j, n, c, gviewp<false>(u, n, 0), gviewp<false>(u, n, 1),
-                                                               gview(p, vld), a);
-        } else {
-            if (block_interior(n, 2))
-                cell_apply_auto<true, true, true, false, false>(i, j, n, c, gviewu(u, 2 * n + 1),
-                                                                gviewu(u + n2, 2 * n + 1), gviewu(p, n + 1), a);
-            else
-                cell_apply_auto<true, true, true, false, true>(i, j, n, c, gview(u, 2 * n + 1), gview(u + n2, 2 * n + 1),
-                                                               gview(p, n + 1), a);
-        }
         const CellNodes cn = cell_nodes_dom(i, j, n, dom);
         const int ld = 2 * n + 1;
+        const size_t vi = (size_t)j * vld + i;
+        auto at = [&](int s) {   // index of node s, component 0, and the step to component 1
+            const int X = 2 * i + (s & 1), Y = 2 * j + (s >> 1);
+            return PL ? (size_t)pl_u(n, X, Y) : (size_t)Y * ld + X;
+        };
+        const size_t cs = PL ? 1 : n2;
+        Acc<T> a;
+        constexpr bool SUB = kSubtract<T>;
+        if constexpr (SUB) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const bool unk = slot_unknown(cn, s);
+                a.au[0][s] = unk ? f[at(s)] : T(0);
+                a.au[1][s] = unk ? f[at(s) + cs] : T(0);
+            }
+            a.bu = g[vi];
+        }
+        if constexpr (PL) {
+            if (block_interior(n, 2))
+                cell_apply_auto<true, true, true, false, false, SUB>(i, j, n, c, gviewp<true>(u, n, 0), gviewp<true>(u, n, 1),
+                                                                     gviewu(p, vld), a);
+            else
+                cell_apply_auto<true, true, true, false, true, SUB>(i, j, n, c, gviewp<false>(u, n, 0), gviewp<false>(u, n, 1),
+                                                                    gview(p, vld), a);
+        } else {
+            if (block_interior(n, 2))
+                cell_apply_auto<true, true, true, false, false, SUB>(i, j, n, c, gviewu(u, 2 * n + 1), gviewu(u + n2, 2 * n + 1),
+                                                                     gviewu(p, n + 1), a);
+            else
+                cell_apply_auto<true, true, true, false, true, SUB>(i, j, n, c, gview(u, 2 * n + 1), gview(u + n2, 2 * n + 1),
+                                                                    gview(p, n + 1), a);
+        }
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             if (!slot_exists(cn, s)) continue;
-            int X, Y;
-            slot_pos(i, j, s, X, Y);
-            const size_t idx = PL ? (size_t)pl_u(n, X, Y) : (size_t)Y * ld + X;
+            const bool unk = slot_unknown(cn, s);
 #pragma unroll
             for (int comp = 0; comp < 2; ++comp) {
-                const size_t k = PL ? idx + comp : comp * n2 + idx;
-                TO r = TO(0);
-                if (slot_unknown(cn, s)) {
-                    const T rr = f[k] - a.au[comp][s] - a.bt[comp][s];
-                    r = (TO)rr;
-                    ss += (double)rr * (double)rr;
-                }
-                ru[k] = r;
-                if (!PL && ru2) ru2[k] = (float)r;
+                const size_t k = at(s) + comp * cs;
+                const T rr = !unk ? T(0) : SUB ? a.au[comp][s] : f[k] - a.au[comp][s] - a.bt[comp][s];
+                ss += (double)rr * (double)rr;
+                ru[k] = (TO)rr;
+                if (!PL && ru2) ru2[k] = (float)rr;
             }
         }
-        const size_t vi = (size_t)j * vld + i;
-        const T r = (dom == kDomL && l_masked_vertex(i, j, n)) ? T(0) : g[vi] - a.bu;
+        const T r = (dom == kDomL && l_masked_vertex(i, j, n)) ? T(0) : SUB ? a.bu : g[vi] - a.bu;
         rp[vi] = (TO)r;
         if (!PL && rp2) rp2[vi] = (float)r;
         ss += (double)r * (double)r;
@@ -114,35 +117,45 @@ __global__ void __launch_bounds__(NT) k_residual(int n, const __grid_constant__ 
     pdl_trigger();
 }
 
-// float32: four CTAs per SM (64 registers; a few spilled) for more loads in flight
+// float32: four CTAs per SM (64 registers; a few spilled) for more loads in flight; float64: two (128), so that
+// the float64 pipes have work while other warps wait for their windows
 template <typename T>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) k_uzawa_u(int n, const __grid_constant__ OpCoef<T> c, T tau,
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 2) k_uzawa_u(int n, const __grid_constant__ OpCoef<T> c, T tau,
                                                 const T* __restrict__ u, const T* __restrict__ p,
                                                 const T* __restrict__ f, T* __restrict__ uh, int dom) {
     pdl_wait();
     CELL_INDEX
     if (!active) return;
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
-    Acc<T> a;
-    if (block_interior(n, 2))
-        cell_apply_auto<true, true, false, true, false>(i, j, n, c, gviewu(u, 2 * n + 1), gviewu(u + n2, 2 * n + 1),
-                                                        gviewu(p, n + 1), a);
-    else
-        cell_apply_auto<true, true, false, true, true>(i, j, n, c, gview(u, 2 * n + 1), gview(u + n2, 2 * n + 1),
-                                                       gview(p, n + 1), a);
     const CellNodes cn = cell_nodes_dom(i, j, n, dom);
     const int ld = 2 * n + 1;
+    Acc<T> a;
+    constexpr bool SUB = kSubtract<T>;
+    if constexpr (SUB) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const size_t k = (size_t)(2 * j + (s >> 1)) * ld + 2 * i + (s & 1);
+            const bool unk = slot_unknown(cn, s);
+            a.au[0][s] = unk ? f[k] : T(0);
+            a.au[1][s] = unk ? f[n2 + k] : T(0);
+        }
+    }
+    if (block_interior(n, 2))
+        cell_apply_auto<true, true, false, true, false, SUB>(i, j, n, c, gviewu(u, 2 * n + 1), gviewu(u + n2, 2 * n + 1),
+                                                             gviewu(p, n + 1), a);
+    else
+        cell_apply_auto<true, true, false, true, true, SUB>(i, j, n, c, gview(u, 2 * n + 1), gview(u + n2, 2 * n + 1),
+                                                            gview(p, n + 1), a);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
         if (!slot_exists(cn, s)) continue;
-        int X, Y;
-        slot_pos(i, j, s, X, Y);
-        const size_t idx = (size_t)Y * ld + X;
         const bool unk = slot_unknown(cn, s);
+        const T ti = tau * a.idg[s];
 #pragma unroll
         for (int comp = 0; comp < 2; ++comp) {
-            const size_t k = comp * n2 + idx;
-            uh[k] = unk ? u[k] + tau * (f[k] - a.au[comp][s] - a.bt[comp][s]) * a.idg[s] : T(0);
+            const size_t k = comp * n2 + (size_t)(2 * j + (s >> 1)) * ld + 2 * i + (s & 1);
+            if constexpr (SUB) uh[k] = unk ? fma(ti, a.au[comp][s], u[k]) : T(0);
+            else uh[k] = unk ? u[k] + tau * (f[k] - a.au[comp][s] - a.bt[comp][s]) * a.idg[s] : T(0);
         }
     }
     pdl_trigger();
@@ -157,16 +170,18 @@ __global__ void __launch_bounds__(NT) k_uzawa_p(int n, const __grid_constant__ O
     CELL_INDEX
     if (!active) return;
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
-    Acc<T> a;
-    if (block_interior(n, 1))
-        cell_apply_auto<false, false, true, false, false>(i, j, n, c, gviewu(uh, 2 * n + 1), gviewu(uh + n2, 2 * n + 1),
-                                                          gviewu((const T*)nullptr, n + 1), a);
-    else
-        cell_apply_auto<false, false, true, false, false>(i, j, n, c, gview(uh, 2 * n + 1), gview(uh + n2, 2 * n + 1),
-                                                          gview((const T*)nullptr, n + 1), a);
     const size_t vi = (size_t)j * (n + 1) + i;
+    Acc<T> a;
+    constexpr bool SUB = kSubtract<T>;
+    if constexpr (SUB) a.bu = g[vi];
+    if (block_interior(n, 1))
+        cell_apply_auto<false, false, true, false, false, SUB>(i, j, n, c, gviewu(uh, 2 * n + 1), gviewu(uh + n2, 2 * n + 1),
+                                                               gviewu((const T*)nullptr, n + 1), a);
+    else
+        cell_apply_auto<false, false, true, false, false, SUB>(i, j, n, c, gview(uh, 2 * n + 1), gview(uh + n2, 2 * n + 1),
+                                                               gview((const T*)nullptr, n + 1), a);
     // p^{m} = p^{m-1} - sigma Shat^{-1} (g - B u^{m-1/2})
-    const T d = sigma * sinv[vi] * (a.bu - g[vi]);
+    const T d = SUB ? -sigma * sinv[vi] * a.bu : sigma * sinv[vi] * (a.bu - g[vi]);
     p[vi] += d;
     dp[vi] = d;
     pdl_trigger();
@@ -196,11 +211,13 @@ __global__ void __launch_bounds__(NT) k_uzawa_u2(int n, const __grid_constant__ 
         slot_pos(i, j, s, X, Y);
         const size_t idx = (size_t)Y * ld + X;
         const bool unk = slot_unknown(cn, s);
+        const T ti = tau * a.idg[s];
 #pragma unroll
         for (int comp = 0; comp < 2; ++comp) {
             const size_t k = comp * n2 + idx;
-            // u^{m} = u^{m-1/2} - tau Ahat^{-1} B^T (p^{m} - p^{m-1})
-            u[k] = unk ? uh[k] - tau * a.bt[comp][s] * a.idg[s] : T(0);
+            // u^{m} = u^{m-1/2} - tau Ahat^{-1} B^T (p^{m} - p^{m-1}); the V rows of B^T are zero
+            if constexpr (kSubtract<T>) u[k] = !unk ? T(0) : s == 0 ? uh[k] : fma(-ti, a.bt[comp][s], uh[k]);
+            else u[k] = unk ? uh[k] - tau * a.bt[comp][s] * a.idg[s] : T(0);
         }
     }
     pdl_trigger();
@@ -209,7 +226,8 @@ __global__ void __launch_bounds__(NT) k_uzawa_u2(int n, const __grid_constant__ 
 template <typename T>
 void launch_uzawa(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T sigma, T* u, T* p, const T* f,
                   const T* g, const T* sinv, T* uh, T* dp, int bx, int by, int dom) {
-    const dim3 blk(bx, by), grid((n + 1 + bx - 1) / bx, (n + 1 + by - 1) / by);
+    const dim3 blk = bx > 0 ? dim3(bx, by) : cells_block(n);
+    const dim3 grid((n + 1 + blk.x - 1) / blk.x, (n + 1 + blk.y - 1) / blk.y);
     launch_pdl(k_uzawa_u<T>, grid, blk, 0, s, n, c, tau, u, p, f, uh, dom);
     // dp = 0 where Shat^{-1} = 0: on the L the vertices outside it
     launch_pdl(k_uzawa_p<T>, grid, blk, 0, s, n, c, sigma, uh, p, g, sinv, dp);
@@ -275,7 +293,7 @@ __global__ void __launch_bounds__(NT) k_normal_update(int n, const __grid_consta
 template <typename T>
 void launch_normal_eq(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T* u, T* p, const T* f,
                       const T* g, const T* sinv, T* zu, T* zp) {
-    const dim3 grid = cells_grid(n), blk(BX, BY);
+    const dim3 grid = cells_grid(n), blk = cells_block(n);
     launch_pdl(k_residual<T, T, false>, grid, blk, 0, s, n, c, u, p, f, g, zu, zp, nullptr, nullptr, nullptr,
                (int)kDomSquare);
     launch_pdl(k_scale_L<T>, grid, blk, 0, s, n, c, zu, zp, sinv);
@@ -285,13 +303,13 @@ void launch_normal_eq(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T* u, T*
 template <typename T, typename TO>
 void launch_residual(cudaStream_t s, int n, const OpCoef<T>& c, const T* u, const T* p, const T* f,
                      const T* g, TO* ru, TO* rp, double* partial, float* ru2, float* rp2, int dom) {
-    launch_pdl(k_residual<T, TO, false>, cells_grid(n), dim3(BX, BY), 0, s, n, c, u, p, f, g, ru, rp, partial, ru2, rp2,
+    launch_pdl(k_residual<T, TO, false>, cells_grid(n), cells_block(n), 0, s, n, c, u, p, f, g, ru, rp, partial, ru2, rp2,
                dom);
 }
 
 void launch_residual_planar(cudaStream_t s, int n, const OpCoef<float>& c, const float* u, const float* p,
                             const float* f, const float* g, float* ru, float* rp) {
-    launch_pdl(k_residual<float, float, true>, cells_grid(n), dim3(BX, BY), 0, s, n, c, u, p, f, g, ru, rp,
+    launch_pdl(k_residual<float, float, true>, cells_grid(n), cells_block(n), 0, s, n, c, u, p, f, g, ru, rp,
                (double*)nullptr, (float*)nullptr, (float*)nullptr, (int)kDomSquare);
 }
 
@@ -300,24 +318,32 @@ void launch_residual_planar(cudaStream_t s, int n, const OpCoef<float>& c, const
 // Every fine point is owned by one coarse square (local fine offsets 0..3 in each direction);
 // points on the far edges belong to the neighbouring square, where the weights of the nodes not
 // shared with it vanish, so the sum over the 1-4 squares of a coarse node's patch is exact.
-template <int O, int SQ, int R, typename T>
-__device__ __forceinline__ void restrict_rows(const T (&v)[2][4][4], T (&acc)[2][4]) {
+template <int O, int SQ, int R, int P, typename T>
+__device__ __forceinline__ void restrict_term(const T (&v)[2][4][4], T (&acc)[2][4]) {
+    constexpr int L = sq_row(SQ, R), s = sq_slot(SQ, R), fa = P % 4, fb = P / 4;
+    constexpr T w = (T)embed_weight(O, L, fa, fb);
+    if constexpr (w != T(0)) {
+        acc[0][s] = fma(w, v[0][fb][fa], acc[0][s]);
+        acc[1][s] = fma(w, v[1][fb][fa], acc[1][s]);
+    }
+}
+template <int O, int SQ, int R, typename T, int... P>
+__device__ __forceinline__ void restrict_rows(const T (&v)[2][4][4], T (&acc)[2][4], std::integer_sequence<int, P...> pts) {
     if constexpr (R < sq_nrows(SQ)) {
-        constexpr int L = sq_row(SQ, R), s = sq_slot(SQ, R);
-#pragma unroll
-        for (int fb = 0; fb < 4; ++fb)
-#pragma unroll
-            for (int fa = 0; fa < 4; ++fa) {
-                const T w = W2<T>(O, L, fb, fa);
-                acc[0][s] = fma(w, v[0][fb][fa], acc[0][s]);
-                acc[1][s] = fma(w, v[1][fb][fa], acc[1][s]);
-            }
-        restrict_rows<O, SQ, R + 1>(v, acc);
+        (restrict_term<O, SQ, R, P>(v, acc), ...);
+        restrict_rows<O, SQ, R + 1>(v, acc, pts);
     }
 }
 
+// global arrays go through the read-only path; shared-memory arrays (the coarse sub-cycle) do not
+template <bool LDG, typename T>
+__device__ __forceinline__ T ldv(const T* p) {
+    if constexpr (LDG) return __ldg(p);
+    else return *p;
+}
+
 // Strides of the arrays a transfer reads and writes, each pointer at the array's (0, 0) entry: the dense
-// level arrays (dense_layout), or float32 levels in the planar layout (template flags PF / PC of the
+// level arrays (dense_layout), the padded shared-memory arrays of the coarse cycle, or float32 levels in the planar layout (template flags PF / PC of the
 // fine / coarse level; there the row stride is in floats, the component stride is 1 and psf / psc is the
 // parity-plane stride).
 struct XferLayout {
@@ -355,7 +381,7 @@ __host__ __device__ __forceinline__ int lat_at(int X, int Y, int ld, int ps) {
     else return Y * ld + X;
 }
 
-template <int SQ, bool PF, typename T>
+template <int SQ, bool LDG, bool PF, typename T>
 __device__ __forceinline__ void restrict_visit(int I, int J, int nc, const T* __restrict__ ru, T (&acc)[2][4],
                                                const XferLayout& lay) {
     const int SI = I - (SQ & 1), SJ = J - (SQ >> 1);
@@ -366,25 +392,26 @@ __device__ __forceinline__ void restrict_visit(int I, int J, int nc, const T* __
 #pragma unroll
         for (int fa = 0; fa < 4; ++fa) {
             const int k = lat_at<PF>(4 * SI + fa, 4 * SJ + fb, lay.ldf, lay.psf);
-            v[0][fb][fa] = __ldg(ru + k);
-            v[1][fb][fa] = __ldg(ru + lay.n2f + k);
+            v[0][fb][fa] = ldv<LDG>(ru + k);
+            v[1][fb][fa] = ldv<LDG>(ru + lay.n2f + k);
         }
-    if (orient(SI, SJ, nc)) restrict_rows<1, SQ, 0>(v, acc);
-    else restrict_rows<0, SQ, 0>(v, acc);
+    constexpr auto P16 = std::make_integer_sequence<int, 16>{};
+    if (orient(SI, SJ, nc)) restrict_rows<1, SQ, 0>(v, acc, P16);
+    else restrict_rows<0, SQ, 0>(v, acc, P16);
 }
 
 // coarse cell (i, j) of level nc: its owned coarse velocity nodes and vertex
-template <typename T, bool PF, bool PC>
+template <bool LDG, typename T, bool PF, bool PC>
 __device__ __forceinline__ void restrict_cell(int i, int j, int nc, const T* __restrict__ ru, const T* __restrict__ rp,
                                               T* __restrict__ fc, T* __restrict__ gc, const XferLayout& lay,
                                               int dom = kDomSquare) {
     T acc[2][4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) acc[0][s] = acc[1][s] = T(0);
-    restrict_visit<0, PF>(i, j, nc, ru, acc, lay);
-    restrict_visit<1, PF>(i, j, nc, ru, acc, lay);
-    restrict_visit<2, PF>(i, j, nc, ru, acc, lay);
-    restrict_visit<3, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<0, LDG, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<1, LDG, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<2, LDG, PF>(i, j, nc, ru, acc, lay);
+    restrict_visit<3, LDG, PF>(i, j, nc, ru, acc, lay);
     const CellNodes cn = cell_nodes_dom(i, j, nc, dom);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -427,7 +454,7 @@ __global__ void __launch_bounds__(NT) k_restrict(int nc, const T* __restrict__ r
     CELL_INDEX
     if (!active) return;
     const XferLayout lay = xfer_layout(nc, PF, PC);
-    restrict_cell<T, PF, PC>(i, j, nc, ru, rp, fc, gc, lay, dom);
+    restrict_cell<true, T, PF, PC>(i, j, nc, ru, rp, fc, gc, lay, dom);
     if (uc) {
         const CellNodes cn = cell_nodes(i, j, nc);
 #pragma unroll
@@ -446,23 +473,53 @@ __global__ void __launch_bounds__(NT) k_restrict(int nc, const T* __restrict__ r
 
 template <typename T>
 void launch_restrict(cudaStream_t s, int nc, const T* ru, const T* rp, T* fc, T* gc, T* uc, T* pc, int dom) {
-    launch_pdl(k_restrict<T, false, false>, cells_grid(nc), dim3(BX, BY), 0, s, nc, ru, rp, fc, gc, uc, pc, dom);
+    launch_pdl(k_restrict<T, false, false>, cells_grid(nc), cells_block(nc), 0, s, nc, ru, rp, fc, gc, uc, pc, dom);
 }
 
 void launch_restrict_planar(cudaStream_t s, int nc, bool pc_planar, const float* ru, const float* rp, float* fc,
                             float* gc, float* uc, float* pc) {
     if (pc_planar)
-        launch_pdl(k_restrict<float, true, true>, cells_grid(nc), dim3(BX, BY), 0, s, nc, ru, rp, fc, gc, uc, pc,
+        launch_pdl(k_restrict<float, true, true>, cells_grid(nc), cells_block(nc), 0, s, nc, ru, rp, fc, gc, uc, pc,
                    (int)kDomSquare);
     else
-        launch_pdl(k_restrict<float, true, false>, cells_grid(nc), dim3(BX, BY), 0, s, nc, ru, rp, fc, gc, uc, pc,
+        launch_pdl(k_restrict<float, true, false>, cells_grid(nc), cells_block(nc), 0, s, nc, ru, rp, fc, gc, uc, pc,
                    (int)kDomSquare);
+}
+
+// u += the coarse P2 function with values z on the coarse square (i, j) at its fine point P = 4 fb + fa
+template <int O, int P, typename T, bool PF, int... L>
+__device__ __forceinline__ void prolong_point(int i, int j, int nf, const T (&z)[2][9], T* __restrict__ u, const XferLayout& lay,
+                                              int dom, std::integer_sequence<int, L...>) {
+    constexpr int fa = P % 4, fb = P / 4;
+    const int X = 4 * i + fa, Y = 4 * j + fb;
+    if (!interior2(X, Y, nf) || (dom == kDomL && l_masked_node(X, Y, nf))) return;
+    const int k = lat_at<PF>(X, Y, lay.ldf, lay.psf);
+    // float64: on top of u (two additions fewer); float32: the sum first
+    constexpr bool onto = sizeof(T) == 8;
+    const T ox = u[k], oy = u[lay.n2f + k];
+    T sx = onto ? ox : T(0), sy = onto ? oy : T(0);
+    auto term = [&](auto ll) {
+        constexpr int l = decltype(ll)::value;
+        constexpr T w = (T)embed_weight(O, l, fa, fb);
+        if constexpr (w != T(0)) {
+            sx = fma(w, z[0][l], sx);
+            sy = fma(w, z[1][l], sy);
+        }
+    };
+    (term(std::integral_constant<int, L>{}), ...);
+    u[k] = onto ? sx : ox + sx;
+    u[lay.n2f + k] = onto ? sy : oy + sy;
+}
+template <int O, typename T, bool PF, int... P>
+__device__ __forceinline__ void prolong_square(int i, int j, int nf, const T (&z)[2][9], T* __restrict__ u, const XferLayout& lay,
+                                               int dom, std::integer_sequence<int, P...>) {
+    (prolong_point<O, P, T, PF>(i, j, nf, z, u, lay, dom, std::make_integer_sequence<int, 9>{}), ...);
 }
 
 // Prolongation (Sec. 3, canonical embedding): every fine point owned by coarse square (I, J) is
 // the coarse P2 function of that square evaluated there; P1 values are vertex injection and
 // averages along coarse edges.
-template <typename T, bool PF, bool PC>
+template <bool LDG, typename T, bool PF, bool PC>
 __device__ __forceinline__ void prolong_cell(int i, int j, int nc, const T* __restrict__ uc, const T* __restrict__ pc,
                                              T* __restrict__ u, T* __restrict__ p, const XferLayout& lay,
                                              int dom = kDomSquare) {
@@ -472,30 +529,15 @@ __device__ __forceinline__ void prolong_cell(int i, int j, int nc, const T* __re
 #pragma unroll
         for (int m = 0; m < 9; ++m) {
             const int k = lat_at<PC>(2 * i + m % 3, 2 * j + m / 3, lay.ldc, lay.psc);
-            z[0][m] = __ldg(uc + k);
-            z[1][m] = __ldg(uc + lay.n2c + k);
+            z[0][m] = ldv<LDG>(uc + k);
+            z[1][m] = ldv<LDG>(uc + lay.n2c + k);
         }
-        const int o = orient(i, j, nc);
-#pragma unroll
-        for (int fb = 0; fb < 4; ++fb)
-#pragma unroll
-            for (int fa = 0; fa < 4; ++fa) {
-                const int X = 4 * i + fa, Y = 4 * j + fb;
-                if (!interior2(X, Y, nf) || (dom == kDomL && l_masked_node(X, Y, nf))) continue;
-                T sx = T(0), sy = T(0);
-#pragma unroll
-                for (int L = 0; L < 9; ++L) {
-                    const T w = W2<T>(o, L, fb, fa);
-                    sx = fma(w, z[0][L], sx);
-                    sy = fma(w, z[1][L], sy);
-                }
-                const int k = lat_at<PF>(X, Y, lay.ldf, lay.psf);
-                u[k] += sx;
-                u[lay.n2f + k] += sy;
-            }
+        constexpr auto P16 = std::make_integer_sequence<int, 16>{};
+        if (orient(i, j, nc)) prolong_square<1, T, PF>(i, j, nf, z, u, lay, dom, P16);
+        else prolong_square<0, T, PF>(i, j, nf, z, u, lay, dom, P16);
     }
     const int ldp = lay.ldpc, ldpf = lay.ldpf;
-    auto P = [&](int a, int b) { return __ldg(pc + (b * ldp + a)); };
+    auto P = [&](int a, int b) { return ldv<LDG>(pc + (b * ldp + a)); };
     const T p00 = P(i, j);
     // on the L, fine vertices strictly inside the removed quadrant keep their zero
     auto live = [&](int x, int y) { return !(dom == kDomL && l_masked_vertex(x, y, nf)); };
@@ -515,21 +557,21 @@ __global__ void __launch_bounds__(NT) k_prolong(int nc, const T* __restrict__ uc
     const int n = nc;
     CELL_INDEX
     if (!active) return;
-    prolong_cell<T, PF, PC>(i, j, nc, uc, pc, u, p, xfer_layout(nc, PF, PC), dom);
+    prolong_cell<true, T, PF, PC>(i, j, nc, uc, pc, u, p, xfer_layout(nc, PF, PC), dom);
     pdl_trigger();
 }
 
 template <typename T>
 void launch_prolong_add(cudaStream_t s, int nc, const T* uc, const T* pc, T* u, T* p, int dom) {
-    launch_pdl(k_prolong<T, false, false>, cells_grid(nc), dim3(BX, BY), 0, s, nc, uc, pc, u, p, dom);
+    launch_pdl(k_prolong<T, false, false>, cells_grid(nc), cells_block(nc), 0, s, nc, uc, pc, u, p, dom);
 }
 
 void launch_prolong_add_planar(cudaStream_t s, int nc, bool pc_planar, const float* uc, const float* pc, float* u,
                                float* p) {
     if (pc_planar)
-        launch_pdl(k_prolong<float, true, true>, cells_grid(nc), dim3(BX, BY), 0, s, nc, uc, pc, u, p, (int)kDomSquare);
+        launch_pdl(k_prolong<float, true, true>, cells_grid(nc), cells_block(nc), 0, s, nc, uc, pc, u, p, (int)kDomSquare);
     else
-        launch_pdl(k_prolong<float, true, false>, cells_grid(nc), dim3(BX, BY), 0, s, nc, uc, pc, u, p, (int)kDomSquare);
+        launch_pdl(k_prolong<float, true, false>, cells_grid(nc), cells_block(nc), 0, s, nc, uc, pc, u, p, (int)kDomSquare);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -631,20 +673,21 @@ __global__ void __launch_bounds__(NT) k_schur(int n, const __grid_constant__ OpC
 
 template <typename T>
 void launch_schur_diag(cudaStream_t s, int n, const OpCoef<double>& c, T* sinv, int dom, int vld) {
-    k_schur<T><<<cells_grid(n), dim3(BX, BY), 0, s>>>(n, c, sinv, dom, vld > 0 ? vld : n + 1);
+    k_schur<T><<<cells_grid(n), cells_block(n), 0, s>>>(n, c, sinv, dom, vld > 0 ? vld : n + 1);
 }
 
 // ------------------------------------------------------------------------------------------
 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_pmean_partial(int n, const T* __restrict__ p, double* __restrict__ partial,
-                                                      int dom) {
+                                                      double wscale, int dom) {
     pdl_wait();
     CELL_INDEX
+    // w_i = (triangles at vertex i) h^2 / 6: counted per vertex, scaled per block
     double v = 0.0;
-    if (active) v = vertex_weight_dom(i, j, n, dom) * (double)p[(size_t)j * (n + 1) + i];
+    if (active) v = (double)vertex_triangles_dom(i, j, n, dom) * (double)p[(size_t)j * (n + 1) + i];
     const double t = block_sum2d(v, tid);
-    if (tid == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = t;
+    if (tid == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = t * wscale;
     pdl_trigger();
 }
 
@@ -684,25 +727,59 @@ cudaError_t launch_reduce(cudaStream_t s, const double* partial, int count, doub
 
 template <typename T>
 void launch_pmean(cudaStream_t s, int n, T* p, double* partial, double* scalar, int dom) {
-    const dim3 grid = cells_grid(n), blk(BX, BY);
-    launch_pdl(k_pmean_partial<T>, grid, blk, 0, s, n, p, partial, dom);
+    const dim3 grid = cells_grid(n), blk = cells_block(n);
+    launch_pdl(k_pmean_partial<T>, grid, blk, 0, s, n, p, partial, 1.0 / (6.0 * (double)n * (double)n), dom);
     launch_pdl(k_reduce, 1, 1024, 0, s, partial, grid.x * grid.y, scalar);
     launch_pdl(k_psub<T>, grid, blk, 0, s, n, p, scalar, dom);
 }
 
 template <typename T>
 void launch_psub(cudaStream_t s, int n, T* p, const double* scalar, int dom) {
-    launch_pdl(k_psub<T>, cells_grid(n), dim3(BX, BY), 0, s, n, p, scalar, dom);
+    launch_pdl(k_psub<T>, cells_grid(n), cells_block(n), 0, s, n, p, scalar, dom);
 }
 template void launch_psub<double>(cudaStream_t, int, double*, const double*, int);
 
 // ------------------------------------------------------------------------------------------
 // load vectors (data f, g of Sec. 1 given by nodal values)
+// a.au = M_U v at the cell's nodes (the merged rows of class C; points off the lattice read as zero)
+// (MASK: and so do the boundary nodes)
+template <int C, bool MASK, typename T>
+__device__ __forceinline__ void mass_rows(int i, int j, int n, const MassCoef<T>& m, const T* __restrict__ v, Acc<T>& a) {
+    constexpr auto K25 = std::make_integer_sequence<int, 25>{};
+    const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
+    T wx[25], wy[25];
+    win_load<C, true, false, MASK>(i, j, n, gview(v, 2 * n + 1), gview(v + n2, 2 * n + 1), wx, wy, K25);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) a.au[0][s] = a.au[1][s] = T(0);
+    ma_row<false, C, 0>(m.MM, wx, wy, a.au[0][0], a.au[1][0], K25);
+    ma_row<false, C, 1>(m.MM, wx, wy, a.au[0][1], a.au[1][1], K25);
+    ma_row<false, C, 2>(m.MM, wx, wy, a.au[0][2], a.au[1][2], K25);
+    ma_row<false, C, 3>(m.MM, wx, wy, a.au[0][3], a.au[1][3], K25);
+}
+template <bool MASK, typename T>
+__device__ __forceinline__ void mass_rows_auto(int i, int j, int n, const MassCoef<T>& m, const T* __restrict__ v, Acc<T>& a) {
+    switch (stencil_class(i, j, n)) {
+        case 0: mass_rows<0, MASK>(i, j, n, m, v, a); break;
+        case 1: mass_rows<1, MASK>(i, j, n, m, v, a); break;
+        case 2: mass_rows<2, MASK>(i, j, n, m, v, a); break;
+        case 3: mass_rows<3, MASK>(i, j, n, m, v, a); break;
+        case 4: mass_rows<4, MASK>(i, j, n, m, v, a); break;
+        case 5: mass_rows<5, MASK>(i, j, n, m, v, a); break;
+        default: mass_rows<6, MASK>(i, j, n, m, v, a); break;
+    }
+}
 template <typename T>
 __device__ __forceinline__ void mp_row(int i, int j, int n, const MassCoef<T>& m, const T* __restrict__ gn,
                                        T& mg, double& w) {
     mg = T(0);
     w = 0.0;
+    if (i > 0 && j > 0 && i < n && j < n) {   // all four squares: the merged row of the vertex's class
+        const int k = stencil_class(i, j, n);
+#pragma unroll
+        for (int v = 0; v < 9; ++v) mg = fma(m.MMP[k][v], gn[(size_t)(j + v / 3 - 1) * (n + 1) + i + v % 3 - 1], mg);
+        w = (double)m.MW[k];
+        return;
+    }
 #pragma unroll
     for (int SQ = 0; SQ < 4; ++SQ) {
         const int si = i - (SQ & 1), sj = j - (SQ >> 1);
@@ -719,15 +796,14 @@ __device__ __forceinline__ void mp_row(int i, int j, int n, const MassCoef<T>& m
 }
 
 template <typename T>
-__global__ void __launch_bounds__(NT) k_load(int n, const __grid_constant__ MassCoef<T> m, const __grid_constant__ OpCoef<T> c,
-                                             const T* __restrict__ fn, const T* __restrict__ gn,
-                                             T* __restrict__ f, T* __restrict__ g, double* __restrict__ partial) {
+__global__ void __launch_bounds__(NT) k_load(int n, const __grid_constant__ MassCoef<T> m, const T* __restrict__ fn,
+                                             const T* __restrict__ gn, T* __restrict__ f, T* __restrict__ g, double* __restrict__ partial) {
     CELL_INDEX
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
     double wg = 0.0;
     if (active) {
         Acc<T> a;
-        cell_apply<true, false, false, false, false>(i, j, n, m.M, c, gview(fn, 2 * n + 1), gview(fn + n2, 2 * n + 1), gview((const T*)nullptr, n + 1), a);
+        mass_rows_auto<false>(i, j, n, m, fn, a);   // boundary values included
         const CellNodes cn = cell_nodes(i, j, n);
         const int ld = 2 * n + 1;
 #pragma unroll
@@ -757,13 +833,17 @@ __global__ void __launch_bounds__(NT) k_gproj(int n, const __grid_constant__ Mas
     CELL_INDEX
     if (!active) return;
     double w = 0.0;
+    if (i > 0 && j > 0 && i < n && j < n) {
+        w = (double)m.MW[stencil_class(i, j, n)];
+    } else {
 #pragma unroll
-    for (int SQ = 0; SQ < 4; ++SQ) {
-        const int si = i - (SQ & 1), sj = j - (SQ >> 1);
-        if (si < 0 || sj < 0 || si >= n || sj >= n) continue;
-        const int o = orient(si, sj, n);
+        for (int SQ = 0; SQ < 4; ++SQ) {
+            const int si = i - (SQ & 1), sj = j - (SQ >> 1);
+            if (si < 0 || sj < 0 || si >= n || sj >= n) continue;
+            const int o = orient(si, sj, n);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) w += (double)m.MP[o][SQ][r];
+            for (int r = 0; r < 4; ++r) w += (double)m.MP[o][SQ][r];
+        }
     }
     // M_P (g - c 1) = M_P g - c w,  c = int g_h = sum_i w_i g_i
     g[(size_t)j * (n + 1) + i] -= (T)(w * (*scalar));
@@ -772,9 +852,8 @@ __global__ void __launch_bounds__(NT) k_gproj(int n, const __grid_constant__ Mas
 template <typename T>
 void launch_load(cudaStream_t s, int n, const MassCoef<T>& m, const T* fn, const T* gn, T* f, T* g,
                  int project_g, double* partial, double* scalar) {
-    const dim3 grid = cells_grid(n), blk(BX, BY);
-    OpCoef<T> dummy{};
-    k_load<T><<<grid, blk, 0, s>>>(n, m, dummy, fn, gn, f, g, partial);
+    const dim3 grid = cells_grid(n), blk = cells_block(n);
+    k_load<T><<<grid, blk, 0, s>>>(n, m, fn, gn, f, g, partial);
     if (project_g) {
         launch_pdl(k_reduce, 1, 1024, 0, s, partial, grid.x * grid.y, scalar);
         k_gproj<T><<<grid, blk, 0, s>>>(n, m, g, scalar);
@@ -782,7 +861,6 @@ void launch_load(cudaStream_t s, int n, const MassCoef<T>& m, const T* fn, const
 }
 
 __global__ void __launch_bounds__(NT) k_mass_dot(int n, const __grid_constant__ MassCoef<double> m,
-                                                 const __grid_constant__ OpCoef<double> c,
                                                  const double* __restrict__ av, const double* __restrict__ bv,
                                                  double* __restrict__ partial) {
     CELL_INDEX
@@ -790,7 +868,7 @@ __global__ void __launch_bounds__(NT) k_mass_dot(int n, const __grid_constant__ 
     double acc = 0.0;
     if (active) {
         Acc<double> a;
-        cell_apply<true, false, false, false, true>(i, j, n, m.M, c, gview(bv, 2 * n + 1), gview(bv + n2, 2 * n + 1), gview((const double*)nullptr, n + 1), a);
+        mass_rows_auto<true>(i, j, n, m, bv, a);
         const CellNodes cn = cell_nodes(i, j, n);
         const int ld = 2 * n + 1;
 #pragma unroll
@@ -808,8 +886,7 @@ __global__ void __launch_bounds__(NT) k_mass_dot(int n, const __grid_constant__ 
 
 void launch_mass_dot(cudaStream_t s, int n, const MassCoef<double>& m, const double* a, const double* b,
                      double* partial) {
-    OpCoef<double> dummy{};
-    k_mass_dot<<<cells_grid(n), dim3(BX, BY), 0, s>>>(n, m, dummy, a, b, partial);
+    k_mass_dot<<<cells_grid(n), cells_block(n), 0, s>>>(n, m, a, b, partial);
 }
 
 __global__ void __launch_bounds__(NT) k_rhs_norm(int n, const double* __restrict__ f, const double* __restrict__ g,
@@ -836,7 +913,7 @@ __global__ void __launch_bounds__(NT) k_rhs_norm(int n, const double* __restrict
 }
 
 void launch_rhs_norm(cudaStream_t s, int n, const double* f, const double* g, double* partial) {
-    k_rhs_norm<<<cells_grid(n), dim3(BX, BY), 0, s>>>(n, f, g, partial);
+    k_rhs_norm<<<cells_grid(n), cells_block(n), 0, s>>>(n, f, g, partial);
 }
 
 __global__ void __launch_bounds__(NT) k_sum_partial(int n, const double* __restrict__ g, double* __restrict__ partial) {
@@ -853,7 +930,7 @@ __global__ void __launch_bounds__(NT) k_sub_w(int n, double* __restrict__ g, con
 }
 
 void launch_make_consistent(cudaStream_t s, int n, double* g, double* partial, double* scalar) {
-    const dim3 grid = cells_grid(n), blk(BX, BY);
+    const dim3 grid = cells_grid(n), blk = cells_block(n);
     k_sum_partial<<<grid, blk, 0, s>>>(n, g, partial);
     launch_pdl(k_reduce, 1, 1024, 0, s, partial, grid.x * grid.y, scalar);
     k_sub_w<<<grid, blk, 0, s>>>(n, g, scalar);
@@ -932,6 +1009,8 @@ void launch_mask_l(cudaStream_t s, int n, double* u, double* p) {
     const int blocks = std::min((ld * ld + 255) / 256, 4096);
     k_mask_l<<<blocks, 256, 0, s>>>(n, u, p);
 }
+
+#include "coarse_cycle.cuh"
 
 // ------------------------------------------------------------------------------------------
 #define INST(T)                                                                                         \

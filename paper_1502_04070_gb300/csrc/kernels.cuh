@@ -11,9 +11,6 @@ namespace smg {
 // cells_blocks(n).
 int cells_blocks(int n);
 
-// Transfer weight table (constant memory), set once per device.
-cudaError_t upload_transfer_weights(const double* P2 /* [2][9][5][5] */);
-
 // r = F - A x with per-block partial sums of r.r (over unknowns) in `partial` (may be null) and an
 // optional float32 copy of r in (ru2, rp2).
 // dom: kDomSquare or kDomL (common.cuh: on the L, the nodes outside it are not unknowns)
@@ -29,7 +26,7 @@ void launch_residual(cudaStream_t s, int n, const OpCoef<T>& c, const T* u, cons
 //   u  = uh - tau Ahat^{-1} B^T dp
 template <typename T>
 void launch_uzawa(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T sigma, T* u, T* p, const T* f,
-                  const T* g, const T* sinv, T* uh, T* dp, int bx = 32, int by = 8, int dom = kDomSquare);
+                  const T* g, const T* sinv, T* uh, T* dp, int bx = 0, int by = 0, int dom = kDomSquare);   // bx 0: cells_block(n)
 
 // Refinement update (see refine.cu): float32 correction e, float64 iterate x, residual r stored as
 // (hi, lo) float pairs in the 8-byte slots of a float64 array:
@@ -90,8 +87,9 @@ struct alignas(16) MidLists {
     E2<float> BT[kStencilClasses][kListBT], B[kStencilClasses][kListB], BU[kStencilClasses][kListB];
     float ti[kStencilClasses][4];        // tau / diag A
 };
-// what the kernels of a planar level take beside its arrays and operator: its lists (device), and whether
-// other solves share the GPU (a batch), which favours tall tiles
+// what the kernels of a planar level take beside its arrays and operator: its lists (device; null: tiles on the
+// mid-lines run the per-cell rows and the tile heights balance the SMs alone, the arithmetic of stokes_cycle), and
+// whether other solves share the GPU (a batch), which favours tall tiles
 struct PlanarLevel {
     const MidLists* lists = nullptr;
     bool shared = false;
@@ -244,6 +242,27 @@ void launch_rhs_norm(cudaStream_t s, int n, const double* f, const double* g, do
 // g <- g - (1^T g) w  with w = M_P 1: the pressure right-hand side becomes orthogonal to the
 // constant pressure (the kernel of the saddle-point matrix)
 void launch_make_consistent(cudaStream_t s, int n, double* g, double* partial, double* scalar);
+
+// The float32 V-cycle of levels 0..a.top (top <= 4) in one CTA with shared-memory arrays
+// (coarse_cycle.cuh); the kernel's shared-memory limit is raised by prepare_coarse_cycle().
+constexpr int kCoarseCycleTop = 4;
+struct CoarseCycleArgs {
+    OpCoef<float> c[kCoarseCycleTop];     // levels 1..top at index l - 1
+    const float* sinv[kCoarseCycleTop];   // Shat^{-1} of levels 1..top (global)
+    const double* inv;                    // level-0 bordered inverse (27 x 27, global)
+    float* u;                             // iterate of level `top` (global; read at start, written at end)
+    float* p;
+    const float* f;                       // right-hand side of level `top` (global)
+    const float* g;
+    float tau, sigma;
+    int nu_pre, nu_post;
+    int top;                              // 1 <= top <= kCoarseCycleTop
+};
+// kernel parameters are limited to 32,764 bytes
+static_assert(sizeof(CoarseCycleArgs) <= 32764, "coarse-cycle parameters exceed the launch limit");
+
+cudaError_t prepare_coarse_cycle();
+void launch_coarse_cycle(cudaStream_t s, const CoarseCycleArgs& a);
 
 // batched solver: device-side WHILE condition and result store (batch.cu)
 void launch_batch_check(cudaStream_t s, cudaGraphConditionalHandle hnd, const double* scal, double tol2,

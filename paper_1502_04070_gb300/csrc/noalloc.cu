@@ -91,7 +91,7 @@ extern "C" stokes_status stokes_residual_norm2_noalloc(int levels, double beta, 
     // work left pending in the runtime is neither blamed on this call nor cleared by it
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = cells_grid(n);
-    cfg.blockDim = dim3(BX, BY);
+    cfg.blockDim = cells_block(n);
     cfg.stream = s;
     if (cudaLaunchKernelEx(&cfg, k_residual_sumsq, n, c, u, p, f, g, scratch) != cudaSuccess) return STOKES_ERR_CUDA;
     if (launch_reduce(s, scratch, cells_blocks(n), norm2) != cudaSuccess) return STOKES_ERR_CUDA;

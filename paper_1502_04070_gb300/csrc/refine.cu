@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(NT, 4) k_ir_update_df(int n, const __grid_cons
 // true float64 residual r = F - A x (x, F float64), written as two-float r and float32 r32 (PL: r32
 // in the planar layout)
 template <bool PL>
-__global__ void __launch_bounds__(NT) k_residual_df(int n, const __grid_constant__ OpCoef<double> c,
+__global__ void __launch_bounds__(NT, 2) k_residual_df(int n, const __grid_constant__ OpCoef<double> c,
                                                     const double* __restrict__ u, const double* __restrict__ p,
                                                     const double* __restrict__ f, const double* __restrict__ g,
                                                     float2* __restrict__ ru, float2* __restrict__ rp,
@@ -350,11 +350,23 @@ __global__ void __launch_bounds__(NT) k_residual_df(int n, const __grid_constant
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
     double ss = 0.0;
     if (active) {
-        Acc<double> a;
-        cell_apply_auto<true, true, true, false, true>(i, j, n, c, gview(u, 2 * n + 1), gview(u + n2, 2 * n + 1),
-                                                  gview(p, n + 1), a);
         const CellNodes cn = cell_nodes_dom(i, j, n, dom);
         const int ld = 2 * n + 1;
+        Acc<double> a;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const size_t k = (size_t)(2 * j + (s >> 1)) * ld + 2 * i + (s & 1);
+            const bool unk = slot_unknown(cn, s);
+            a.au[0][s] = unk ? f[k] : 0.0;
+            a.au[1][s] = unk ? f[n2 + k] : 0.0;
+        }
+        a.bu = g[(size_t)j * (n + 1) + i];
+        if (block_interior(n, 2))
+            cell_apply_auto<true, true, true, false, false, true>(i, j, n, c, gviewu(u, 2 * n + 1), gviewu(u + n2, 2 * n + 1),
+                                                                  gviewu(p, n + 1), a);
+        else
+            cell_apply_auto<true, true, true, false, true, true>(i, j, n, c, gview(u, 2 * n + 1), gview(u + n2, 2 * n + 1),
+                                                                 gview(p, n + 1), a);
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             if (!slot_exists(cn, s)) continue;
@@ -365,16 +377,15 @@ __global__ void __launch_bounds__(NT) k_residual_df(int n, const __grid_constant
 #pragma unroll
             for (int comp = 0; comp < 2; ++comp) {
                 const size_t k = comp * n2 + idx;
-                double r = 0.0;
-                if (slot_unknown(cn, s)) r = f[k] - a.au[comp][s] - a.bt[comp][s];
+                const double r = slot_unknown(cn, s) ? a.au[comp][s] : 0.0;
                 const float hi = (float)r;
                 ru[k] = make_float2(hi, (float)(r - (double)hi));
                 r32u[PL ? i32 + comp : k] = hi;
-                ss += r * r;
+                ss = fma(r, r, ss);
             }
         }
         const size_t vi = (size_t)j * (n + 1) + i;
-        const double r = (dom == kDomL && l_masked_vertex(i, j, n)) ? 0.0 : g[vi] - a.bu;
+        const double r = (dom == kDomL && l_masked_vertex(i, j, n)) ? 0.0 : a.bu;
         const float hi = (float)r;
         rp[vi] = make_float2(hi, (float)(r - (double)hi));
         r32p[PL ? (size_t)j * pl_vpitch(n) + i : vi] = hi;
@@ -388,7 +399,7 @@ __global__ void __launch_bounds__(NT) k_residual_df(int n, const __grid_constant
 void launch_ir_update_df(cudaStream_t s, int n, const OpCoef<float>& chi, const OpCoef<float>& clo,
                          const float* eu, const float* ep, double* xu, double* xp, double* ru, double* rp,
                          float* r32u, float* r32p, double* partial, double* wpartial, bool planar, int dom) {
-    launch_pdl(planar ? k_ir_update_df<true> : k_ir_update_df<false>, cells_grid(n), dim3(BX, BY), 0, s, n, chi, clo,
+    launch_pdl(planar ? k_ir_update_df<true> : k_ir_update_df<false>, cells_grid(n), cells_block(n), 0, s, n, chi, clo,
                make_df_pairs(chi, clo), eu, ep, xu, xp, reinterpret_cast<float2*>(ru), reinterpret_cast<float2*>(rp), r32u,
                r32p, partial, wpartial, 1.0 / (6.0 * (double)n * (double)n), dom);
 }
@@ -396,7 +407,7 @@ void launch_ir_update_df(cudaStream_t s, int n, const OpCoef<float>& chi, const 
 void launch_residual_df(cudaStream_t s, int n, const OpCoef<double>& c, const double* u, const double* p,
                         const double* f, const double* g, double* ru, double* rp, float* r32u, float* r32p,
                         double* partial, bool planar, int dom) {
-    launch_pdl(planar ? k_residual_df<true> : k_residual_df<false>, cells_grid(n), dim3(BX, BY), 0, s, n, c, u, p, f,
+    launch_pdl(planar ? k_residual_df<true> : k_residual_df<false>, cells_grid(n), cells_block(n), 0, s, n, c, u, p, f,
                g, reinterpret_cast<float2*>(ru), reinterpret_cast<float2*>(rp), r32u, r32p, partial, dom);
 }
 

@@ -5,7 +5,6 @@
 #include <algorithm>
 #include <cmath>
 
-#include "coef.h"
 #include "common.cuh"
 
 namespace smg {
@@ -189,24 +188,16 @@ struct alignas(16) E2 {              // the x and the y coefficient and an offse
 __host__ __device__ constexpr int list_start(int s) { return s == 0 ? 0 : 18 + 9 * s; }
 constexpr int kListA = 54, kListBT = 12, kListB = 16;   // per class: 27 + 9 + 9 + 9, 4 + 4 + 4, 16
 
-// Which entries there are, read once off the float64 stencils at beta h^2 = 1, where stiffness and mass are of
-// one size (at small beta h^2 the entries that only the mass has are tiny, and yet they count: leaving them
-// out below 1e-6 of the largest made float32 W-cycles a hundred times less accurate).
+// Which entries there are (window points, -1: none), from the masks of common.cuh.  (Not from a level's own
+// coefficients: at small beta h^2 the entries that only the mass has are tiny, and yet they count; leaving them
+// out below 1e-6 of the largest made float32 W-cycles a hundred times less accurate.)
 struct ListStructure {
-    signed char A[kStencilClasses][kListA], BT[kStencilClasses][kListBT], B[kStencilClasses][kListB];   // window points, -1: none
+    signed char A[kStencilClasses][kListA], BT[kStencilClasses][kListBT], B[kStencilClasses][kListB];
     bool ok = true;
 };
 inline const ListStructure& list_structure() {
     static const ListStructure S = [] {
         ListStructure r;
-        const OpCoef<double> c = make_coef<double>(4, 16.0);
-        double amax = 0.0, bmax = 0.0;
-        for (int k = 0; k < kStencilClasses; ++k)
-            for (int w = 0; w < 25; ++w) {
-                for (int s = 0; s < 4; ++s) amax = std::max(amax, std::fabs(c.MA[k][s][w]));
-                bmax = std::max({bmax, std::fabs(c.MBx[k][w]), std::fabs(c.MBy[k][w])});
-            }
-        const double ta = 1e-12 * amax, tb = 1e-12 * bmax;
         for (int k = 0; k < kStencilClasses; ++k) {
             for (auto& v : r.A[k]) v = -1;
             for (auto& v : r.BT[k]) v = -1;
@@ -214,20 +205,20 @@ inline const ListStructure& list_structure() {
             for (int s = 0; s < 4; ++s) {
                 int m = 0;
                 for (int w = 0; w < 25; ++w)
-                    if (std::fabs(c.MA[k][s][w]) > ta) {
+                    if (nz_MA(k, s, w)) {
                         if (m == (s == 0 ? (k == 6 ? 21 : 18) : 9)) r.ok = false;
                         else r.A[k][list_start(s) + m++] = (signed char)w;
                     }
                 m = 0;
                 for (int v = 0; v < 9; ++v)
-                    if (std::fabs(c.MBTx[k][s][v]) > tb || std::fabs(c.MBTy[k][s][v]) > tb) {
+                    if (nz_MBT(k, s, v)) {
                         if (s == 0 || m == 4) r.ok = false;
                         else r.BT[k][4 * (s - 1) + m++] = (signed char)v;
                     }
             }
             int m = 0;
             for (int w = 0; w < 25; ++w)
-                if (std::fabs(c.MBx[k][w]) > tb || std::fabs(c.MBy[k][w]) > tb) {
+                if (nz_MB(k, w)) {
                     if (m == (k == 6 ? 16 : 12)) r.ok = false;
                     else r.B[k][m++] = (signed char)w;
                 }

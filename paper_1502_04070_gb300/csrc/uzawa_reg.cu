@@ -26,7 +26,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <type_traits>
 
 #include <cuda.h>
 
@@ -1169,12 +1168,26 @@ __device__ __forceinline__ void embed_apply(const EmbedJob& jb, int n, int TY, i
         addp(2 * I + 1, 2 * J + 1, 0.5f * (orient(I, J, nc) == 0 ? jb.p00 + jb.p11 : jb.p10 + jb.p01));
 }
 
+// what the tiles on the mid-lines read: the level's lists, or its operator (the per-cell rows)
+template <bool LISTS>
+struct RowTables {
+    const MidLists* ml;
+    __device__ __forceinline__ const OpCoef<float>* op() const { return nullptr; }
+    __device__ __forceinline__ const MidLists* lists() const { return ml; }
+};
+template <>
+struct RowTables<false> {
+    OpCoef<float> c;
+    __device__ __forceinline__ const OpCoef<float>* op() const { return &c; }
+    __device__ __forceinline__ const MidLists* lists() const { return nullptr; }
+};
+
 // pf > 0: also prefetch into L2 the tiles of tile blockIdx.x + pf (about one wave of resident CTAs
 // ahead), so that the CTA that takes it finds its tiles in L2
-template <int NW, int MINB, bool PAIR = false>
+template <int NW, int MINB, bool PAIR, bool LISTS>
 __global__ void __launch_bounds__(32 * NW, MINB)
-    k_uzawa_tma(int n, int TY, TileOrder ord, const __grid_constant__ RegCoef q, const MidLists* __restrict__ ml,
-                float sigma, const __grid_constant__ TmaMaps maps, float* __restrict__ u_out,
+    k_uzawa_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t, const __grid_constant__ RegCoef q,
+                float tau, float sigma, const __grid_constant__ TmaMaps maps, float* __restrict__ u_out,
                 float* __restrict__ p_out, int pf, const float* __restrict__ uc, const float* __restrict__ pc, int pcp) {
     using G = TmaTile;
     extern __shared__ unsigned char smem_raw[];
@@ -1232,7 +1245,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         }
         __syncthreads();
     }
-    reg_phases<G, true, NW, PAIR, true>(n, TY, i0, j0, nullptr, q, ml, 0.f, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, true, NW, PAIR, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -1448,9 +1461,9 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
     }
 }
 
-template <int NW, int MINB, bool PC>
+template <int NW, int MINB, bool PC, bool LISTS>
 __global__ void __launch_bounds__(32 * NW, MINB)
-    k_restrict_tma(int n, int TY, TileOrder ord, const MidLists* __restrict__ ml, const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
+    k_restrict_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t, const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
                    const __grid_constant__ TmaMaps maps, float* __restrict__ fc, float* __restrict__ gc,
                    float* __restrict__ uc, float* __restrict__ pc) {
     using G = TmaTile;
@@ -1490,7 +1503,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         }
         return;
     }
-    defect_restrict<G, NW, PC, true>(n, TY, i0, j0, nullptr, q, ml, wt, sU, sF, sP, sG, fc, gc, uc, pc);
+    defect_restrict<G, NW, PC, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), wt, sU, sF, sP, sG, fc, gc, uc, pc);
     pdl_trigger();
 }
 
@@ -1838,21 +1851,24 @@ cudaError_t reg_smem_attr() {
 }
 template <int NW, int MINB, bool PAIR = false>
 cudaError_t tma_smem_attr() {
-    return cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)TmaTile::bytes(kRegMaxRows));
+    const cudaError_t e = cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)TmaTile::bytes(kRegMaxRows));
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR, true>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TmaTile::bytes(kRegMaxRows));
 }
 
 // Rows per tile for level size n, among the tile heights that keep at least MINB CTAs of kernel k (dynamic
-// shared memory G::bytes(ty)) resident per SM.  The planar step (TmaTile): a model of its measured time, the longer of
+// shared memory G::bytes(ty)) resident per SM.  `model`: a model of the planar step's measured time, the longer of
 // two terms plus a third of the shorter.  The first is the longest CTA, a tile on a mid-line: one unit per pass
 // of its 8 warps over the rows of a phase, ceil((ty + 4) / 8) + ceil((ty + 2) / 8) + ceil(ty / 8), and three for the launch and the
 // tile's arrival; the second the whole GPU's work, tiles x (ty + 7.3) / (9.4 per SM) (the unit is 0.87 us on a GB300).  It
 // picks 4, 4, 12 and 20 or more rows at N = 128, 256, 512 and from 1024 on: 5.5, 6.8, 11.1 us a step, where
 // balancing the tiles over the SMs alone took 5.9, 8.7, 12.9.  `shared` (the solves of a batch, which fill the GPU
-// together): the work plus a third of the longest CTA (24 uneven solves 33.5 against 37.8 ms).  The compact step (RegTile): the least work on the busiest
-// SM, (tiles per SM, rounded up) x (ty + 4).
+// together): the work plus a third of the longest CTA (24 uneven solves 33.5 against 37.8 ms).  Without `model`: the least
+// work on the busiest SM, (tiles per SM, rounded up) x (ty + 4).
 template <class G, class K>
-int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false, bool shared = false) {
+int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false, bool model = false, bool shared = false) {
     const int lv = 31 - __builtin_clz((unsigned)n);
     int& r = cache[lv & 31];
     if (r) return r;
@@ -1870,7 +1886,7 @@ int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false,
             continue;
         const long tiles = (long)cols * ((n + 1 + ty - 1) / ty);
         double cost = (double)((tiles + sms - 1) / sms) * (ty + 4);
-        if (std::is_same<G, TmaTile>::value) {
+        if (model) {
             const double lat = 3.0 + (ty + 11) / 8 + (ty + 9) / 8 + (ty + 7) / 8, thr = (double)tiles * (ty + 7.3) / (9.4 * sms);
             cost = shared ? thr + 0.35 * lat : std::max(lat, thr) + 0.35 * std::min(lat, thr);
         }
@@ -1886,8 +1902,11 @@ int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false,
 
 template <bool PC>
 cudaError_t rt_smem_attr() {
-    return cudaFuncSetAttribute(k_restrict_tma<8, 3, PC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)TmaTile::bytes(kRegMaxRows));
+    const cudaError_t e = cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)TmaTile::bytes(kRegMaxRows));
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)TmaTile::bytes(kRegMaxRows));
 }
 
 template <int NW, int MINB>
@@ -1896,9 +1915,10 @@ int reg_rows(int n) {
     return tile_rows<RegTile>(n, k_uzawa_reg<NW, MINB>, 32 * NW, MINB, cache);
 }
 template <int NW, int MINB, bool PAIR = false>
-int tma_rows(int n, bool shared) {
-    static int cache[2][32] = {};
-    return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR>, 32 * NW, MINB, cache[shared], PAIR, shared);
+int tma_rows(int n, const PlanarLevel& pl) {
+    static int cache[3][32] = {};
+    if (!pl.lists) return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR, false>, 32 * NW, MINB, cache[0], PAIR);
+    return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR, true>, 32 * NW, MINB, cache[1 + pl.shared], PAIR, true, pl.shared);
 }
 template <class G>
 TileOrder tile_order(int n, int ty) {
@@ -1967,12 +1987,12 @@ bool make_tma_maps(int n, int ty, const float* u, const float* p, const float* f
 }
 
 template <int NW, int MINB, bool PAIR = false>
-bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau, float sigma, const float* u, const float* p,
+bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau, float sigma, const float* u, const float* p,
                   const float* f, const float* g, const float* sinv, float* u_out, float* p_out, bool prefetch,
                   const CoarseCorrection& cc) {
     RegCoef q;
     if (!make_reg_coef(c, tau, q)) return false;
-    int ty = tma_rows<NW, MINB, PAIR>(n, ml.shared);
+    int ty = tma_rows<NW, MINB, PAIR>(n, pl);
     if (cc.u) ty = std::min(ty, kEmbedMaxRows);
     TmaMaps m;
     if (!make_tma_maps(n, ty, u, p, f, g, sinv, m)) return false;
@@ -1982,14 +2002,19 @@ bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLev
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_uzawa_tma<NW, MINB, PAIR>, 32 * NW,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_uzawa_tma<NW, MINB, PAIR, true>, 32 * NW,
                                                           TmaTile::bytes(ty)) != cudaSuccess)
             per_sm = MINB;
         cudaGetLastError();
         pf = std::max(1, sms) * std::max(1, per_sm);
     }
-    launch_pdl(k_uzawa_tma<NW, MINB, PAIR>, dim3(ord.cols * ord.rows), dim3(32 * NW), TmaTile::bytes(ty), s, n, ty, ord, q,
-               ml.lists, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
+    const dim3 grid(ord.cols * ord.rows), block(32 * NW);
+    if (pl.lists)
+        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, true>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
+                   tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
+    else
+        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, false>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q, tau,
+                   sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
     return true;
 }
 
@@ -2021,16 +2046,21 @@ const RestrictWeights& restrict_weights() {
 }
 
 template <bool PC>
-bool launch_rt(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, const float* u, const float* p, const float* f,
+bool launch_rt(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, const float* u, const float* p, const float* f,
                const float* g, float* fc, float* gc, float* uc, float* pc) {
     RegCoef q;
     if (!make_reg_coef(c, 1.0f, q)) return false;
-    const int ty = std::max(4, tma_rows<8, 3>(n, ml.shared) & ~1);   // even: whole coarse cells per tile
+    const int ty = std::max(4, tma_rows<8, 3>(n, pl) & ~1);   // even: whole coarse cells per tile
     TmaMaps m;
     if (!make_tma_maps(n, ty, u, p, f, g, g, m)) return false;   // no Shat^{-1} tile (its map is unused)
     const TileOrder ord = tile_order<TmaTile>(n, ty);
-    launch_pdl(k_restrict_tma<8, 3, PC>, dim3(ord.cols * ord.rows), dim3(256), TmaTile::bytes(ty), s, n, ty, ord, ml.lists, q,
-               restrict_weights(), m, fc, gc, uc, pc);
+    const dim3 grid(ord.cols * ord.rows);
+    if (pl.lists)
+        launch_pdl(k_restrict_tma<8, 3, PC, true>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
+                   restrict_weights(), m, fc, gc, uc, pc);
+    else
+        launch_pdl(k_restrict_tma<8, 3, PC, false>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q,
+                   restrict_weights(), m, fc, gc, uc, pc);
     return true;
 }
 
@@ -2083,10 +2113,10 @@ cudaError_t launch_small_cycle(cudaStream_t s, const SmallCycleHost& h) {
     return cudaLaunchKernelEx(&cfg, k_small_cycle, A);
 }
 
-bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& ml,
+bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& pl,
                          const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc, float* pc) {
-    return pc_planar ? launch_rt<true>(s, n, c, ml, u, p, f, g, fc, gc, uc, pc)
-                     : launch_rt<false>(s, n, c, ml, u, p, f, g, fc, gc, uc, pc);
+    return pc_planar ? launch_rt<true>(s, n, c, pl, u, p, f, g, fc, gc, uc, pc)
+                     : launch_rt<false>(s, n, c, pl, u, p, f, g, fc, gc, uc, pc);
 }
 
 cudaError_t prepare_uzawa_reg() {
@@ -2110,29 +2140,29 @@ bool launch_uzawa_reg(int variant, cudaStream_t s, int n, const OpCoef<float>& c
 }
 
 namespace {
-int g_tma_choice[32] = {};     // planar step variant per level size (log2 N)
+int g_tma_choice[2][32] = {};  // planar step variant per level size (log2 N), with the lists and without
 bool g_tma_tuned[32] = {};
 int lvl(int n) { return (31 - __builtin_clz((unsigned)n)) & 31; }
 }  // namespace
 
-bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
+bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau,
                               float sigma, const float* u, const float* p, const float* f, const float* g, const float* sinv,
                               float* u_out, float* p_out, const CoarseCorrection& cc) {
     if (cc.u && (!cc.p || !embed_table_matches())) return false;
     switch (variant) {
-        case 1: return launch_tma_v<8, 3>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        case 2: return launch_tma_v<8, 4>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
-        case 3: return launch_tma_v<8, 4>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        case 4: return launch_tma_v<8, 2, true>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        case 5: return launch_tma_v<8, 3, true>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
-        default: return launch_tma_v<8, 3>(s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
+        case 1: return launch_tma_v<8, 3>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        case 2: return launch_tma_v<8, 4>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
+        case 3: return launch_tma_v<8, 4>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        case 4: return launch_tma_v<8, 2, true>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        case 5: return launch_tma_v<8, 3, true>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
+        default: return launch_tma_v<8, 3>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
     }
 }
 
-bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau, float sigma,
+bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau, float sigma,
                       const float* u, const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
                       const CoarseCorrection& cc) {
-    return launch_uzawa_tma_variant(g_tma_choice[lvl(n)], s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
+    return launch_uzawa_tma_variant(g_tma_choice[pl.lists == nullptr][lvl(n)], s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
 }
 
 bool uzawa_tma_embed_available() { return uzawa_tma_available() && embed_table_matches(); }
@@ -2144,16 +2174,16 @@ void embed_weights_table(double* w) {
                 for (int fa = 0; fa < 4; ++fa) w[((o * 9 + L) * 4 + fb) * 4 + fa] = embed_weight(o, L, fa, fb);
 }
 
-int tma_choice(int n) { return g_tma_choice[lvl(n)]; }
+int tma_choice(int n) { return g_tma_choice[0][lvl(n)]; }
 bool tma_tuned(int n) { return g_tma_tuned[lvl(n)]; }
 bool set_tma_choice(int n, int v) {
     if (v < 0 || v >= kTmaVariants) return false;
-    g_tma_choice[lvl(n)] = v;
+    g_tma_choice[0][lvl(n)] = g_tma_choice[1][lvl(n)] = v;
     g_tma_tuned[lvl(n)] = true;
     return true;
 }
 
-cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
+cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau,
                                float sigma, float* u, float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return cudaErrorUnknown;
@@ -2166,11 +2196,11 @@ cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, co
     float bms = 1e30f;
     cudaError_t err = cudaSuccess;
     for (int v = 0; v < kTmaVariants && err == cudaSuccess; ++v) {
-        if (!launch_uzawa_tma_variant(v, s, n, c, ml, tau, sigma, u, p, f, g, sinv, u_out, p_out)) continue;   // warm-up
+        if (!launch_uzawa_tma_variant(v, s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out)) continue;   // warm-up
         bool sw = true;
         cudaEventRecord(e0, s);
         for (int r = 0; r < reps; ++r) {
-            launch_uzawa_tma_variant(v, s, n, c, ml, tau, sigma, sw ? u_out : u, sw ? p_out : p, f, g, sinv, sw ? u : u_out,
+            launch_uzawa_tma_variant(v, s, n, c, pl, tau, sigma, sw ? u_out : u, sw ? p_out : p, f, g, sinv, sw ? u : u_out,
                                      sw ? p : p_out);
             sw = !sw;
         }
@@ -2186,7 +2216,7 @@ cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, co
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (err != cudaSuccess) return err;
-    g_tma_choice[lvl(n)] = best;
+    g_tma_choice[pl.lists == nullptr][lvl(n)] = best;
     g_tma_tuned[lvl(n)] = true;
     return cudaGetLastError();
 }
