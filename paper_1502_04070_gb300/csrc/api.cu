@@ -458,11 +458,12 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
     }
 }
 
-// True float64 residual of the finest state, its norm^2 into scal[0].  In MIXED mode the residual
-// is kept in float64 (the finest temporaries) for the refinement updates and copied to float32 as
-// the right-hand side of the next correction problem.
-void residual_norm_fin(stokes_handle* h, bool timed = false) {
+// True float64 residual of the finest state, its norm^2 into scal[0] (and, with `mean`, w^T p into scal[1]),
+// then the loop's test.  In MIXED mode the residual is kept in float64 (the finest temporaries) for the
+// refinement updates and copied to float32 as the right-hand side of the next correction problem.
+void residual_norm_fin(stokes_handle* h, bool timed = false, bool mean = false, const LoopCheck& ck = LoopCheck{}) {
     Level<double>& F = h->fin();
+    const int nb = cells_blocks(F.n);
     const int k = timed ? ev_begin(h, kEvResid) : -1;
     if (k >= 0) h->ev_resid++;
     if (h->mixed()) {
@@ -471,14 +472,25 @@ void residual_norm_fin(stokes_handle* h, bool timed = false) {
         launch_residual_df(h->st, F.n, F.c, F.u, F.p, F.f, F.g, F.tu, F.tp, E.f, E.g, h->partial, E.planar, h->dom);
     } else {
         launch_residual<double, double>(h->st, F.n, F.c, F.u, F.p, F.f, F.g, F.tu, F.tp, h->partial, nullptr, nullptr,
-                                        h->dom);
+                                        h->dom, mean ? h->partial + nb : nullptr);
     }
     ev_end(h, k);
-    launch_reduce(h->st, h->partial, cells_blocks(F.n), h->scal);
+    launch_reduce_step(h->st, h->partial, nb, h->scal, mean, ck);
 }
 
-// One outer iteration on the internal finest state, ending with ||F - A x||^2 in scal[0].
-void record_step(stokes_handle* h) {
+// One outer iteration on the internal finest state, ending with ||F - A x||^2 in scal[0] and the loop's test.  FP64:
+// the zero-mean projection follows the residual (a constant pressure is in the operator's kernel), which sums the mean
+// on the way.  MIXED: the refinement update sums the mean of the new x_p into scal[1] and takes the previous step's
+// off, so x_p is one projection behind until finish_steps; start_steps clears scal[1].  Every step of a solve thus
+// ends with one launch after its update; stokes_cycle (plain) projects its own result.
+void start_steps(stokes_handle* h) {
+    if (h->mixed()) cudaMemsetAsync(h->scal + 1, 0, sizeof(double), h->st);
+}
+void finish_steps(stokes_handle* h) {
+    Level<double>& F = h->fin();
+    if (h->mixed()) launch_psub<double>(h->st, F.n, F.p, h->scal + 1, h->dom);
+}
+void record_step(stokes_handle* h, const LoopCheck& ck = LoopCheck{}) {
     Level<double>& F = h->fin();
     if (h->mixed()) {
         Level<float>& E = h->h32.back();
@@ -491,15 +503,14 @@ void record_step(stokes_handle* h) {
         // the same pass leaves the partial sums of the zero-mean projection of x_p (second half)
         const int nb = cells_blocks(F.n);
         launch_ir_update_df(h->st, F.n, h->chi, h->clo, E.u, E.p, F.u, F.p, F.tu, F.tp, E.f, E.g, h->partial,
-                            h->partial + nb, E.planar, h->dom);
+                            h->partial + nb, E.planar, h->dom, h->plain ? nullptr : h->scal + 1);
         ev_end(h, k);
-        launch_reduce(h->st, h->partial, nb, h->scal);
-        launch_reduce(h->st, h->partial + nb, nb, h->scal + 1);
-        launch_psub<double>(h->st, F.n, F.p, h->scal + 1, h->dom);
+        launch_reduce_step(h->st, h->partial, nb, h->scal, true, ck);
+        if (h->plain) launch_psub<double>(h->st, F.n, F.p, h->scal + 1, h->dom);
     } else {
         mg_cycle<double>(h, h->h64, h->L - 1);
-        launch_pmean<double>(h->st, F.n, F.p, h->partial, h->scal + 1, h->dom);
-        residual_norm_fin(h, true);
+        residual_norm_fin(h, true, true, ck);
+        launch_psub<double>(h->st, F.n, F.p, h->scal + 1, h->dom);
     }
 }
 
@@ -545,7 +556,7 @@ stokes_status build_plain_graph(stokes_handle* h) {
 }
 
 // The solve loop on the device: one conditional WHILE node whose body is one step followed by
-// k_solve_check (convergence, step limit, divergence).  No event records (not allowed in bodies).
+// the loop's test (convergence, step limit, divergence).  No event records (not allowed in bodies).
 stokes_status build_loop(stokes_handle* h) {
     if (h->loop) return STOKES_OK;
     cudaGraph_t top = nullptr;
@@ -567,8 +578,14 @@ stokes_status build_loop(stokes_handle* h) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(h->st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            record_step(h);
-            launch_solve_check(h->st, hnd, h->scal, h->dctl, h->ictl, h->dhist, stokes_handle_t::kHistCap);
+            LoopCheck ck;
+            ck.mode = 1;
+            ck.hnd = hnd;
+            ck.ctl = h->dctl;
+            ck.ictl = h->ictl;
+            ck.hist = h->dhist;
+            ck.cap = stokes_handle_t::kHistCap;
+            record_step(h, ck);
             e = cudaStreamEndCapture(h->st, &body);
         }
         if (e == cudaSuccess) {
@@ -978,6 +995,7 @@ stokes_status stokes_solve(stokes_handle* h, double* u, double* p, const double*
     if ((s = read_scalar(h, 2, &nF2)) != STOKES_OK) return s;
     const double nF = std::sqrt(nF2);
     residual_norm_fin(h);
+    start_steps(h);
     h->launches += 2;
 
     double r2 = 0.0;
@@ -1064,6 +1082,10 @@ stokes_status stokes_solve(stokes_handle* h, double* u, double* p, const double*
             ++cycles;
             if (history) history[cycles] = r;
         }
+    }
+    if (cycles > 0 && h->mixed()) {
+        finish_steps(h);
+        h->launches += 1;
     }
     if ((s = copy_out(h, u, p)) != STOKES_OK) return s;
     CK(cudaStreamSynchronize(h->st));
@@ -1465,6 +1487,7 @@ static stokes_status batch_build(stokes_batch* b, double* const* u, double* cons
         launch_rhs_norm(st, F.n, F.f, F.g, h->partial);
         launch_reduce(st, h->partial, cells_blocks(F.n), h->scal + 2);
         residual_norm_fin(h);
+        start_steps(h);
         cudaMemsetAsync(b->d_count + i, 0, sizeof(int), st);
         if ((e = cudaStreamEndCapture(st, &gp)) != cudaSuccess) break;
         cudaGraphNode_t np, nc, ne;
@@ -1485,13 +1508,19 @@ static stokes_status batch_build(stokes_batch* b, double* const* u, double* cons
         if ((e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
             cudaSuccess)
             break;
-        record_step(h);
-        launch_batch_check(st, hnd, h->scal, tol * tol, max_cycles, b->d_count + i);
+        LoopCheck ck;
+        ck.mode = 2;
+        ck.hnd = hnd;
+        ck.tol2 = tol * tol;
+        ck.max_cycles = max_cycles;
+        ck.count = b->d_count + i;
+        record_step(h, ck);
         if ((e = cudaStreamEndCapture(st, &body)) != cudaSuccess) break;
         b->body_kernels[i] = count_kernels(body);
         // epilogue: true residual, results out
         cudaGraph_t ge = nullptr;
         if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) break;
+        finish_steps(h);
         residual_norm_fin(h);
         launch_batch_store(st, h->scal, b->d_count + i, b->d_res + 3 * i);
         copy_out(h, u[i], p[i]);
@@ -1613,6 +1642,7 @@ static cudaError_t add_euler_chain(cudaGraph_t top, cudaGraphNode_t* dep, stokes
             launch_rhs_norm(st, F.n, F.f, F.g, h->partial);
             launch_reduce(st, h->partial, cells_blocks(F.n), h->scal + 2);
             residual_norm_fin(h);
+            start_steps(h);
             cudaMemsetAsync(count + n, 0, sizeof(int), st);
         });
         if (e != cudaSuccess) break;
@@ -1629,13 +1659,21 @@ static cudaError_t add_euler_chain(cudaGraph_t top, cudaGraphNode_t* dep, stokes
         if ((e = cudaStreamBeginCaptureToGraph(st, bg, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
             cudaSuccess)
             break;
-        record_step(h);
-        if (h->mixed()) residual_norm_fin(h);   // the test uses the true residual, not the updated one
-        launch_batch_check(st, hnd, h->scal, tol * tol, max_cycles, count + n);
+        LoopCheck ck;
+        ck.mode = 2;
+        ck.hnd = hnd;
+        ck.tol2 = tol * tol;
+        ck.max_cycles = max_cycles;
+        ck.count = count + n;
+        record_step(h, h->mixed() ? LoopCheck{} : ck);
+        if (h->mixed()) residual_norm_fin(h, false, false, ck);   // the test uses the true residual, not the updated one
         if ((e = cudaStreamEndCapture(st, &bg)) != cudaSuccess) break;
         *body = graph_kernels(bg);
         *dep = nc;
-        e = child([&] { launch_batch_store(st, h->scal, count + n, res + 3 * n); });
+        e = child([&] {
+            finish_steps(h);
+            launch_batch_store(st, h->scal, count + n, res + 3 * n);
+        });
     }
     if (e == cudaSuccess)
         e = child([&] {

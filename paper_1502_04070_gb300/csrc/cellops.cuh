@@ -453,5 +453,4 @@ __device__ __forceinline__ double block_sum2d(double v, int tid) {
     return s;
 }
 
-
 }  // namespace smg

@@ -50,13 +50,14 @@ __global__ void __launch_bounds__(NT) k_residual(int n, const __grid_constant__ 
                                                  const T* __restrict__ f, const T* __restrict__ g,
                                                  TO* __restrict__ ru, TO* __restrict__ rp,
                                                  double* __restrict__ partial, float* __restrict__ ru2,
-                                                 float* __restrict__ rp2, int dom) {
+                                                 float* __restrict__ rp2, int dom, double* __restrict__ wpartial,
+                                                 double wscale) {
     static_assert(!PL || (sizeof(T) == 4 && sizeof(TO) == 4), "the planar layout is float32 only");
     pdl_wait();
     CELL_INDEX
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
     const int vld = PL ? pl_vpitch(n) : n + 1;
-    double ss = 0.0;
+    double ss = 0.0, wp = 0.0;
     if (active) {
         const CellNodes cn = cell_nodes_dom(i, j, n, dom);
         const int ld = 2 * n + 1;
@@ -109,8 +110,15 @@ __global__ void __launch_bounds__(NT) k_residual(int n, const __grid_constant__ 
         rp[vi] = (TO)r;
         if (!PL && rp2) rp2[vi] = (float)r;
         ss += (double)r * (double)r;
+        if (wpartial) wp = (double)vertex_triangles_dom(i, j, n, dom) * (double)p[vi];
     }
-    if (partial) {
+    if (wpartial) {   // and the zero-mean projection's numerator sum_i w_i p_i, w_i = (triangles at i) h^2 / 6
+        const double2 t = block_sum2d_pair(ss, wp, tid);
+        if (tid == 0) {
+            partial[blockIdx.y * gridDim.x + blockIdx.x] = t.x;
+            wpartial[blockIdx.y * gridDim.x + blockIdx.x] = t.y * wscale;
+        }
+    } else if (partial) {
         const double t = block_sum2d(ss, tid);
         if (tid == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
@@ -295,22 +303,22 @@ void launch_normal_eq(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T* u, T*
                       const T* g, const T* sinv, T* zu, T* zp) {
     const dim3 grid = cells_grid(n), blk = cells_block(n);
     launch_pdl(k_residual<T, T, false>, grid, blk, 0, s, n, c, u, p, f, g, zu, zp, nullptr, nullptr, nullptr,
-               (int)kDomSquare);
+               (int)kDomSquare, (double*)nullptr, 0.0);
     launch_pdl(k_scale_L<T>, grid, blk, 0, s, n, c, zu, zp, sinv);
     launch_pdl(k_normal_update<T>, grid, blk, 0, s, n, c, tau, zu, zp, sinv, u, p);
 }
 
 template <typename T, typename TO>
 void launch_residual(cudaStream_t s, int n, const OpCoef<T>& c, const T* u, const T* p, const T* f,
-                     const T* g, TO* ru, TO* rp, double* partial, float* ru2, float* rp2, int dom) {
+                     const T* g, TO* ru, TO* rp, double* partial, float* ru2, float* rp2, int dom, double* wpartial) {
     launch_pdl(k_residual<T, TO, false>, cells_grid(n), cells_block(n), 0, s, n, c, u, p, f, g, ru, rp, partial, ru2, rp2,
-               dom);
+               dom, wpartial, 1.0 / (6.0 * (double)n * (double)n));
 }
 
 void launch_residual_planar(cudaStream_t s, int n, const OpCoef<float>& c, const float* u, const float* p,
                             const float* f, const float* g, float* ru, float* rp) {
     launch_pdl(k_residual<float, float, true>, cells_grid(n), cells_block(n), 0, s, n, c, u, p, f, g, ru, rp,
-               (double*)nullptr, (float*)nullptr, (float*)nullptr, (int)kDomSquare);
+               (double*)nullptr, (float*)nullptr, (float*)nullptr, (int)kDomSquare, (double*)nullptr, 0.0);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -678,19 +686,6 @@ void launch_schur_diag(cudaStream_t s, int n, const OpCoef<double>& c, T* sinv, 
 
 // ------------------------------------------------------------------------------------------
 
-template <typename T>
-__global__ void __launch_bounds__(NT) k_pmean_partial(int n, const T* __restrict__ p, double* __restrict__ partial,
-                                                      double wscale, int dom) {
-    pdl_wait();
-    CELL_INDEX
-    // w_i = (triangles at vertex i) h^2 / 6: counted per vertex, scaled per block
-    double v = 0.0;
-    if (active) v = (double)vertex_triangles_dom(i, j, n, dom) * (double)p[(size_t)j * (n + 1) + i];
-    const double t = block_sum2d(v, tid);
-    if (tid == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = t * wscale;
-    pdl_trigger();
-}
-
 // p -= (w^T p) / |Omega| at the pressure unknowns; |Omega| = sum_i w_i = 1 (square) or 3/4 (L)
 template <typename T>
 __global__ void __launch_bounds__(NT) k_psub(int n, T* __restrict__ p, const double* __restrict__ scalar, int dom) {
@@ -721,16 +716,51 @@ __global__ void k_reduce(const double* __restrict__ partial, int count, double* 
     pdl_trigger();
 }
 
-cudaError_t launch_reduce(cudaStream_t s, const double* partial, int count, double* out) {
-    return launch_pdl(k_reduce, 1, 1024, 0, s, partial, count, out);
+// one thread: the test of LoopCheck (kernels.cuh)
+__device__ void loop_check(const LoopCheck& q, double r2, double f2) {
+    if (q.mode == 1) {
+        const int c = q.ictl[0] + 1;
+        q.ictl[0] = c;
+        if (c < q.cap) q.hist[c] = r2;
+        const int grow = r2 > q.ctl[2] ? q.ictl[1] + 1 : 0;
+        q.ictl[1] = grow;
+        q.ctl[2] = r2;
+        const bool go = isfinite(r2) && r2 > q.ctl[0] * f2 && c < (int)q.ctl[1] && grow < 8;
+        cudaGraphSetConditional(q.hnd, go ? 1u : 0u);
+    } else if (q.mode == 2) {
+        const int c = *q.count + 1;
+        *q.count = c;
+        const bool go = isfinite(r2) && r2 > q.tol2 * f2 && c < q.max_cycles;
+        cudaGraphSetConditional(q.hnd, go ? 1u : 0u);
+    }
 }
 
-template <typename T>
-void launch_pmean(cudaStream_t s, int n, T* p, double* partial, double* scalar, int dom) {
-    const dim3 grid = cells_grid(n), blk = cells_block(n);
-    launch_pdl(k_pmean_partial<T>, grid, blk, 0, s, n, p, partial, 1.0 / (6.0 * (double)n * (double)n), dom);
-    launch_pdl(k_reduce, 1, 1024, 0, s, partial, grid.x * grid.y, scalar);
-    launch_pdl(k_psub<T>, grid, blk, 0, s, n, p, scalar, dom);
+// The end of a step: CTA 0 sums the residual's partial sums into scal[0] and decides whether the loop goes on
+// (loop_check), CTA 1 the pressure mean's (`count` further on) into scal[1]; each a fixed-order tree.
+__global__ void k_reduce_step(const double* __restrict__ partial, int count, double* __restrict__ scal, LoopCheck ck) {
+    pdl_wait();
+    __shared__ double red[1024];
+    const double* p = partial + (blockIdx.x ? count : 0);
+    double s = 0.0;
+    for (int k = threadIdx.x; k < count; k += blockDim.x) s += p[k];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        scal[blockIdx.x] = red[0];
+        if (blockIdx.x == 0) loop_check(ck, red[0], scal[2]);
+    }
+    pdl_trigger();
+}
+void launch_reduce_step(cudaStream_t s, const double* partial, int count, double* scal, bool mean, const LoopCheck& ck) {
+    launch_pdl(k_reduce_step, mean ? 2 : 1, 1024, 0, s, partial, count, scal, ck);
+}
+
+cudaError_t launch_reduce(cudaStream_t s, const double* partial, int count, double* out) {
+    return launch_pdl(k_reduce, 1, 1024, 0, s, partial, count, out);
 }
 
 template <typename T>
@@ -1022,18 +1052,17 @@ void launch_mask_l(cudaStream_t s, int n, double* u, double* p) {
     template void launch_prolong_add<T>(cudaStream_t, int, const T*, const T*, T*, T*, int);              \
     template void launch_coarse_solve<T>(cudaStream_t, const double*, const T*, const T*, T*, T*);        \
     template void launch_schur_diag<T>(cudaStream_t, int, const OpCoef<double>&, T*, int, int);           \
-    template void launch_pmean<T>(cudaStream_t, int, T*, double*, double*, int);                          \
     template void launch_load<T>(cudaStream_t, int, const MassCoef<T>&, const T*, const T*, T*, T*, int,  \
                                  double*, double*);
 INST(float)
 INST(double)
 template void launch_residual<double, double>(cudaStream_t, int, const OpCoef<double>&, const double*,
                                               const double*, const double*, const double*, double*, double*,
-                                              double*, float*, float*, int);
+                                              double*, float*, float*, int, double*);
 template void launch_residual<float, float>(cudaStream_t, int, const OpCoef<float>&, const float*, const float*,
-                                            const float*, const float*, float*, float*, double*, float*, float*, int);
+                                            const float*, const float*, float*, float*, double*, float*, float*, int, double*);
 template void launch_residual<double, float>(cudaStream_t, int, const OpCoef<double>&, const double*,
                                              const double*, const double*, const double*, float*, float*,
-                                             double*, float*, float*, int);
+                                             double*, float*, float*, int, double*);
 
 }  // namespace smg

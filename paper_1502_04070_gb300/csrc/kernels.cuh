@@ -17,7 +17,7 @@ int cells_blocks(int n);
 template <typename T, typename TO>
 void launch_residual(cudaStream_t s, int n, const OpCoef<T>& c, const T* u, const T* p, const T* f,
                      const T* g, TO* ru, TO* rp, double* partial, float* ru2 = nullptr, float* rp2 = nullptr,
-                     int dom = kDomSquare);
+                     int dom = kDomSquare, double* wpartial = nullptr);   // wpartial: partial sums of w^T p too
 
 
 // Uzawa step (Sec. 4), three kernels:
@@ -36,7 +36,7 @@ void launch_uzawa(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T sigma, T* 
 void launch_ir_update_df(cudaStream_t s, int n, const OpCoef<float>& chi, const OpCoef<float>& clo,
                          const float* eu, const float* ep, double* xu, double* xp, double* ru, double* rp,
                          float* r32u, float* r32p, double* partial, double* wpartial, bool planar = false,
-                         int dom = kDomSquare);
+                         int dom = kDomSquare, const double* mean = nullptr);   // mean: taken from x_p first
 // p -= *scalar on every vertex (the zero-mean projection once the integral of p is reduced); on the
 // L (dom = kDomL) p -= *scalar / (3/4) at the L's vertices
 template <typename T>
@@ -220,10 +220,22 @@ constexpr int kMaxCoarseLevel = 3;   // N = 16: a bordered system of 2212 unknow
 template <typename T>
 void launch_schur_diag(cudaStream_t s, int n, const OpCoef<double>& c, T* sinv, int dom = kDomSquare, int vld = 0);
 
-// p <- p - sum_i w_i p_i  (w = M_P 1, sum w = 1): partial sums then subtraction
-template <typename T>
-void launch_pmean(cudaStream_t s, int n, T* p, double* partial, double* scalar, int dom = kDomSquare);
-
+// What a step's last kernel decides on the device (0: nothing): whether the conditional WHILE node runs its body
+// again, from the step's ||r||^2 and ||F||^2.
+//   1, a single solve: ctl: [0] threshold factor (stop when r^2 <= ctl[0] ||F||^2), [1] max steps, [2] previous r^2;
+//      ictl: [0] step count, [1] consecutive growths (8: diverged); hist[c] = r^2 after step c (c < cap);
+//   2, an instance of a batch or a time step: stop at r^2 <= tol2 ||F||^2 or after max_cycles (*count so far).
+struct LoopCheck {
+    int mode = 0;
+    cudaGraphConditionalHandle hnd = 0;
+    double *ctl = nullptr, *hist = nullptr;
+    int *ictl = nullptr, *count = nullptr;
+    int cap = 0, max_cycles = 0;
+    double tol2 = 0.0;
+};
+// scal[0] = sum of partial[0..count), with `mean` also scal[1] = sum of partial[count..2 count), and the loop's test
+// of scal[0] against scal[2]
+void launch_reduce_step(cudaStream_t s, const double* partial, int count, double* scal, bool mean, const LoopCheck& ck);
 // out[0] = sum of partial[0..count); returns the launch's own status
 cudaError_t launch_reduce(cudaStream_t s, const double* partial, int count, double* out);
 
@@ -264,12 +276,8 @@ static_assert(sizeof(CoarseCycleArgs) <= 32764, "coarse-cycle parameters exceed 
 cudaError_t prepare_coarse_cycle();
 void launch_coarse_cycle(cudaStream_t s, const CoarseCycleArgs& a);
 
-// batched solver: device-side WHILE condition and result store (batch.cu)
-void launch_batch_check(cudaStream_t s, cudaGraphConditionalHandle hnd, const double* scal, double tol2,
-                        int max_cycles, int* count);
+// batched solver: result store (batch.cu)
 void launch_batch_store(cudaStream_t s, const double* scal, const int* count, double* out);
-void launch_solve_check(cudaStream_t s, cudaGraphConditionalHandle hnd, const double* scal, double* ctl, int* ictl,
-                        double* hist, int cap);
 
 // x64 += e32 (count elements), and float64 -> float32 conversion
 void launch_add_f32(cudaStream_t s, size_t count, const float* e, double* x);

@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(NT, 4) k_ir_update_df(int n, const __grid_cons
                                                      float2* __restrict__ ru, float2* __restrict__ rp,
                                                      float* __restrict__ r32u, float* __restrict__ r32p,
                                                      double* __restrict__ partial, double* __restrict__ wpartial,
-                                                     double wscale, int dom) {
+                                                     double wscale, int dom, const double* __restrict__ mean) {
     pdl_wait();
     CELL_INDEX
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
@@ -319,7 +319,9 @@ __global__ void __launch_bounds__(NT, 4) k_ir_update_df(int n, const __grid_cons
         }
         const size_t vi = (size_t)j * (n + 1) + i, vi32 = PL ? (size_t)j * pl_vpitch(n) + i : vi;
         if (!(dom == kDomL && l_masked_vertex(i, j, n))) {   // vertices outside the L keep zero
-            const double xpn = xp[vi] + (double)ep[vi32];
+            // the zero-mean projection of the step before, where the solve takes it along instead of in a pass of its own
+            const double m = mean ? (dom == kDomL ? *mean / 0.75 : *mean) : 0.0;
+            const double xpn = (xp[vi] - m) + (double)ep[vi32];
             xp[vi] = xpn;
             wp = (double)vertex_triangles_dom(i, j, n, dom) * xpn;
             const float2 r = df_sub(rp[vi], a.bu);
@@ -398,10 +400,10 @@ __global__ void __launch_bounds__(NT, 2) k_residual_df(int n, const __grid_const
 
 void launch_ir_update_df(cudaStream_t s, int n, const OpCoef<float>& chi, const OpCoef<float>& clo,
                          const float* eu, const float* ep, double* xu, double* xp, double* ru, double* rp,
-                         float* r32u, float* r32p, double* partial, double* wpartial, bool planar, int dom) {
+                         float* r32u, float* r32p, double* partial, double* wpartial, bool planar, int dom, const double* mean) {
     launch_pdl(planar ? k_ir_update_df<true> : k_ir_update_df<false>, cells_grid(n), cells_block(n), 0, s, n, chi, clo,
                make_df_pairs(chi, clo), eu, ep, xu, xp, reinterpret_cast<float2*>(ru), reinterpret_cast<float2*>(rp), r32u,
-               r32p, partial, wpartial, 1.0 / (6.0 * (double)n * (double)n), dom);
+               r32p, partial, wpartial, 1.0 / (6.0 * (double)n * (double)n), dom, mean);
 }
 
 void launch_residual_df(cudaStream_t s, int n, const OpCoef<double>& c, const double* u, const double* p,
