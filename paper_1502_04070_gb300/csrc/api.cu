@@ -250,13 +250,23 @@ PlanarLevel planar_level(const stokes_handle* h, const Level<T>& lv) {
     return PlanarLevel{h->plain ? nullptr : lv.mid, h->shared};
 }
 
+// Does an iteration on level l that starts from zero (mg_cycle's `zero`) ignore what (u, p) hold?  Then nobody has
+// to clear them: the exact solve, the cluster cycle, and the planar step's first pre-smoothing step.
+template <typename T>
+bool ignores_iterate(const stokes_handle* h, const std::vector<Level<T>>& H, int l) {
+    if (h->plain || h->prm.smoother != STOKES_UZAWA || l <= h->small_top) return false;
+    return l == h->clev || (l <= h->cl_top && !H[l].planar) || (H[l].planar && h->prm.nu_pre > 0);
+}
+
 // nu smoothing steps on level lv.  The state is in (u, p) when `sw` is false and in (tu, tp)
 // when true; returns where it is afterwards.  The fused float32 Uzawa kernel writes the other
 // buffer pair (ping-pong); the float64 and normal-equation steps work in place and use the other
 // pair as scratch.  With `coarse` given (a planar level), the first step adds the coarse-grid
-// correction P x_c of that coarse level to its staged tiles before it smooths.
+// correction P x_c of that coarse level to its staged tiles before it smooths; with `zero` it starts from zero
+// (a planar level's arrays may then hold anything).
 template <typename T>
-bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw, const Level<T>* coarse = nullptr) {
+bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw, const Level<T>* coarse = nullptr,
+                  bool zero = false) {
     const stokes_params& P = h->prm;
     const bool f32 = sizeof(T) == 4 && P.smoother == STOKES_UZAWA;
     for (int s = 0; s < steps; ++s) {
@@ -272,11 +282,13 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
         } else if constexpr (sizeof(T) == 4) {
             if (h->dom == kDomL) {   // the L: the per-phase kernels (in place), the removed quadrant kept zero
                 launch_uzawa<float>(h->st, lv.n, lv.c, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op,
-                                    0, 0, h->dom);
+                                    0, 0, h->dom, zero && s == 0 && !h->plain);
             } else if (lv.planar) {
                 CoarseCorrection cc;
                 if (coarse && s == 0) cc = CoarseCorrection{coarse->u, coarse->p, coarse->planar};
-                if (launch_uzawa_tma(h->st, lv.n, lv.c, planar_level(h, lv), (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou,
+                PlanarLevel pl = planar_level(h, lv);
+                pl.zero = zero && s == 0 && pl.lists;
+                if (launch_uzawa_tma(h->st, lv.n, lv.c, pl, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou,
                                      op, cc))
                     sw = !sw;
                 else
@@ -286,7 +298,8 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
                 sw = !sw;
             }
         } else {
-            launch_uzawa<T>(h->st, lv.n, lv.c, (T)P.tau, (T)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op, 0, 0, h->dom);
+            launch_uzawa<T>(h->st, lv.n, lv.c, (T)P.tau, (T)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op, 0, 0, h->dom,
+                            zero && s == 0);
         }
         ev_end(h, k);
     }
@@ -425,20 +438,22 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
         return;
     }
     const bool top = l == (int)H.size() - 1;
-    bool sw = smooth_level(h, lv, h->prm.nu_pre, top, false);
+    bool sw = smooth_level(h, lv, h->prm.nu_pre, top, false, (const Level<T>*)nullptr, zero);
     const Level<T>* fused_coarse = nullptr;   // the coarse-grid correction goes into the first post-smoothing step
     T* xu = sw ? lv.tu : lv.u;
     T* xp = sw ? lv.tp : lv.p;
     T* ru = sw ? lv.u : lv.tu;
     T* rp = sw ? lv.p : lv.tp;
     Level<T>& cl = H[l - 1];
+    const bool clear = !ignores_iterate(h, H, l - 1);         // the coarse iterate := 0 with the restriction
+    T *zu = clear ? cl.u : nullptr, *zp = clear ? cl.p : nullptr;
     const int visits = l - 1 == h->clev ? 1 : h->prm.gamma;   // a second exact solve would return the same values
     if constexpr (sizeof(T) == 4) {
         if (lv.planar) {
             // the defect and its restriction in one kernel on the staged tiles (the defect stays on chip)
-            if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, planar_level(h, lv), xu, xp, lv.f, lv.g, cl.f, cl.g, cl.u, cl.p)) {
+            if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, planar_level(h, lv), xu, xp, lv.f, lv.g, cl.f, cl.g, zu, zp)) {
                 launch_residual_planar(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp);
-                launch_restrict_planar(h->st, cl.n, cl.planar, ru, rp, cl.f, cl.g, cl.u, cl.p);
+                launch_restrict_planar(h->st, cl.n, cl.planar, ru, rp, cl.f, cl.g, zu, zp);
             }
             for (int r = 0; r < visits; ++r) mg_cycle(h, H, l - 1, r == 0);
             if (h->fuse_prolong && h->prm.nu_post > 0) fused_coarse = &cl;
@@ -447,7 +462,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
     }
     if (!lv.planar) {
         launch_residual<T, T>(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp, nullptr, nullptr, nullptr, h->dom);
-        launch_restrict<T>(h->st, cl.n, ru, rp, cl.f, cl.g, cl.u, cl.p, h->dom);   // and the coarse iterate := 0
+        launch_restrict<T>(h->st, cl.n, ru, rp, cl.f, cl.g, zu, zp, h->dom);
         for (int r = 0; r < visits; ++r) mg_cycle(h, H, l - 1, r == 0);
         launch_prolong_add<T>(h->st, cl.n, cl.u, cl.p, xu, xp, h->dom);
     }
@@ -494,8 +509,10 @@ void record_step(stokes_handle* h, const LoopCheck& ck = LoopCheck{}) {
     Level<double>& F = h->fin();
     if (h->mixed()) {
         Level<float>& E = h->h32.back();
-        cudaMemsetAsync(E.u, 0, 2 * E.n2 * sizeof(float), h->st);
-        cudaMemsetAsync(E.p, 0, E.n1 * sizeof(float), h->st);
+        if (!ignores_iterate(h, h->h32, h->L - 1)) {
+            cudaMemsetAsync(E.u, 0, 2 * E.n2 * sizeof(float), h->st);
+            cudaMemsetAsync(E.p, 0, E.n1 * sizeof(float), h->st);
+        }
         for (int c = 0; c < h->prm.inner_cycles; ++c) mg_cycle<float>(h, h->h32, h->L - 1, c == 0);
         // x += e, r -= A e (two-float residual, error-free float32 products), r32 = float(r)
         const int k = ev_begin(h, kEvResid);

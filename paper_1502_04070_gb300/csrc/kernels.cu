@@ -169,6 +169,28 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 2) k_uzawa_u(int n, c
     pdl_trigger();
 }
 
+// the same from u = 0, p = 0: uh = tau Ahat^{-1} f
+template <typename T>
+__global__ void __launch_bounds__(NT) k_uzawa_zero(int n, const __grid_constant__ OpCoef<T> c, T tau, const T* __restrict__ f,
+                                                   T* __restrict__ uh, int dom) {
+    pdl_wait();
+    CELL_INDEX
+    if (!active) return;
+    const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
+    const CellNodes cn = cell_nodes_dom(i, j, n, dom);
+    const int cls = stencil_class(i, j, n), ld = 2 * n + 1;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        if (!slot_exists(cn, s)) continue;
+        const size_t k = (size_t)(2 * j + (s >> 1)) * ld + 2 * i + (s & 1);
+        const bool unk = slot_unknown(cn, s);
+        const T ti = tau * c.MIdg[cls][s];
+        uh[k] = unk ? ti * f[k] : T(0);
+        uh[n2 + k] = unk ? ti * f[n2 + k] : T(0);
+    }
+    pdl_trigger();
+}
+
 template <typename T>
 __global__ void __launch_bounds__(NT) k_uzawa_p(int n, const __grid_constant__ OpCoef<T> c, T sigma,
                                                 const T* __restrict__ uh, T* __restrict__ p,
@@ -233,10 +255,11 @@ __global__ void __launch_bounds__(NT) k_uzawa_u2(int n, const __grid_constant__ 
 
 template <typename T>
 void launch_uzawa(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T sigma, T* u, T* p, const T* f,
-                  const T* g, const T* sinv, T* uh, T* dp, int bx, int by, int dom) {
+                  const T* g, const T* sinv, T* uh, T* dp, int bx, int by, int dom, bool zero) {
     const dim3 blk = bx > 0 ? dim3(bx, by) : cells_block(n);
     const dim3 grid((n + 1 + blk.x - 1) / blk.x, (n + 1 + blk.y - 1) / blk.y);
-    launch_pdl(k_uzawa_u<T>, grid, blk, 0, s, n, c, tau, u, p, f, uh, dom);
+    if (zero) launch_pdl(k_uzawa_zero<T>, grid, blk, 0, s, n, c, tau, f, uh, dom);
+    else launch_pdl(k_uzawa_u<T>, grid, blk, 0, s, n, c, tau, u, p, f, uh, dom);
     // dp = 0 where Shat^{-1} = 0: on the L the vertices outside it
     launch_pdl(k_uzawa_p<T>, grid, blk, 0, s, n, c, sigma, uh, p, g, sinv, dp);
     launch_pdl(k_uzawa_u2<T>, grid, blk, 0, s, n, c, tau, uh, dp, u, dom);
@@ -1045,7 +1068,7 @@ void launch_mask_l(cudaStream_t s, int n, double* u, double* p) {
 // ------------------------------------------------------------------------------------------
 #define INST(T)                                                                                         \
     template void launch_uzawa<T>(cudaStream_t, int, const OpCoef<T>&, T, T, T*, T*, const T*, const T*, \
-                                  const T*, T*, T*, int, int, int);                                                 \
+                                  const T*, T*, T*, int, int, int, bool);                                           \
     template void launch_normal_eq<T>(cudaStream_t, int, const OpCoef<T>&, T, T*, T*, const T*, const T*, \
                                       const T*, T*, T*);                                                  \
     template void launch_restrict<T>(cudaStream_t, int, const T*, const T*, T*, T*, T*, T*, int);                 \

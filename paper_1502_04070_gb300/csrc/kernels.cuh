@@ -26,7 +26,8 @@ void launch_residual(cudaStream_t s, int n, const OpCoef<T>& c, const T* u, cons
 //   u  = uh - tau Ahat^{-1} B^T dp
 template <typename T>
 void launch_uzawa(cudaStream_t s, int n, const OpCoef<T>& c, T tau, T sigma, T* u, T* p, const T* f,
-                  const T* g, const T* sinv, T* uh, T* dp, int bx = 0, int by = 0, int dom = kDomSquare);   // bx 0: cells_block(n)
+                  const T* g, const T* sinv, T* uh, T* dp, int bx = 0, int by = 0, int dom = kDomSquare,   // bx 0: cells_block(n)
+                  bool zero = false);   // zero: u and p hold zero, the operator of the first kernel is skipped
 
 // Refinement update (see refine.cu): float32 correction e, float64 iterate x, residual r stored as
 // (hi, lo) float pairs in the 8-byte slots of a float64 array:
@@ -93,6 +94,7 @@ struct alignas(16) MidLists {
 struct PlanarLevel {
     const MidLists* lists = nullptr;
     bool shared = false;
+    bool zero = false;   // the step starts from u = 0, p = 0 whatever the arrays hold (lists given only)
 };
 bool fill_mid_lists(MidLists& q, const OpCoef<float>& c, float tau);   // host; false: a stencil has more entries
 bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau, float sigma,
@@ -119,7 +121,7 @@ bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<f
                               float* u_out, float* p_out, const CoarseCorrection& cc = CoarseCorrection{});
 // r = F - A x on a planar level (N = n) and its restriction (fc, gc) = I^T r to the coarse level
 // (planar or not: pc_planar), with the coarse iterate (uc, pc) set to zero, in one kernel on the
-// tiles of the planar step; the fine defect stays in shared memory.  False (nothing launched) as
+// tiles of the planar step (uc, pc null: the coarse iterate is left alone); the fine defect stays in shared memory.  False (nothing launched) as
 // for launch_uzawa_tma.
 bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& ml,
                          const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc, float* pc);

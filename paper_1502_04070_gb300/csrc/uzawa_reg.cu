@@ -660,12 +660,32 @@ __device__ __forceinline__ void mid_cover(bool col, bool right, int h, int first
     }
     for (int r = m + (((warp - m) % NW) + NW) % NW; r < e; r += NW) row(r);
 }
+// u^{m-1/2} = tau Ahat^{-1} f of a step that starts from u = 0, p = 0 (f is zero at the nodes that are not unknowns);
+// ml given: a tile on a mid-line
+template <class G, int NW>
+__device__ __forceinline__ void zero_phase1(int n, int TY, int i0, int j0, const RegCoef& q, const MidLists* ml, float2* sF) {
+    const int FPL = G::fpl(TY), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cls = orient(i0, j0, n);
+    for (int r = warp; r < TY + 4; r += NW) {
+        const int k = ml ? mid_class(i0 - 2 + lane, j0 - 2 + r, n) : 0;
+        float2* fr = sF + r * G::FW + lane;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const float ti = ml ? __ldg(&ml->ti[k][s]) : q.ti[cls][s > 0];
+            const float2 v = fr[s * FPL];
+            fr[s * FPL] = f2(ti * v.x, ti * v.y);
+        }
+    }
+}
+
 template <class G, bool PLO, int NW>
-__device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const RegCoef& q, const MidLists& ml, float sigma,
+__device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const RegCoef& q, const MidLists& ml, bool zero,
+                                           float sigma,
                                            const float2* sU, float2* sF, const float* sP, float* sG, const float* sS,
                                            float* __restrict__ u_out, float* __restrict__ p_out) {
     const int UPL = G::upl(TY), FPL = G::fpl(TY), lane = threadIdx.x & 31, h = n >> 1;
     const bool col = h >= i0 - 2 && h < i0 + G::TX + 2, right = i0 >= h;
+    if (zero) zero_phase1<G, NW>(n, TY, i0, j0, q, &ml, sF);
+    else
     mid_cover(col, right, h, j0 - 2, TY + 4, NW,
               [&](int cls, int r, int end, int step) {
                   if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n);
@@ -702,7 +722,7 @@ __device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const 
 // the new state of the CTA's cells to (u_out, p_out).
 template <class G, bool PLO, int NW, bool PAIR = false, bool LISTS = false>
 __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
-                                           const MidLists* ml, float tau, float sigma, const float2* sU, float2* sF, const float* sP,
+                                           const MidLists* ml, bool zero, float tau, float sigma, const float2* sU, float2* sF, const float* sP,
                                            float* sG, const float* sS, float* __restrict__ u_out,
                                            float* __restrict__ p_out) {
     constexpr int TX = G::TX;
@@ -715,7 +735,7 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
 
     if constexpr (LISTS) {
         if (!fast) {
-            mid_phases<G, PLO, NW>(n, TY, i0, j0, q, *ml, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+            mid_phases<G, PLO, NW>(n, TY, i0, j0, q, *ml, zero, sigma, sU, sF, sP, sG, sS, u_out, p_out);
             return;
         }
     }
@@ -726,7 +746,9 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
     const QuadLat<G> vhy{sF, FPL, i0 - 2, j0 - 2, true};
 
     // ---- u^{m-1/2} on cells (i0 - 2 + lane, j0 - 2 + r), written over f
-    if (fast && PAIR) {
+    if (LISTS && zero) {
+        zero_phase1<G, NW>(n, TY, i0, j0, q, nullptr, sF);
+    } else if (fast && PAIR) {
         if (inner) {
             if (cls == 0) phase1_pair<G, 0, true>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
             else phase1_pair<G, 1, true>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
@@ -930,7 +952,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
     __syncthreads();
 
 
-    reg_phases<G, false, NW>(n, TY, i0, j0, &c, q, nullptr, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, false, NW>(n, TY, i0, j0, &c, q, nullptr, false, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -989,12 +1011,14 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, i
                  : "memory");
 }
 // the five tiles of the tile at (i0, j0) into L2, for the CTA that will take that tile later
-__device__ __forceinline__ void tma_prefetch_tile(int TY, int i0, int j0, const TmaMaps& maps) {
+__device__ __forceinline__ void tma_prefetch_tile(int TY, int i0, int j0, const TmaMaps& maps, bool from0) {
     using G = TmaTile;
-    tma_prefetch_3d(&maps.u, 2 * (i0 - G::UX), 2 * (j0 - 3), 0);
+    if (!from0) {
+        tma_prefetch_3d(&maps.u, 2 * (i0 - G::UX), 2 * (j0 - 3), 0);
+        tma_prefetch_2d(&maps.p, i0 - G::PX, j0 - 3);
+    }
     tma_prefetch_3d(&maps.f0, 2 * (i0 - 2), j0 - 2, 0);
     tma_prefetch_3d(&maps.f1, 2 * (i0 - 2), j0 - 2, 0);
-    tma_prefetch_2d(&maps.p, i0 - G::PX, j0 - 3);
     tma_prefetch_2d(&maps.g, i0 - G::DX, j0 - 1);
     tma_prefetch_2d(&maps.s, i0 - G::DX, j0 - 1);
 }
@@ -1188,7 +1212,7 @@ template <int NW, int MINB, bool PAIR, bool LISTS>
 __global__ void __launch_bounds__(32 * NW, MINB)
     k_uzawa_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t, const __grid_constant__ RegCoef q,
                 float tau, float sigma, const __grid_constant__ TmaMaps maps, float* __restrict__ u_out,
-                float* __restrict__ p_out, int pf, const float* __restrict__ uc, const float* __restrict__ pc, int pcp) {
+                float* __restrict__ p_out, int pf, const float* __restrict__ uc, const float* __restrict__ pc, int pcp, int zero) {
     using G = TmaTile;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -1208,23 +1232,29 @@ __global__ void __launch_bounds__(32 * NW, MINB)
     __syncthreads();
     pdl_wait();   // the inputs are the previous kernel's outputs
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(G::tx_bytes(TY)) : "memory");
+        const bool from0 = LISTS && zero;   // u = 0, p = 0: their tiles are not read
+        const unsigned bytes = G::tx_bytes(TY) - (from0 ? 8u * 2u * G::upl(TY) + 4u * G::PW * (TY + 6) : 0u);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
         const unsigned du = (unsigned)__cvta_generic_to_shared(sU), df = (unsigned)__cvta_generic_to_shared(sF);
-        tma_3d(du, &maps.u, 2 * (i0 - G::UX), 2 * (j0 - 3), 0, bar);
+        if (!from0) {
+            tma_3d(du, &maps.u, 2 * (i0 - G::UX), 2 * (j0 - 3), 0, bar);
+            tma_2d((unsigned)__cvta_generic_to_shared(sP), &maps.p, i0 - G::PX, j0 - 3, bar);
+        }
         tma_3d(df, &maps.f0, 2 * (i0 - 2), j0 - 2, 0, bar);
         tma_3d(df + 8 * 2 * G::fpl(TY), &maps.f1, 2 * (i0 - 2), j0 - 2, 0, bar);
-        tma_2d((unsigned)__cvta_generic_to_shared(sP), &maps.p, i0 - G::PX, j0 - 3, bar);
         tma_2d((unsigned)__cvta_generic_to_shared(sG), &maps.g, i0 - G::DX, j0 - 1, bar);
         tma_2d((unsigned)__cvta_generic_to_shared(sS), &maps.s, i0 - G::DX, j0 - 1, bar);
         const int ahead = (int)blockIdx.x + pf;
         if (pf > 0 && ahead < (int)gridDim.x) {
             int ac, ar;
             ord.tile(ahead, ac, ar);
-            tma_prefetch_tile(TY, ac * G::TX, ar * TY, maps);
+            tma_prefetch_tile(TY, ac * G::TX, ar * TY, maps, from0);
         }
     }
     // uc, pc given: the step starts from x + P x_c; each thread loads the coarse values of its
     // square while the tiles are in flight
+    if (LISTS && zero)   // the new p is p + dp
+        for (int t = threadIdx.x; t < G::PW * (TY + 6); t += 32 * NW) sP[t] = 0.f;
     const EmbedGrid<G> eg(TY, i0, j0);
     EmbedJob jb;
     if (uc) embed_load(jb, threadIdx.x, eg, n >> 1, uc, pc, pcp != 0);
@@ -1245,7 +1275,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         }
         __syncthreads();
     }
-    reg_phases<G, true, NW, PAIR, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, true, NW, PAIR, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), LISTS && zero, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -1350,7 +1380,7 @@ __device__ __forceinline__ void restrict_sq(const RestrictWeights& wt, int I, in
 // The defect on fine cells and vertices [i0 - 2, i0 + TX) x [j0 - 2, j0 + TY) of the staged tiles
 // (r_u over sF, r_p over sG, whose tile starts at vertex row j0 - 2) and its restriction to the
 // coarse cells [i0 / 2, i0 / 2 + TX / 2) x [j0 / 2, j0 / 2 + TY / 2) of level n / 2 (planar: PC), with
-// the coarse iterate of those cells set to zero.  All threads of the CTA take part.
+// the coarse iterate of those cells set to zero if given.  All threads of the CTA take part.
 template <class G, int NW, bool PC, bool LISTS = false>
 __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
                                                 const MidLists* ml,
@@ -1431,13 +1461,12 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
             if constexpr (PC) {
                 const int o = pl_u(nc, X, Y);
                 *reinterpret_cast<float2*>(fc + o) = v;
-                *reinterpret_cast<float2*>(uc + o) = f2(0.f, 0.f);
+                if (uc) *reinterpret_cast<float2*>(uc + o) = f2(0.f, 0.f);
             } else {
                 const int ld = 2 * nc + 1, o = Y * ld + X;
                 fc[o] = v.x;
                 fc[ld * ld + o] = v.y;
-                uc[o] = 0.f;
-                uc[ld * ld + o] = 0.f;
+                if (uc) uc[o] = uc[ld * ld + o] = 0.f;
             }
         }
         // P1: the fine vertex (2I, 2J), and halves of the fine vertices halfway along the coarse
@@ -1457,7 +1486,7 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
         if (x > 0 && y < nf && orient(I - 1, J, nc) == 1) half += R(x - 1, y + 1);
         const int vi = PC ? J * pl_vpitch(nc) + I : J * (nc + 1) + I;
         gc[vi] = fmaf(0.5f, half, sv);
-        pc[vi] = 0.f;
+        if (pc) pc[vi] = 0.f;
     }
 }
 
@@ -1767,7 +1796,7 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
             const int i0 = (t % cols) * G::TX, j0 = (t / cols) * TY;
             stage_compact(n, TY, i0, j0, j0 - 1, xu, xp, L.f, L.g, L.sinv, sU, sF, sP, sG, sS);
             __syncthreads();
-            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, A.tau, A.sigma, sU, sF, sP, sG,
+            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, false, A.tau, A.sigma, sU, sF, sP, sG,
                                            sS, ou, op);
             __syncthreads();
         }
@@ -2011,10 +2040,12 @@ bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLev
     const dim3 grid(ord.cols * ord.rows), block(32 * NW);
     if (pl.lists)
         launch_pdl(k_uzawa_tma<NW, MINB, PAIR, true>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
-                   tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
+                   tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0,
+                   pl.zero ? 1 : 0);
     else
         launch_pdl(k_uzawa_tma<NW, MINB, PAIR, false>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q, tau,
-                   sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0);
+                   sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0,
+                   pl.zero ? 1 : 0);
     return true;
 }
 
