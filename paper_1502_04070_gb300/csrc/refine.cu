@@ -260,8 +260,10 @@ __device__ __forceinline__ float2 df_sub(float2 a, const DF& b) {
     return renorm(s, __fadd_rn(e, __fsub_rn(a.y, b.lo)));
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 template <bool PL>
-__global__ void __launch_bounds__(NT, 4) k_ir_update_df(int n, const __grid_constant__ OpCoef<float> ch,
+__global__ void __launch_bounds__(NT, 5) k_ir_update_df(int n, const __grid_constant__ OpCoef<float> ch,
                                                      const __grid_constant__ OpCoef<float> cl,
                                                      const __grid_constant__ DFPairCoef cq,
                                                      const float* __restrict__ eu, const float* __restrict__ ep,
@@ -270,9 +272,26 @@ __global__ void __launch_bounds__(NT, 4) k_ir_update_df(int n, const __grid_cons
                                                      float* __restrict__ r32u, float* __restrict__ r32p,
                                                      double* __restrict__ partial, double* __restrict__ wpartial,
                                                      double wscale, int dom, const double* __restrict__ mean) {
-    pdl_wait();
     CELL_INDEX
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
+    // x and r (four fifths of the bytes) on their way to L2 while the windows of e are read and summed: the kernel waits
+    // on loads, and five CTAs of 48 registers per SM leave none to hold them.  h = 1/2048: 421 us without, 357 us with
+    // (363 us with four CTAs of 64 registers; requests a wave of CTAs ahead, for e too, gained nothing).
+    if (active) {
+        const size_t k = (size_t)(2 * j) * (2 * n + 1) + 2 * i, vi = (size_t)j * (n + 1) + i;
+        const size_t up = j < n ? 2 * n + 1 : 0;
+        prefetch_l2(xu + k);
+        prefetch_l2(xu + k + up);
+        prefetch_l2(xu + n2 + k);
+        prefetch_l2(xu + n2 + k + up);
+        prefetch_l2(ru + k);
+        prefetch_l2(ru + k + up);
+        prefetch_l2(ru + n2 + k);
+        prefetch_l2(ru + n2 + k + up);
+        prefetch_l2(xp + vi);
+        prefetch_l2(rp + vi);
+    }
+    pdl_wait();
     float ss = 0.f;
     // (triangles at vertex i) x_p,i of the updated pressure; times wscale = h^2 / 6 per block, the
     // zero-mean projection's numerator sum_i w_i x_p,i (float64 work kept to the additions)
