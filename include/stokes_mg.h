@@ -97,10 +97,10 @@ typedef struct stokes_params {
                           unknowns; entries of u, p, f, g there are ignored on input and zero on output,
                           and the zero-mean pressure is over the L.  It needs the Uzawa smoother,
                           coarse_level = 1 (the L's level 0) and levels >= 2; with STOKES_MIXED its
-                          float32 levels keep the compact layout and the per-phase step; load vectors,
-                          Euler right-hand sides and mass products are square-only (they return
+                          float32 levels follow tma_level as the square's do, the levels below it that no
+                          cluster takes run the per-phase step; load vectors, Euler right-hand sides and mass products are square-only (they return
                           STOKES_ERR_BAD_ARG on an L handle) */
-    int tma_level;     /* STOKES_MIXED with the Uzawa smoother on the unit square: the float32 levels
+    int tma_level;     /* STOKES_MIXED with the Uzawa smoother: the float32 levels
                           k >= tma_level are held in a padded layout whose rows start on 16-byte
                           boundaries and smoothed by a one-kernel step whose tiles arrive by
                           tensor-memory-access box copies (the other levels as set by
@@ -171,7 +171,9 @@ stokes_status stokes_sizes(const stokes_handle* h, int* N, size_t* n_vel, size_t
  * (u, p), followed by the zero-mean projection of p.  Under STOKES_MIXED it is one refinement
  * step: float64 residual, params.inner_cycles float32 cycles on the correction, float64 update; it keeps
  * the float32 order of operations of one launch per phase or step (and of the one-CTA cycle below N = 64),
- * whose rounding its result carries, where the steps of a solve run the faster cluster cycle. */
+ * whose rounding its result carries, where the steps of a solve run the faster cluster cycle.  On the L with
+ * levels >= tma_level it works on compact float32 levels of its own, allocated by the first such call (as do
+ * stokes_smooth_f32 and stokes_residual_restrict_f32). */
 stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double* f, const double* g);
 
 /* Iterates stokes_cycle from the given (u, p) until ||F - A x||_2 <= tol ||F||_2 or max_cycles.

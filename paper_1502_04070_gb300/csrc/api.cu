@@ -156,6 +156,7 @@ struct stokes_handle_t {
     int L = 0;                              // number of levels
     std::vector<Level<double>> h64;         // FP64: all levels; MIXED: finest only
     std::vector<Level<float>> h32;          // MIXED: all levels
+    std::vector<Level<float>> cyc32;        // MIXED on the L: compact ones (make_cycle_levels)
     double* inv = nullptr;                  // level-0 bordered inverse (27 x 27)
     int dom = kDomSquare;                   // the domain: kDomSquare, or kDomL (common.cuh)
     int clev = 0;                           // coarsest level of the iteration (exact solve there)
@@ -247,7 +248,7 @@ stokes_status take_launch_failure(stokes_handle* h, stokes_status st = STOKES_OK
 
 template <typename T>
 PlanarLevel planar_level(const stokes_handle* h, const Level<T>& lv) {
-    return PlanarLevel{h->plain ? nullptr : lv.mid, h->shared};
+    return PlanarLevel{h->plain ? nullptr : lv.mid, h->shared, h->dom};
 }
 
 // Does an iteration on level l that starts from zero (mg_cycle's `zero`) ignore what (u, p) hold?  Then nobody has
@@ -280,7 +281,7 @@ bool smooth_level(stokes_handle* h, Level<T>& lv, int steps, bool timed, bool sw
         if (P.smoother == STOKES_NORMAL_EQ) {
             launch_normal_eq<T>(h->st, lv.n, lv.c, (T)P.tau, xu, xp, lv.f, lv.g, lv.sinv, ou, op);
         } else if constexpr (sizeof(T) == 4) {
-            if (h->dom == kDomL) {   // the L: the per-phase kernels (in place), the removed quadrant kept zero
+            if (h->dom == kDomL && !lv.planar) {   // the L: the per-phase kernels (in place), the removed quadrant kept zero
                 launch_uzawa<float>(h->st, lv.n, lv.c, (float)P.tau, (float)P.sigma, xu, xp, lv.f, lv.g, lv.sinv, ou, op,
                                     0, 0, h->dom, zero && s == 0 && !h->plain);
             } else if (lv.planar) {
@@ -452,6 +453,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
         if (lv.planar) {
             // the defect and its restriction in one kernel on the staged tiles (the defect stays on chip)
             if (!launch_restrict_tma(h->st, lv.n, cl.planar, lv.c, planar_level(h, lv), xu, xp, lv.f, lv.g, cl.f, cl.g, zu, zp)) {
+                if (h->dom != kDomSquare) h->launch_failed = true;   // these know no mask
                 launch_residual_planar(h->st, lv.n, lv.c, xu, xp, lv.f, lv.g, ru, rp);
                 launch_restrict_planar(h->st, cl.n, cl.planar, ru, rp, cl.f, cl.g, zu, zp);
             }
@@ -561,7 +563,8 @@ stokes_status build_graph(stokes_handle* h) { return capture_step(h, &h->step, &
 
 // stokes_cycle on a MIXED handle: its result is one float32 cycle's, rounding included, and nothing after it removes
 // that rounding; it keeps the order of float32 operations it has always had (the one-CTA coarse cycle, per-cell
-// rows on the mid-lines), so that it returns the same values, about half as fast as a step inside a solve.
+// rows on the mid-lines; on the L the compact layout), so that it returns the same values, about half as fast as a step
+// inside a solve.
 stokes_status build_plain_graph(stokes_handle* h) {
     const bool timing = h->timing;
     h->timing = false;
@@ -667,6 +670,37 @@ stokes_status upload_cluster_tables(stokes_handle* h, const std::vector<Level<T>
     return STOKES_OK;
 }
 
+// stokes_cycle of a MIXED handle on the L runs the compact layout on every level (see build_plain_graph), and so do the
+// float32 step and restriction on a caller's arrays: the first such call gives levels that are planar in h32 a compact
+// twin, the others are h32's own.
+void fill_cycle_levels(stokes_handle* h) {
+    for (size_t k = 0; k < h->cyc32.size(); ++k) {
+        Level<float>& lv = h->cyc32[k];
+        if (!h->h32[k].planar) {
+            lv = h->h32[k];
+            continue;
+        }
+        lv.c = h->h32[k].c;
+        launch_schur_diag<float>(h->st, lv.n, make_coef<double>(lv.n, h->prm.beta), lv.sinv, h->dom, 0);
+    }
+}
+stokes_status make_cycle_levels(stokes_handle* h) {
+    if (h->dom != kDomL || !h->has_planar || !h->cyc32.empty()) return STOKES_OK;
+    std::vector<Level<float>> H(h->h32.size());
+    for (size_t k = 0; k < H.size(); ++k) {
+        if (!h->h32[k].planar) continue;
+        const stokes_status s = alloc_level(H[k], (int)k, h->mem);
+        if (s != STOKES_OK) {
+            for (auto& lv : H) h->mem.put(lv.slab);
+            return s;
+        }
+    }
+    h->cyc32.swap(H);
+    fill_cycle_levels(h);
+    CK(cudaGetLastError());
+    return STOKES_OK;
+}
+
 stokes_status rebuild_beta(stokes_handle* h) {
     const double beta = h->prm.beta;
     for (auto& lv : h->h64) {
@@ -688,6 +722,7 @@ stokes_status rebuild_beta(stokes_handle* h) {
         launch_schur_diag<float>(h->st, lv.n, make_coef<double>(lv.n, beta), lv.sinv, h->dom,
                                  lv.planar ? pl_vpitch(lv.n) : 0);
     }
+    fill_cycle_levels(h);
     if (h->cl_top > 0) {
         const stokes_status s = h->mixed() ? upload_cluster_tables(h, h->h32, h->cl_tab32)
                                            : upload_cluster_tables(h, h->h64, h->cl_tab64);
@@ -869,7 +904,7 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
         if ((s = alloc_level(h->h64[0], kfin, h->mem)) != STOKES_OK) return bail(s);
         h->h32.resize(P.levels);
         const int tlev = P.tma_level > 0 ? P.tma_level : kDefaultTmaLevel;
-        const bool tma = P.smoother == STOKES_UZAWA && P.domain == STOKES_UNIT_SQUARE && uzawa_tma_available();
+        const bool tma = P.smoother == STOKES_UZAWA && uzawa_tma_available();
         for (int k = 0; k < P.levels; ++k)
             if ((s = alloc_level(h->h32[k], k, h->mem, tma && k >= tlev)) != STOKES_OK) return bail(s);
         h->has_planar = tma && tlev < P.levels;
@@ -986,9 +1021,14 @@ stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double*
     stokes_status s;
     if ((s = copy_in(h, u, p, f, g)) != STOKES_OK) return s;
     if (h->mixed()) {
+        if ((s = make_cycle_levels(h)) != STOKES_OK) return s;
+        const bool own = !h->cyc32.empty();
+        if (own) h->h32.swap(h->cyc32);
         residual_norm_fin(h);   // float64 residual and the float32 right-hand side of the correction
         h->launches += 2;
-        if ((s = build_plain_graph(h)) != STOKES_OK) return s;
+        s = build_plain_graph(h);
+        if (own) h->h32.swap(h->cyc32);
+        if (s != STOKES_OK) return s;
         CK(cudaGraphLaunch(h->plain_step, h->st));
         h->launches += h->plain_kernels;
     } else {
@@ -1156,7 +1196,10 @@ stokes_status stokes_smooth(stokes_handle* h, double* u, double* p, const double
 stokes_status stokes_smooth_f32(stokes_handle* h, float* u, float* p, const float* f, const float* g, int nu) {
     ApiRange nvtx_range("stokes_smooth_f32");
     if (!h || !u || !p || !f || !g || nu < 0 || !h->mixed()) return STOKES_ERR_BAD_ARG;
-    Level<float> lv = h->h32.back();   // coefficients, diagonals and ping-pong partners of the finest level
+    const stokes_status sc = make_cycle_levels(h);   // the L: on the caller's compact arrays
+    if (sc != STOKES_OK) return sc;
+    // coefficients, diagonals and ping-pong partners of the finest level
+    Level<float> lv = h->cyc32.empty() ? h->h32.back() : h->cyc32.back();
     if (lv.planar) {
         // the caller's compact arrays into the level's own planar buffers, and the result back
         launch_to_planar(h->st, lv.n, u, p, lv.u, lv.p);
@@ -1185,8 +1228,11 @@ stokes_status stokes_residual_restrict_f32(stokes_handle* h, const float* u, con
                                            const float* g, float* fc, float* gc) {
     ApiRange nvtx_range("stokes_residual_restrict_f32");
     if (!h || !u || !p || !f || !g || !fc || !gc || !h->mixed() || h->L < 2) return STOKES_ERR_BAD_ARG;
-    Level<float>& lv = h->h32.back();
-    Level<float>& cl = h->h32[h->L - 2];
+    const stokes_status sc = make_cycle_levels(h);
+    if (sc != STOKES_OK) return sc;
+    std::vector<Level<float>>& H = h->cyc32.empty() ? h->h32 : h->cyc32;
+    Level<float>& lv = H.back();
+    Level<float>& cl = H[h->L - 2];
     if (lv.planar) {
         launch_to_planar(h->st, lv.n, u, p, lv.u, lv.p);
         launch_to_planar(h->st, lv.n, f, g, lv.f, lv.g);
@@ -1354,7 +1400,7 @@ unsigned long long stokes_kernel_launches(const stokes_handle* h) { return h ? h
 // Times the float32 Uzawa step variants on each not-yet-tuned level of h's float32 hierarchy
 // (process-wide choice per level size) and leaves the buffers zero as a fresh handle has them.
 static stokes_status autotune_levels(stokes_handle* h, cudaStream_t st) {
-    // the L's float32 levels run the per-phase step only: nothing to choose
+    // (the L's compact levels run the per-phase step, its planar ones the square's choice)
     if (!h->mixed() || h->prm.smoother != STOKES_UZAWA || h->dom != kDomSquare) return STOKES_OK;
     for (int l = 1; l < (int)h->h32.size(); ++l) {
         Level<float>& lv = h->h32[l];
@@ -1400,6 +1446,7 @@ struct stokes_batch_t {
     bool own_stream = false;
     std::vector<stokes_handle*> inst;
     std::vector<int> body_kernels;      // kernels per loop iteration of each instance
+    std::vector<int> end_kernels;       // kernels before and after its loop
     cudaGraphExec_t exec = nullptr;
     std::vector<const void*> key;       // pointers, tol and max_cycles the graph was built for
     double tol = -1.0;
@@ -1480,6 +1527,7 @@ static stokes_status batch_build(stokes_batch* b, double* const* u, double* cons
     cudaGraph_t top = nullptr;
     CK(cudaGraphCreate(&top, 0));
     b->body_kernels.assign(b->count, 0);
+    b->end_kernels.assign(b->count, 0);
     auto count_kernels = [](cudaGraph_t gr) {
         size_t nn = 0;
         cudaGraphGetNodes(gr, nullptr, &nn);
@@ -1508,6 +1556,7 @@ static stokes_status batch_build(stokes_batch* b, double* const* u, double* cons
         cudaMemsetAsync(b->d_count + i, 0, sizeof(int), st);
         if ((e = cudaStreamEndCapture(st, &gp)) != cudaSuccess) break;
         cudaGraphNode_t np, nc, ne;
+        b->end_kernels[i] = count_kernels(gp);
         e = cudaGraphAddChildGraphNode(&np, top, nullptr, 0, gp);
         cudaGraphDestroy(gp);
         if (e != cudaSuccess) break;
@@ -1542,6 +1591,7 @@ static stokes_status batch_build(stokes_batch* b, double* const* u, double* cons
         launch_batch_store(st, h->scal, b->d_count + i, b->d_res + 3 * i);
         copy_out(h, u[i], p[i]);
         if ((e = cudaStreamEndCapture(st, &ge)) != cudaSuccess) break;
+        b->end_kernels[i] += count_kernels(ge);
         e = cudaGraphAddChildGraphNode(&ne, top, &nc, 1, ge);
         cudaGraphDestroy(ge);
     }
@@ -1580,7 +1630,7 @@ stokes_status stokes_batch_solve(stokes_batch* b, double* const* u, double* cons
         const int steps = (int)b->h_res[3 * i + 2];
         const double nF = std::sqrt(b->h_res[3 * i + 1]);
         double r = std::sqrt(b->h_res[3 * i]);
-        b->launches += 4 + 3 + (unsigned long long)steps * (b->body_kernels[i] + 1);
+        b->launches += (unsigned long long)b->end_kernels[i] + (unsigned long long)steps * b->body_kernels[i];
         int total = steps;
         if (!(r <= tol * nF)) {
             // rare: the true residual misses the tolerance; continue this instance on its own

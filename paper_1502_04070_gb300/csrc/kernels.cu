@@ -37,7 +37,10 @@ bool fuse_prolong_enabled() {
 }
 
 // float64 kernels subtract the products from the right-hand side as they go (their time is the number of float64
-// instructions); the float32 ones keep the order of operations that defines the result of a float32 cycle
+// instructions); the float32 ones keep the order of operations that defines the result of a float32 cycle.  With the
+// structural zeros left out as well: 257 -> 162 float64 instructions per cell and Uzawa step, 193 -> 133 per residual, 288 ->
+// 104 per restriction; at h = 1/2048 k_uzawa_u 1329 -> 1000 us, k_uzawa_p 392 -> 194, k_uzawa_u2 440 -> 239, k_residual 1628 ->
+// 1128, a whole V(3,3) cycle 26.4 -> 15.6 ms
 template <typename T>
 constexpr bool kSubtract = sizeof(T) == 8;
 

@@ -94,6 +94,7 @@ struct alignas(16) MidLists {
 struct PlanarLevel {
     const MidLists* lists = nullptr;
     bool shared = false;
+    int dom = kDomSquare;   // kDomL (lists given only)
     bool zero = false;   // the step starts from u = 0, p = 0 whatever the arrays hold (lists given only)
 };
 bool fill_mid_lists(MidLists& q, const OpCoef<float>& c, float tau);   // host; false: a stencil has more entries

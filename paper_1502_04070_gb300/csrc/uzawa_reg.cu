@@ -120,6 +120,18 @@ constexpr int kRegMaxRows = 24;
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
+// The L-shaped domain on planar levels: lattice nodes with X >= mf and Y >= mf are not unknowns (mf = N, the closed
+// removed quadrant).  Tiles that reach them are not interior and test every node; the
+// vertices inside it need no test, Shat^{-1} and the defect are zero there.  The square: NoMask, no test at all
+// (testing against a bound cost its step 4 % at N = 2048, 14 % at N = 256).  A mixed solve on the L at h = 1/512 takes
+// 15.8 ms with planar levels, 22.9 ms with the three-kernel step on compact ones.
+struct NoMask {};
+struct QuadrantMask {
+    int from;   // N
+};
+__device__ __forceinline__ bool masked(int, int, NoMask) { return false; }
+__device__ __forceinline__ bool masked(int X, int Y, QuadrantMask m) { return X >= m.from && Y >= m.from; }
+
 // 4-byte asynchronous copy global -> shared, zero-filled when !valid (the source is then not read)
 __device__ __forceinline__ void cp4(void* dst, const float* src, bool valid) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -233,9 +245,9 @@ __device__ __forceinline__ float mid_bu(const E2<float>* e, int k, const float2*
     return t;
 }
 // Node s of cell `x` of row r of the u^{m-1/2} region (STEP), or of the defect (r_u over f)
-template <class G, bool STEP>
+template <class G, bool STEP, class MF = NoMask>
 __device__ __forceinline__ void mid_node(const MidLists& ml, int k, int s, const float2* sU, int UPL, const float* sP,
-                                         float2* sF, int FPL, int r, int x, int i0, int j0, int n) {
+                                         float2* sF, int FPL, int r, int x, int i0, int j0, int n, MF mf) {
     const int X = 2 * (i0 - 2 + x) + (s & 1), Y = 2 * (j0 - 2 + r) + (s >> 1);
     const float2* t0 = sU + 2 * (r + 1) * G::UWH + x + G::UX - 2;
     float2* fr = sF + r * G::FW + x + s * FPL;
@@ -254,7 +266,7 @@ __device__ __forceinline__ void mid_node(const MidLists& ml, int k, int s, const
         const float ti = __ldg(&ml.ti[k][s]);
         t = __ffma2_rn(f2(ti, ti), t, t0[(s >> 1) * G::UWH + (s & 1) * UPL]);
     }
-    *fr = interior2(X, Y, n) ? t : f2(0.f, 0.f);
+    *fr = interior2(X, Y, n) && !masked(X, Y, mf) ? t : f2(0.f, 0.f);
 }
 // r_p = g - B u at vertex `x` of row r (over g; that tile starts two rows below the CTA's)
 template <class G>
@@ -272,9 +284,9 @@ __device__ __forceinline__ void mid_dp(const MidLists& ml, const float2* sF, int
     sG[q] = sigma * sS[q] * (mid_bu(ml.B[k], k, sF + (r + 1) * G::FW + x + 1, FPL) - sG[q]);
 }
 // the new u at node s (and p, with node 0) of cell `x` of row r
-template <class G, bool PLO>
+template <class G, bool PLO, class MF = NoMask>
 __device__ __forceinline__ void mid_out(const MidLists& ml, int s, const float2* sF, int FPL, const float* sG, const float* sP,
-                                        int r, int x, int i0, int j0, int n, float* __restrict__ u_out,
+                                        int r, int x, int i0, int j0, int n, MF mf, float* __restrict__ u_out,
                                         float* __restrict__ p_out) {
     const int ci = i0 + x, cj = j0 + r;
     if (ci > n || cj > n) return;
@@ -286,7 +298,7 @@ __device__ __forceinline__ void mid_out(const MidLists& ml, int s, const float2*
             const float ti = __ldg(&ml.ti[k][s]);
             o = __ffma2_rn(f2(-ti, -ti), mid_sum_bt(ml.BT[k] + 4 * (s - 1), dp), o);
         }
-        store_node<PLO>(u_out, n, X, Y, interior2(X, Y, n) ? o : f2(0.f, 0.f));
+        store_node<PLO>(u_out, n, X, Y, interior2(X, Y, n) && !masked(X, Y, mf) ? o : f2(0.f, 0.f));
     }
     if (s == 0) p_out[vert_at<PLO>(n, ci, cj)] = sP[(r + 3) * G::PW + x + G::PX] + dp[0];
 }
@@ -359,9 +371,10 @@ __device__ __forceinline__ void load_coef(const RegCoef& q, float2 (&a)[kGroups]
     }
 }
 
-template <class G, int C, bool INNER>
+template <class G, int C, bool INNER, class MF = NoMask>
 __device__ __forceinline__ void phase1_fast(const RegCoef& q, const float2* sU, int UPL, const float* sP, float2* sF,
-                                           int FPL, int r0, int rb, int rs, int lane, int i0, int j0, int n) {
+                                           int FPL, int r0, int rb, int rs, int lane, int i0, int j0, int n,
+                                           MF mf = MF{}) {
     float2 a[kGroups];
     load_coef<C>(q, a);
     const float ti0 = q.ti[C][0], ti1 = q.ti[C][1];
@@ -395,7 +408,7 @@ __device__ __forceinline__ void phase1_fast(const RegCoef& q, const float2* sU, 
             if (s > 0) t = __ffma2_rn(mb, bt[s], t);
             const float2 h = __ffma2_rn(f2(ti, ti), t, ctr[s]);
             if constexpr (INNER) fr[s * FPL] = h;
-            else fr[s * FPL] = unk[s] ? h : f2(0.f, 0.f);
+            else fr[s * FPL] = unk[s] && !masked(2 * (i0 - 2 + lane) + (s & 1), 2 * (j0 - 2 + r) + (s >> 1), mf) ? h : f2(0.f, 0.f);
         }
     }
 }
@@ -414,10 +427,11 @@ __device__ __forceinline__ void phase2_fast(const RegCoef& q, const float2* sF, 
     }
 }
 
-template <class G, bool PLO, int C, bool INNER>
+template <class G, bool PLO, int C, bool INNER, class MF = NoMask>
 __device__ __forceinline__ void phase3_fast(const RegCoef& q, const float2* sF, int FPL, const float* sG,
                                             const float* sP, int r0, int rb, int rs, int lane, int i0,
-                                            int j0, int n, float* __restrict__ u_out, float* __restrict__ p_out) {
+                                            int j0, int n, float* __restrict__ u_out, float* __restrict__ p_out,
+                                            MF mf = MF{}) {
     const float nb1 = -q.ti[C][1] * q.b;
     for (int r = r0; r < rb; r += rs) {
         if (lane >= G::TX) break;
@@ -441,7 +455,7 @@ __device__ __forceinline__ void phase3_fast(const RegCoef& q, const float2* sF, 
             for (int s = 0; s < 4; ++s) {
                 if (!slot_exists(cn, s)) continue;
                 store_node<PLO>(u_out, n, 2 * ci + (s & 1), 2 * cj + (s >> 1),
-                                slot_unknown(cn, s) ? o[s] : f2(0.f, 0.f));
+                                slot_unknown(cn, s) && !masked(2 * ci + (s & 1), 2 * cj + (s >> 1), mf) ? o[s] : f2(0.f, 0.f));
             }
         }
         p_out[vert_at<PLO>(n, ci, cj)] = sP[(r + 3) * G::PW + lane + G::PX] + sG[(r + 1) * G::DW + lane + G::DX];
@@ -540,10 +554,10 @@ __device__ __forceinline__ void b_pair_rows(const float2* f0, int fpl, float& ac
 }
 
 // u^{m-1/2} of the cells of row r from their A and B^T rows (written over f)
-template <class G, bool INNER>
+template <class G, bool INNER, class MF = NoMask>
 __device__ __forceinline__ void u_half_row(const float2 (&au)[4], const float2 (&ctr)[4], const float2 (&bt)[4],
                                            float ti0, float ti1, float2 mb, float2* sF, int FPL, int r, int lane,
-                                           int i0, int j0, int n) {
+                                           int i0, int j0, int n, MF mf) {
     bool unk[4] = {true, true, true, true};
     if constexpr (!INNER) {
         const int ci = i0 - 2 + lane, cj = j0 - 2 + r;
@@ -563,13 +577,14 @@ __device__ __forceinline__ void u_half_row(const float2 (&au)[4], const float2 (
         if (s > 0) t = __ffma2_rn(mb, bt[s], t);
         const float2 h = __ffma2_rn(f2(ti, ti), t, ctr[s]);
         if constexpr (INNER) fr[s * FPL] = h;
-        else fr[s * FPL] = unk[s] ? h : f2(0.f, 0.f);
+        else fr[s * FPL] = unk[s] && !masked(2 * (i0 - 2 + lane) + (s & 1), 2 * (j0 - 2 + r) + (s >> 1), mf) ? h : f2(0.f, 0.f);
     }
 }
 
-template <class G, int C, bool INNER>
+template <class G, int C, bool INNER, class MF = NoMask>
 __device__ __forceinline__ void phase1_pair(const RegCoef& q, const float2* sU, int UPL, const float* sP, float2* sF,
-                                           int FPL, int TY, int NW, int warp, int lane, int i0, int j0, int n) {
+                                           int FPL, int TY, int NW, int warp, int lane, int i0, int j0, int n,
+                                           MF mf = MF{}) {
     float2 a[kGroups];
     load_coef<C>(q, a);
     const float ti0 = q.ti[C][0], ti1 = q.ti[C][1];
@@ -582,8 +597,8 @@ __device__ __forceinline__ void phase1_pair(const RegCoef& q, const float2* sU, 
         for (int s = 0; s < 4; ++s) auA[s] = ctrA[s] = btA[s] = auB[s] = ctrB[s] = btB[s] = f2(0.f, 0.f);
         a_pair_rows<C, G::UWH>(a, t0, t1, auA, ctrA, auB, ctrB, std::make_integer_sequence<int, 35>{});
         bt_pair_rows<C, G::PW>(sP + (r + 1) * G::PW + lane + G::PX - 2, btA, btB, std::make_integer_sequence<int, 12>{});
-        u_half_row<G, INNER>(auA, ctrA, btA, ti0, ti1, mb, sF, FPL, r, lane, i0, j0, n);
-        u_half_row<G, INNER>(auB, ctrB, btB, ti0, ti1, mb, sF, FPL, r + 1, lane, i0, j0, n);
+        u_half_row<G, INNER>(auA, ctrA, btA, ti0, ti1, mb, sF, FPL, r, lane, i0, j0, n, mf);
+        u_half_row<G, INNER>(auB, ctrB, btB, ti0, ti1, mb, sF, FPL, r + 1, lane, i0, j0, n, mf);
     }
 }
 
@@ -603,10 +618,11 @@ __device__ __forceinline__ void phase2_pair(const RegCoef& q, const float2* sF, 
 }
 
 // the new (u, p) of the cells of row r from their B^T dp rows
-template <class G, bool PLO, bool INNER>
+template <class G, bool PLO, bool INNER, class MF = NoMask>
 __device__ __forceinline__ void uzawa_out_row(const float2 (&bt)[4], float nb1, const float2* sF, int FPL,
                                               const float* sG, const float* sP, int r, int lane, int i0, int j0,
-                                              int n, float* __restrict__ u_out, float* __restrict__ p_out) {
+                                              int n, float* __restrict__ u_out, float* __restrict__ p_out,
+                                            MF mf) {
     const int ci = i0 + lane, cj = j0 + r;
     if (!INNER && (ci > n || cj > n)) return;
     const float2* hr = sF + (r + 2) * G::FW + lane + 2;
@@ -622,16 +638,18 @@ __device__ __forceinline__ void uzawa_out_row(const float2 (&bt)[4], float nb1, 
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             if (!slot_exists(cn, s)) continue;
-            store_node<PLO>(u_out, n, 2 * ci + (s & 1), 2 * cj + (s >> 1), slot_unknown(cn, s) ? o[s] : f2(0.f, 0.f));
+            store_node<PLO>(u_out, n, 2 * ci + (s & 1), 2 * cj + (s >> 1),
+                            slot_unknown(cn, s) && !masked(2 * ci + (s & 1), 2 * cj + (s >> 1), mf) ? o[s] : f2(0.f, 0.f));
         }
     }
     p_out[vert_at<PLO>(n, ci, cj)] = sP[(r + 3) * G::PW + lane + G::PX] + sG[(r + 1) * G::DW + lane + G::DX];
 }
 
-template <class G, bool PLO, int C, bool INNER>
+template <class G, bool PLO, int C, bool INNER, class MF = NoMask>
 __device__ __forceinline__ void phase3_pair(const RegCoef& q, const float2* sF, int FPL, const float* sG,
                                             const float* sP, int TY, int NW, int warp, int lane, int i0, int j0,
-                                            int n, float* __restrict__ u_out, float* __restrict__ p_out) {
+                                            int n, float* __restrict__ u_out, float* __restrict__ p_out,
+                                            MF mf = MF{}) {
     const float nb1 = -q.ti[C][1] * q.b;
     for (int r = 2 * warp; r < TY; r += 2 * NW) {
         if (lane >= G::TX) break;
@@ -639,8 +657,8 @@ __device__ __forceinline__ void phase3_pair(const RegCoef& q, const float2* sF, 
 #pragma unroll
         for (int s = 0; s < 4; ++s) btA[s] = btB[s] = f2(0.f, 0.f);
         bt_pair_rows<C, G::DW>(sG + (r + 1) * G::DW + lane + G::DX, btA, btB, std::make_integer_sequence<int, 12>{});
-        uzawa_out_row<G, PLO, INNER>(btA, nb1, sF, FPL, sG, sP, r, lane, i0, j0, n, u_out, p_out);
-        uzawa_out_row<G, PLO, INNER>(btB, nb1, sF, FPL, sG, sP, r + 1, lane, i0, j0, n, u_out, p_out);
+        uzawa_out_row<G, PLO, INNER>(btA, nb1, sF, FPL, sG, sP, r, lane, i0, j0, n, u_out, p_out, mf);
+        uzawa_out_row<G, PLO, INNER>(btB, nb1, sF, FPL, sG, sP, r + 1, lane, i0, j0, n, u_out, p_out, mf);
     }
 }
 
@@ -677,9 +695,9 @@ __device__ __forceinline__ void zero_phase1(int n, int TY, int i0, int j0, const
     }
 }
 
-template <class G, bool PLO, int NW>
+template <class G, bool PLO, int NW, class MF = NoMask>
 __device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const RegCoef& q, const MidLists& ml, bool zero,
-                                           float sigma,
+                                           MF mf, float sigma,
                                            const float2* sU, float2* sF, const float* sP, float* sG, const float* sS,
                                            float* __restrict__ u_out, float* __restrict__ p_out) {
     const int UPL = G::upl(TY), FPL = G::fpl(TY), lane = threadIdx.x & 31, h = n >> 1;
@@ -688,13 +706,13 @@ __device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const 
     else
     mid_cover(col, right, h, j0 - 2, TY + 4, NW,
               [&](int cls, int r, int end, int step) {
-                  if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n);
-                  else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n);
+                  if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n, mf);
+                  else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n, mf);
               },
               [&](int r) {
                   const int k = mid_class(i0 - 2 + lane, j0 - 2 + r, n);
 #pragma unroll
-                  for (int s = 0; s < 4; ++s) mid_node<G, true>(ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n);
+                  for (int s = 0; s < 4; ++s) mid_node<G, true>(ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n, mf);
               });
     __syncthreads();
     mid_cover(col, right, h, j0 - 1, TY + 2, NW,
@@ -708,21 +726,21 @@ __device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const 
     __syncthreads();
     mid_cover(col, right, h, j0, TY, NW,
               [&](int cls, int r, int end, int step) {
-                  if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, r, end, step, lane, i0, j0, n, u_out, p_out);
-                  else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, r, end, step, lane, i0, j0, n, u_out, p_out);
+                  if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, r, end, step, lane, i0, j0, n, u_out, p_out, mf);
+                  else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, r, end, step, lane, i0, j0, n, u_out, p_out, mf);
               },
               [&](int r) {
                   if (lane < G::TX)
 #pragma unroll
-                      for (int s = 0; s < 4; ++s) mid_out<G, PLO>(ml, s, sF, FPL, sG, sP, r, lane, i0, j0, n, u_out, p_out);
+                      for (int s = 0; s < 4; ++s) mid_out<G, PLO>(ml, s, sF, FPL, sG, sP, r, lane, i0, j0, n, mf, u_out, p_out);
               });
 }
 
 // The three phases of the step on the staged tiles (sU, sP, sF = f, sG = g, sS = Shat^{-1}); writes
 // the new state of the CTA's cells to (u_out, p_out).
-template <class G, bool PLO, int NW, bool PAIR = false, bool LISTS = false>
+template <class G, bool PLO, int NW, bool PAIR = false, bool LISTS = false, class MF = NoMask>
 __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
-                                           const MidLists* ml, bool zero, float tau, float sigma, const float2* sU, float2* sF, const float* sP,
+                                           const MidLists* ml, bool zero, MF mf, float tau, float sigma, const float2* sU, float2* sF, const float* sP,
                                            float* sG, const float* sS, float* __restrict__ u_out,
                                            float* __restrict__ p_out) {
     constexpr int TX = G::TX;
@@ -730,12 +748,13 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int h = n >> 1;
     const bool fast = (h < i0 - 2 || h >= i0 + TX + 2) && (h < j0 - 2 || h >= j0 + TY + 2);
-    const bool inner = fast && i0 >= 4 && j0 >= 4 && i0 + TX + 3 <= n && j0 + TY + 3 <= n;
+    const bool inner = fast && i0 >= 4 && j0 >= 4 && i0 + TX + 3 <= n && j0 + TY + 3 <= n &&
+                       !masked(2 * (i0 + TX + 3), 2 * (j0 + TY + 3), mf);
     const int cls = orient(i0, j0, n);
 
     if constexpr (LISTS) {
         if (!fast) {
-            mid_phases<G, PLO, NW>(n, TY, i0, j0, q, *ml, zero, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+            mid_phases<G, PLO, NW>(n, TY, i0, j0, q, *ml, zero, mf, sigma, sU, sF, sP, sG, sS, u_out, p_out);
             return;
         }
     }
@@ -753,16 +772,16 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
             if (cls == 0) phase1_pair<G, 0, true>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
             else phase1_pair<G, 1, true>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
         } else {
-            if (cls == 0) phase1_pair<G, 0, false>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
-            else phase1_pair<G, 1, false>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n);
+            if (cls == 0) phase1_pair<G, 0, false>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n, mf);
+            else phase1_pair<G, 1, false>(q, sU, UPL, sP, sF, FPL, TY, NW, warp, lane, i0, j0, n, mf);
         }
     } else if (fast) {
         if (inner) {
             if (cls == 0) phase1_fast<G, 0, true>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
             else phase1_fast<G, 1, true>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
         } else {
-            if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
-            else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n);
+            if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n, mf);
+            else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, warp, TY + 4, NW, lane, i0, j0, n, mf);
         }
     } else if constexpr (!LISTS) {
         for (int r = warp; r < TY + 4; r += NW) {
@@ -819,16 +838,16 @@ __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const 
             if (cls == 0) phase3_pair<G, PLO, 0, true>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
             else phase3_pair<G, PLO, 1, true>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
         } else {
-            if (cls == 0) phase3_pair<G, PLO, 0, false>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
-            else phase3_pair<G, PLO, 1, false>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out);
+            if (cls == 0) phase3_pair<G, PLO, 0, false>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out, mf);
+            else phase3_pair<G, PLO, 1, false>(q, sF, FPL, sG, sP, TY, NW, warp, lane, i0, j0, n, u_out, p_out, mf);
         }
     } else if (fast) {
         if (inner) {
             if (cls == 0) phase3_fast<G, PLO, 0, true>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
             else phase3_fast<G, PLO, 1, true>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
         } else {
-            if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
-            else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out);
+            if (cls == 0) phase3_fast<G, PLO, 0, false>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out, mf);
+            else phase3_fast<G, PLO, 1, false>(q, sF, FPL, sG, sP, warp, TY, NW, lane, i0, j0, n, u_out, p_out, mf);
         }
     } else if constexpr (!LISTS) {
         const SVert<float, G::DW> vd{sG, i0 - G::DX, j0 - 1};
@@ -952,7 +971,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
     __syncthreads();
 
 
-    reg_phases<G, false, NW>(n, TY, i0, j0, &c, q, nullptr, false, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, false, NW>(n, TY, i0, j0, &c, q, nullptr, false, NoMask{}, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -1143,14 +1162,15 @@ __device__ __forceinline__ void embed_load(EmbedJob& jb, int t, const EmbedGrid<
 
 // the job's fine points added to the tiles: the lattice points strictly inside the level and the
 // tile's rows, and the vertices of the level inside the p tile
-template <class G, int CH>
-__device__ __forceinline__ void embed_apply(const EmbedJob& jb, int n, int TY, int i0, int j0, float2* sU, float* sP) {
+template <class G, int CH, class MF = NoMask>
+__device__ __forceinline__ void embed_apply(const EmbedJob& jb, int n, int TY, int i0, int j0, MF mf, float2* sU, float* sP) {
     if (jb.I < 0) return;
     const int nc = n >> 1, I = jb.I, J = jb.J, UPL = G::upl(TY);
     const int pxlo = i0 - G::PX, pylo = j0 - 3;
     // rows [2J, 2J + 2) of vertices (and so [4J, 4J + 4) of lattice points) inside the tiles, and the
     // square strictly inside the level: every point of it is corrected
-    if (I > 0 && J > 0 && I < nc && J < nc && 2 * J >= pylo && 2 * J + 2 <= pylo + TY + 6) {
+    // (on the L the vertices strictly inside the removed quadrant stay zero; its nodes get nothing from its squares)
+    if (I > 0 && J > 0 && I < nc && J < nc && 2 * J >= pylo && 2 * J + 2 <= pylo + TY + 6 && !masked(4 * I + 1, 4 * J + 1, mf)) {
         const int base = (4 * J - 2 * pylo) * G::UWH + ((4 * I - 2 * (i0 - G::UX)) >> 1);
         const int o = orient(I, J, nc);
         if (o == 0) embed_square_full<G, 0, CH>(jb.z, sU + base, sU + base + UPL);
@@ -1182,7 +1202,7 @@ __device__ __forceinline__ void embed_apply(const EmbedJob& jb, int n, int TY, i
     }
     // P1: injection at the coarse vertex, averages halfway along the coarse edges from it
     auto addp = [&](int x, int y, float v) {
-        if (x < pxlo || x >= pxlo + G::PW || y < pylo || y >= pylo + TY + 6 || x > n || y > n) return;
+        if (x < pxlo || x >= pxlo + G::PW || y < pylo || y >= pylo + TY + 6 || x > n || y > n || masked(2 * x - 1, 2 * y - 1, mf)) return;
         sP[(y - pylo) * G::PW + (x - pxlo)] += v;
     };
     addp(2 * I, 2 * J, jb.p00);
@@ -1208,11 +1228,14 @@ struct RowTables<false> {
 
 // pf > 0: also prefetch into L2 the tiles of tile blockIdx.x + pf (about one wave of resident CTAs
 // ahead), so that the CTA that takes it finds its tiles in L2
-template <int NW, int MINB, bool PAIR, bool LISTS>
+// ZERO: the step starts from u = 0, p = 0 and does not read them (a kernel of its own: as a run-time flag it cost the
+// other steps registers, 3 % at N = 2048).  20 instead of 28 values per cell to move, and no first row pass over u: a
+// solve at h = 1/2048 51.1 -> 50.1 ms, a forward and adjoint solve at h = 1/1024 60.9 -> 58.2 ms
+template <int NW, int MINB, bool PAIR, bool LISTS, class MF, bool ZERO = false>
 __global__ void __launch_bounds__(32 * NW, MINB)
     k_uzawa_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t, const __grid_constant__ RegCoef q,
                 float tau, float sigma, const __grid_constant__ TmaMaps maps, float* __restrict__ u_out,
-                float* __restrict__ p_out, int pf, const float* __restrict__ uc, const float* __restrict__ pc, int pcp, int zero) {
+                float* __restrict__ p_out, int pf, const float* __restrict__ uc, const float* __restrict__ pc, int pcp, MF mf) {
     using G = TmaTile;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -1232,11 +1255,10 @@ __global__ void __launch_bounds__(32 * NW, MINB)
     __syncthreads();
     pdl_wait();   // the inputs are the previous kernel's outputs
     if (threadIdx.x == 0) {
-        const bool from0 = LISTS && zero;   // u = 0, p = 0: their tiles are not read
-        const unsigned bytes = G::tx_bytes(TY) - (from0 ? 8u * 2u * G::upl(TY) + 4u * G::PW * (TY + 6) : 0u);
+        const unsigned bytes = G::tx_bytes(TY) - (ZERO ? 8u * 2u * G::upl(TY) + 4u * G::PW * (TY + 6) : 0u);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
         const unsigned du = (unsigned)__cvta_generic_to_shared(sU), df = (unsigned)__cvta_generic_to_shared(sF);
-        if (!from0) {
+        if (!ZERO) {
             tma_3d(du, &maps.u, 2 * (i0 - G::UX), 2 * (j0 - 3), 0, bar);
             tma_2d((unsigned)__cvta_generic_to_shared(sP), &maps.p, i0 - G::PX, j0 - 3, bar);
         }
@@ -1248,12 +1270,12 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         if (pf > 0 && ahead < (int)gridDim.x) {
             int ac, ar;
             ord.tile(ahead, ac, ar);
-            tma_prefetch_tile(TY, ac * G::TX, ar * TY, maps, from0);
+            tma_prefetch_tile(TY, ac * G::TX, ar * TY, maps, ZERO);
         }
     }
     // uc, pc given: the step starts from x + P x_c; each thread loads the coarse values of its
     // square while the tiles are in flight
-    if (LISTS && zero)   // the new p is p + dp
+    if (ZERO)   // the new p is p + dp
         for (int t = threadIdx.x; t < G::PW * (TY + 6); t += 32 * NW) sP[t] = 0.f;
     const EmbedGrid<G> eg(TY, i0, j0);
     EmbedJob jb;
@@ -1268,14 +1290,14 @@ __global__ void __launch_bounds__(32 * NW, MINB)
     }
     if (uc) {
         constexpr int CH = MINB >= 4 ? 8 : 16;   // points corrected at a time (registers)
-        embed_apply<G, CH>(jb, n, TY, i0, j0, sU, sP);
+        embed_apply<G, CH>(jb, n, TY, i0, j0, mf, sU, sP);
         for (int t = threadIdx.x + 32 * NW; t < eg.count; t += 32 * NW) {   // tiles above kEmbedMaxRows only
             embed_load(jb, t, eg, n >> 1, uc, pc, pcp != 0);
-            embed_apply<G, CH>(jb, n, TY, i0, j0, sU, sP);
+            embed_apply<G, CH>(jb, n, TY, i0, j0, mf, sU, sP);
         }
         __syncthreads();
     }
-    reg_phases<G, true, NW, PAIR, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), LISTS && zero, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
+    reg_phases<G, true, NW, PAIR, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), ZERO, mf, tau, sigma, sU, sF, sP, sG, sS, u_out, p_out);
     pdl_trigger();
 }
 
@@ -1312,10 +1334,10 @@ __device__ __forceinline__ float bu_row(const float2* t0, const float2* t1, std:
 }
 
 // the defect on cells and vertices (i0 - 2 + lane, j0 - 2 + r), r < TY + 2, fast path (class C)
-template <class G, int C>
+template <class G, int C, class MF = NoMask>
 __device__ __forceinline__ void defect_fast(const RegCoef& q, const float2* sU, int UPL, const float* sP, float2* sF,
                                            int FPL, float* sG, int r0, int rb, int rs, int lane, int i0,
-                                           int j0, int n) {
+                                           int j0, int n, MF mf = MF{}) {
     float2 a[kGroups];
     load_coef<C>(q, a);
     const float2 mb = f2(-q.b, -q.b);
@@ -1339,7 +1361,7 @@ __device__ __forceinline__ void defect_fast(const RegCoef& q, const float2* sU, 
             const float2 fs = fr[s * FPL];
             float2 t = f2(fs.x - au[s].x, fs.y - au[s].y);
             if (s > 0) t = __ffma2_rn(mb, bt[s], t);
-            fr[s * FPL] = unk[s] ? t : f2(0.f, 0.f);
+            fr[s * FPL] = unk[s] && !masked(2 * ci + (s & 1), 2 * cj + (s >> 1), mf) ? t : f2(0.f, 0.f);
         }
         if (lane < G::DN) {
             const int k = r * G::DW + lane + G::DX - 2;
@@ -1381,9 +1403,9 @@ __device__ __forceinline__ void restrict_sq(const RestrictWeights& wt, int I, in
 // (r_u over sF, r_p over sG, whose tile starts at vertex row j0 - 2) and its restriction to the
 // coarse cells [i0 / 2, i0 / 2 + TX / 2) x [j0 / 2, j0 / 2 + TY / 2) of level n / 2 (planar: PC), with
 // the coarse iterate of those cells set to zero if given.  All threads of the CTA take part.
-template <class G, int NW, bool PC, bool LISTS = false>
+template <class G, int NW, bool PC, bool LISTS = false, class MF = NoMask>
 __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
-                                                const MidLists* ml,
+                                                const MidLists* ml, MF mf,
                                                 const RestrictWeights& wt, const float2* sU, float2* sF,
                                                 const float* sP, float* sG, float* __restrict__ fc,
                                                 float* __restrict__ gc, float* __restrict__ uc,
@@ -1395,18 +1417,18 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
     const int h = n >> 1;
     const bool fast = (h < i0 - 2 || h >= i0 + TX) && (h < j0 - 2 || h >= j0 + TY);
     if (fast) {
-        if (orient(i0, j0, n) == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, warp, TY + 2, NW, lane, i0, j0, n);
-        else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, warp, TY + 2, NW, lane, i0, j0, n);
+        if (orient(i0, j0, n) == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, warp, TY + 2, NW, lane, i0, j0, n, mf);
+        else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, warp, TY + 2, NW, lane, i0, j0, n, mf);
     } else if constexpr (LISTS) {
         mid_cover(h >= i0 - 2 && h < i0 + TX, i0 >= h, h, j0 - 2, TY + 2, NW,
                   [&](int cls, int r, int end, int step) {
-                      if (cls == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, r, end, step, lane, i0, j0, n);
-                      else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, r, end, step, lane, i0, j0, n);
+                      if (cls == 0) defect_fast<G, 0>(q, sU, UPL, sP, sF, FPL, sG, r, end, step, lane, i0, j0, n, mf);
+                      else defect_fast<G, 1>(q, sU, UPL, sP, sF, FPL, sG, r, end, step, lane, i0, j0, n, mf);
                   },
                   [&](int r) {
                       const int k = mid_class(i0 - 2 + lane, j0 - 2 + r, n);
 #pragma unroll
-                      for (int s = 0; s < 4; ++s) mid_node<G, false>(*ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n);
+                      for (int s = 0; s < 4; ++s) mid_node<G, false>(*ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n, mf);
                       if (lane < G::DN) mid_defect_p<G>(*ml, k, sU, UPL, sG, r, lane, i0, j0, n);
                   });
     } else {
@@ -1457,7 +1479,7 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
         for (int s = 0; s < 4; ++s) {
             if (!slot_exists(cn, s)) continue;
             const int X = 2 * I + (s & 1), Y = 2 * J + (s >> 1);
-            const float2 v = slot_unknown(cn, s) ? acc[s] : f2(0.f, 0.f);
+            const float2 v = slot_unknown(cn, s) && !masked(2 * X, 2 * Y, mf) ? acc[s] : f2(0.f, 0.f);
             if constexpr (PC) {
                 const int o = pl_u(nc, X, Y);
                 *reinterpret_cast<float2*>(fc + o) = v;
@@ -1490,11 +1512,11 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
     }
 }
 
-template <int NW, int MINB, bool PC, bool LISTS>
+template <int NW, int MINB, bool PC, bool LISTS, class MF>
 __global__ void __launch_bounds__(32 * NW, MINB)
     k_restrict_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t, const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
                    const __grid_constant__ TmaMaps maps, float* __restrict__ fc, float* __restrict__ gc,
-                   float* __restrict__ uc, float* __restrict__ pc) {
+                   float* __restrict__ uc, float* __restrict__ pc, MF mf) {
     using G = TmaTile;
     constexpr int TX = G::TX;
     extern __shared__ unsigned char smem_raw[];
@@ -1532,7 +1554,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
         }
         return;
     }
-    defect_restrict<G, NW, PC, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), wt, sU, sF, sP, sG, fc, gc, uc, pc);
+    defect_restrict<G, NW, PC, LISTS>(n, TY, i0, j0, t.op(), q, t.lists(), mf, wt, sU, sF, sP, sG, fc, gc, uc, pc);
     pdl_trigger();
 }
 
@@ -1796,7 +1818,7 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
             const int i0 = (t % cols) * G::TX, j0 = (t / cols) * TY;
             stage_compact(n, TY, i0, j0, j0 - 1, xu, xp, L.f, L.g, L.sinv, sU, sF, sP, sG, sS);
             __syncthreads();
-            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, false, A.tau, A.sigma, sU, sF, sP, sG,
+            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, false, NoMask{}, A.tau, A.sigma, sU, sF, sP, sG,
                                            sS, ou, op);
             __syncthreads();
         }
@@ -1825,7 +1847,7 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
                     stage_compact(n, TY, i0, j0, j0 - 2, sw[l] ? L.tu : L.u, sw[l] ? L.tp : L.p, L.f, L.g, nullptr, sU,
                                   sF, sP, sG, sS);
                     __syncthreads();
-                    defect_restrict<G, kSmallNW, false>(n, TY, i0, j0, &sc[l - A.clev - 1], A.q[l], nullptr, A.wt, sU, sF, sP, sG,
+                    defect_restrict<G, kSmallNW, false>(n, TY, i0, j0, &sc[l - A.clev - 1], A.q[l], nullptr, NoMask{}, A.wt, sU, sF, sP, sG,
                                                         C.f, C.g, C.u, C.p);
                     __syncthreads();
                 }
@@ -1880,10 +1902,10 @@ cudaError_t reg_smem_attr() {
 }
 template <int NW, int MINB, bool PAIR = false>
 cudaError_t tma_smem_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR, false, NoMask>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)TmaTile::bytes(kRegMaxRows));
     return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR, true>,
+                            : cudaFuncSetAttribute(k_uzawa_tma<NW, MINB, PAIR, true, NoMask>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TmaTile::bytes(kRegMaxRows));
 }
 
@@ -1931,10 +1953,13 @@ int tile_rows(int n, K k, int nthreads, int minb, int* cache, bool even = false,
 
 template <bool PC>
 cudaError_t rt_smem_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, false, NoMask>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)TmaTile::bytes(kRegMaxRows));
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (e != cudaSuccess) return e;
+    const cudaError_t l = cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, true, QuadrantMask>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TmaTile::bytes(kRegMaxRows));
+    return l != cudaSuccess ? l
+                            : cudaFuncSetAttribute(k_restrict_tma<8, 3, PC, true, NoMask>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)TmaTile::bytes(kRegMaxRows));
 }
 
@@ -1946,8 +1971,8 @@ int reg_rows(int n) {
 template <int NW, int MINB, bool PAIR = false>
 int tma_rows(int n, const PlanarLevel& pl) {
     static int cache[3][32] = {};
-    if (!pl.lists) return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR, false>, 32 * NW, MINB, cache[0], PAIR);
-    return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR, true>, 32 * NW, MINB, cache[1 + pl.shared], PAIR, true, pl.shared);
+    if (!pl.lists) return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR, false, NoMask>, 32 * NW, MINB, cache[0], PAIR);
+    return tile_rows<TmaTile>(n, k_uzawa_tma<NW, MINB, PAIR, true, NoMask>, 32 * NW, MINB, cache[1 + pl.shared], PAIR, true, pl.shared);
 }
 template <class G>
 TileOrder tile_order(int n, int ty) {
@@ -2031,21 +2056,30 @@ bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLev
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_uzawa_tma<NW, MINB, PAIR, true>, 32 * NW,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_uzawa_tma<NW, MINB, PAIR, true, NoMask>, 32 * NW,
                                                           TmaTile::bytes(ty)) != cudaSuccess)
             per_sm = MINB;
         cudaGetLastError();
         pf = std::max(1, sms) * std::max(1, per_sm);
     }
     const dim3 grid(ord.cols * ord.rows), block(32 * NW);
-    if (pl.lists)
-        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, true>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
-                   tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0,
-                   pl.zero ? 1 : 0);
+    if (pl.zero && pl.dom == kDomL)
+        launch_pdl(k_uzawa_tma<8, 3, false, true, QuadrantMask, true>, grid, block, TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<true>{pl.lists}, q, tau, sigma, m, u_out, p_out, pf, (const float*)nullptr, (const float*)nullptr, 0,
+                   QuadrantMask{n});
+    else if (pl.zero)
+        launch_pdl(k_uzawa_tma<8, 3, false, true, NoMask, true>, grid, block, TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<true>{pl.lists}, q, tau, sigma, m, u_out, p_out, pf, (const float*)nullptr, (const float*)nullptr, 0,
+                   NoMask{});
+    else if (pl.dom == kDomL)
+        launch_pdl(k_uzawa_tma<8, 3, false, true, QuadrantMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<true>{pl.lists}, q, tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, QuadrantMask{n});
+    else if (pl.lists)
+        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, true, NoMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
+                   tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, NoMask{});
     else
-        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, false>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q, tau,
-                   sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0,
-                   pl.zero ? 1 : 0);
+        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, false, NoMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q, tau,
+                   sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, NoMask{});
     return true;
 }
 
@@ -2086,12 +2120,15 @@ bool launch_rt(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel&
     if (!make_tma_maps(n, ty, u, p, f, g, g, m)) return false;   // no Shat^{-1} tile (its map is unused)
     const TileOrder ord = tile_order<TmaTile>(n, ty);
     const dim3 grid(ord.cols * ord.rows);
-    if (pl.lists)
-        launch_pdl(k_restrict_tma<8, 3, PC, true>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
-                   restrict_weights(), m, fc, gc, uc, pc);
+    if (pl.dom == kDomL)
+        launch_pdl(k_restrict_tma<8, 3, PC, true, QuadrantMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<true>{pl.lists}, q, restrict_weights(), m, fc, gc, uc, pc, QuadrantMask{n});
+    else if (pl.lists)
+        launch_pdl(k_restrict_tma<8, 3, PC, true, NoMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
+                   restrict_weights(), m, fc, gc, uc, pc, NoMask{});
     else
-        launch_pdl(k_restrict_tma<8, 3, PC, false>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q,
-                   restrict_weights(), m, fc, gc, uc, pc);
+        launch_pdl(k_restrict_tma<8, 3, PC, false, NoMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q,
+                   restrict_weights(), m, fc, gc, uc, pc, NoMask{});
     return true;
 }
 
@@ -2157,6 +2194,15 @@ cudaError_t prepare_uzawa_reg() {
     if (e == cudaSuccess) e = tma_smem_attr<8, 4>();
     if (e == cudaSuccess) e = tma_smem_attr<8, 2, true>();
     if (e == cudaSuccess) e = tma_smem_attr<8, 3, true>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_uzawa_tma<8, 3, false, true, QuadrantMask>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TmaTile::bytes(kRegMaxRows));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_uzawa_tma<8, 3, false, true, QuadrantMask, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TmaTile::bytes(kRegMaxRows));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_uzawa_tma<8, 3, false, true, NoMask, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TmaTile::bytes(kRegMaxRows));
     if (e == cudaSuccess) e = rt_smem_attr<true>();
     if (e == cudaSuccess) e = rt_smem_attr<false>();
     if (e == cudaSuccess) e = small_smem_attr();
@@ -2180,6 +2226,7 @@ bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<f
                               float sigma, const float* u, const float* p, const float* f, const float* g, const float* sinv,
                               float* u_out, float* p_out, const CoarseCorrection& cc) {
     if (cc.u && (!cc.p || !embed_table_matches())) return false;
+    if ((pl.dom == kDomL && variant != 0) || (pl.zero && (variant > 1 || cc.u))) return false;
     switch (variant) {
         case 1: return launch_tma_v<8, 3>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, true, cc);
         case 2: return launch_tma_v<8, 4>(s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, false, cc);
@@ -2193,7 +2240,8 @@ bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<f
 bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau, float sigma,
                       const float* u, const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
                       const CoarseCorrection& cc) {
-    return launch_uzawa_tma_variant(g_tma_choice[pl.lists == nullptr][lvl(n)], s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
+    // the L has one variant, and so have steps from zero
+    return launch_uzawa_tma_variant(pl.dom == kDomL ? 0 : pl.zero ? 1 : g_tma_choice[pl.lists == nullptr][lvl(n)], s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
 }
 
 bool uzawa_tma_embed_available() { return uzawa_tma_available() && embed_table_matches(); }
