@@ -357,8 +357,8 @@ def peaks():
 # The sources that define and launch the float32 Uzawa-step kernels whose DRAM traffic
 # profiles/traffic.json records (the three-kernel step in kernels.cu, the tiles in uzawa_pair.cu and
 # uzawa_reg.cu, the variant table in uzawa_fused.cu, and every header they include).
-TRAFFIC_SOURCES = ("common.cuh", "cellops.cuh", "kernels.cuh", "kernels.cu", "stencil_tables.cuh",
-                   "uzawa_fused.cu", "uzawa_pair.cu", "uzawa_reg.cu", "tiles.cuh")
+TRAFFIC_SOURCES = ("common.cuh", "cellops.cuh", "kernels.cuh", "kernels.cu", "coarse_cycle.cuh",
+                   "stencil_tables.cuh", "uzawa_fused.cu", "uzawa_pair.cu", "uzawa_reg.cu", "tiles.cuh")
 
 
 def _kernel_source_sha():
