@@ -187,7 +187,7 @@ struct stokes_handle_t {
     int step_kernels = 0, plain_kernels = 0;   // kernel nodes in them
     cudaGraphExec_t loop = nullptr;         // WHILE(not converged) { step; device-side test }
     int loop_kernels = 0;                   // kernels per loop iteration
-    double* dctl = nullptr;                 // loop control (see k_solve_check), device
+    double* dctl = nullptr;                 // loop control (see LoopCheck), device
     int* ictl = nullptr;
     double* dhist = nullptr;                // residual^2 per step, device (kHistCap entries)
     double* hhist = nullptr;                // pinned mirror

@@ -34,3 +34,25 @@ def test_lshape_planar_step(levels, gamma, nu_pre, nu_post, beta):
     for x, y in ((ua, ub), (pa, pb)):
         assert float((x - y).abs().max() / x.abs().max()) < 2e-5
     assert float(ub[:, n:, n:].abs().max()) == 0.0 and float(pb[n // 2 + 1:, n // 2 + 1:].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("levels", [7, 8])
+def test_lshape_cycle_on_compact_levels(levels):
+    # a mixed cycle, the float32 step and the restriction on the L give the same bits whatever the layout of a solve
+    from paper_1502_04070_gb300.solver import Solver
+    n = 2 ** levels
+    gen = torch.Generator(device="cuda").manual_seed(levels)
+    u, f = (torch.rand(2, 2 * n + 1, 2 * n + 1, generator=gen, device="cuda") - 0.5 for _ in range(2))
+    p, g = (torch.rand(n + 1, n + 1, generator=gen, device="cuda") - 0.5 for _ in range(2))
+    S = [Solver(levels, 1.0, precision="mixed", domain="lshape", coarse_level=1, tma_level=t) for t in (6, 14)]
+    for beta in (1.0, 1e4):
+        res = []
+        for s in S:
+            s.set_beta(beta)
+            s.solve(f.double() / n ** 2, g.double() / n ** 2, tol=0.0, max_cycles=1)
+            out = list(s.cycle(u.double(), p.double(), f.double() / n ** 2, g.double() / n ** 2))
+            out += list(s.residual_restrict_f32(u, p, f, g))
+            v, q = u.clone(), p.clone()
+            s.smooth_f32(v, q, f, g, 2)
+            res.append(out + [v, q])
+        assert all(torch.equal(a, b) for a, b in zip(*res))
