@@ -536,7 +536,6 @@ void record_step(stokes_handle* h, const LoopCheck& ck = LoopCheck{}) {
 stokes_status capture_step(stokes_handle* h, cudaGraphExec_t* exec, int* kernels) {
     if (*exec) return STOKES_OK;
     cudaGraph_t g = nullptr;
-    h->ev_cursor = h->ev_smooth = h->ev_resid = 0;
     CK(cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
     record_step(h);
     cudaError_t e = cudaStreamEndCapture(h->st, &g);
@@ -559,7 +558,11 @@ stokes_status capture_step(stokes_handle* h, cudaGraphExec_t* exec, int* kernels
     return STOKES_OK;
 }
 
-stokes_status build_graph(stokes_handle* h) { return capture_step(h, &h->step, &h->step_kernels); }
+stokes_status build_graph(stokes_handle* h) {
+    if (h->step) return STOKES_OK;
+    h->ev_cursor = h->ev_smooth = h->ev_resid = 0;   // the events are those of `step`: no other capture records any
+    return capture_step(h, &h->step, &h->step_kernels);
+}
 
 // stokes_cycle on a MIXED handle: its result is one float32 cycle's, rounding included, and nothing after it removes
 // that rounding; it keeps the order of float32 operations it has always had (the one-CTA coarse cycle, per-cell
