@@ -406,7 +406,9 @@ unsigned long long stokes_batch_kernel_launches(const stokes_batch* b);
 /* Timing of the hot kernels inside the captured cycle: with enable != 0, the cycle graph is
  * rebuilt with CUDA event records (cudaEventRecordExternal) around every finest-level smoothing
  * step and around the float64 finest-level residual, and stokes_solve accumulates their durations
- * (milliseconds, counts) until the next stokes_set_timing call, which also resets the totals.
+ * (milliseconds, counts) until the next stokes_set_timing call, which also resets the totals.  A finest
+ * level that otherwise runs inside one launch with the levels below it (float64 N <= 32, float32
+ * N <= 64) then takes its steps by launches of their own: those are what is timed.
  * stokes_get_timing_fused: the finest-level smoothing steps that also add the coarse-grid
  * correction to their staged tiles (the first post-smoothing step of a planar level, Sec. 3),
  * which stokes_get_timing's smoothing totals leave out.  Any output pointer may be NULL. */

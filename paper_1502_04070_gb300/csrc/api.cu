@@ -251,12 +251,19 @@ PlanarLevel planar_level(const stokes_handle* h, const Level<T>& lv) {
     return PlanarLevel{h->plain ? nullptr : lv.mid, h->shared, h->dom};
 }
 
+// Is an iteration on level l of H the cluster kernel's?  Not the finest level's while its smoothing steps are timed:
+// the events lie between launches.
+template <typename T>
+bool in_cluster(const stokes_handle* h, const std::vector<Level<T>>& H, int l) {
+    return l <= h->cl_top && !H[l].planar && !h->plain && !(h->timing && l == (int)H.size() - 1);
+}
+
 // Does an iteration on level l that starts from zero (mg_cycle's `zero`) ignore what (u, p) hold?  Then nobody has
 // to clear them: the exact solve, the cluster cycle, and the planar step's first pre-smoothing step.
 template <typename T>
 bool ignores_iterate(const stokes_handle* h, const std::vector<Level<T>>& H, int l) {
     if (h->plain || h->prm.smoother != STOKES_UZAWA || l <= h->small_top) return false;
-    return l == h->clev || (l <= h->cl_top && !H[l].planar) || (H[l].planar && h->prm.nu_pre > 0);
+    return l == h->clev || in_cluster(h, H, l) || (H[l].planar && h->prm.nu_pre > 0);
 }
 
 // nu smoothing steps on level lv.  The state is in (u, p) when `sw` is false and in (tu, tp)
@@ -434,7 +441,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
             return;
         }
     }
-    if (l <= h->cl_top && !lv.planar && !h->plain) {
+    if (in_cluster(h, H, l)) {
         cluster_visit<T>(h, H, l, zero);
         return;
     }
