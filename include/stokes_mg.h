@@ -110,12 +110,16 @@ typedef struct stokes_params {
                           layout above.  The step needs the register tile's coefficient structure
                           (stokes_step_tables_match): setup and set_beta return STOKES_ERR_BAD_ARG for
                           a beta without it on such a level */
-    int coop_level;    /* STOKES_MIXED with the Uzawa smoother on the unit square: a visit of a float32
-                          level l <= coop_level (and above the coarsest level, below tma_level) runs the
-                          whole V- or W-cycle from l down, the coarsest solve included, as ONE
-                          cooperative launch whose phases meet at grid barriers, instead of one launch
-                          per phase.  0 or -1: off (the default; on a GB300 a phase of that launch
-                          costs about as much as a launch of its own); at most 6 */
+    int coop_level;    /* how the small levels run (Uzawa smoother).  0, the default: a visit of a float32 level
+                          N <= 64 (float64: N <= 32) runs the whole V- or W-cycle from there down in one
+                          thread-block cluster.  1 .. 6, STOKES_MIXED on the unit square: a visit of a
+                          float32 level l <= coop_level (and above the coarsest level, below tma_level) runs
+                          it as ONE cooperative launch whose phases meet at grid barriers, the levels
+                          above by launches of their own (on a GB300 a phase of that launch costs about as
+                          much as a launch); it leaves the cluster out, other handles ignore it.  -1: by
+                          launches alone, float64 too.  Where the cluster is left out, or the device
+                          cannot hold one, a float32 V-cycle down to level 0 on the square runs its levels
+                          N <= 32 in one CTA */
 } stokes_params;
 
 /* Paper defaults: Uzawa, nu = 3+3, tau = sigma = 0.8, V-cycle, float64, one inner cycle, coarsest

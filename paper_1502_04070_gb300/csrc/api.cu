@@ -251,11 +251,17 @@ PlanarLevel planar_level(const stokes_handle* h, const Level<T>& lv) {
     return PlanarLevel{h->plain ? nullptr : lv.mid, h->shared, h->dom};
 }
 
-// Is an iteration on level l of H the cluster kernel's?  Not the finest level's while its smoothing steps are timed:
-// the events lie between launches.
+// Are the smoothing steps of level l of H timed (the finest's, stokes_set_timing)?  It then runs by launches of its
+// own, the events lie between them.
+template <typename T>
+bool timed_level(const stokes_handle* h, const std::vector<Level<T>>& H, int l) {
+    return h->timing && l == (int)H.size() - 1;
+}
+
+// Is an iteration on level l of H the cluster kernel's?
 template <typename T>
 bool in_cluster(const stokes_handle* h, const std::vector<Level<T>>& H, int l) {
-    return l <= h->cl_top && !H[l].planar && !h->plain && !(h->timing && l == (int)H.size() - 1);
+    return l <= h->cl_top && !H[l].planar && !h->plain && !timed_level(h, H, l);
 }
 
 // Does an iteration on level l that starts from zero (mg_cycle's `zero`) ignore what (u, p) hold?  Then nobody has
@@ -390,7 +396,7 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
     }
     if constexpr (sizeof(T) == 4) {
         // small levels: the whole V- or W-cycle from level l down in one cooperative launch
-        if (l <= h->small_top && l > h->clev) {
+        if (l <= h->small_top && l > h->clev && !timed_level(h, H, l)) {
             SmallCycleHost sh{};
             for (int k = h->clev; k <= l; ++k) {
                 Level<float>& L = H[k];
@@ -420,8 +426,9 @@ void mg_cycle(stokes_handle* h, std::vector<Level<T>>& H, int l, bool zero = fal
         }
     }
     if constexpr (sizeof(T) == 4) {
-        if (h->plain && l <= kCoarseCycleTop && h->prm.gamma == 1 && h->prm.smoother == STOKES_UZAWA && h->clev == 0 &&
-            h->dom == kDomSquare) {
+        // stokes_cycle, and solves that no cluster serves: the V-cycle from a small level down in one CTA
+        if ((h->plain || h->cl_top < 0) && l <= kCoarseCycleTop && h->prm.gamma == 1 && h->prm.smoother == STOKES_UZAWA &&
+            h->clev == 0 && h->dom == kDomSquare && !timed_level(h, H, l)) {
             CoarseCycleArgs a;
             for (int k = 1; k <= l; ++k) {
                 a.c[k - 1] = H[k].c;
@@ -933,8 +940,9 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
             }
         }
     }
-    // the cluster cycle of the small levels: Uzawa smoother, at least one level above the coarsest
-    if (P.smoother == STOKES_UZAWA) {
+    // the cluster cycle of the small levels: Uzawa smoother, at least one level above the coarsest, and neither
+    // the cooperative cycle nor launches per phase asked for
+    if (P.smoother == STOKES_UZAWA && h->small_top < 0 && P.coop_level >= 0) {
         const bool f32 = P.precision == STOKES_MIXED;
         const int ctop = std::min(P.levels - 1, f32 ? cluster_top<float>() : cluster_top<double>());
         if (ctop > P.coarse_level && (f32 ? prepare_cluster_cycle<float>() : prepare_cluster_cycle<double>())) {

@@ -1,6 +1,7 @@
 // coarse_cycle.cuh -- the float32 V-cycle below a small level in ONE launch (included by kernels.cu): the
 // arithmetic of stokes_cycle on a mixed-precision handle, whose result is the float32 cycle's own, rounding
-// included.  Solves, which correct that rounding, run cluster_cycle.cu instead, three times as fast.
+// included, and of solves that run without a cluster (stokes_params.coop_level, or a device that holds none).
+// Other solves run cluster_cycle.cu instead, three times as fast.
 //
 // On levels with N <= 32 a multigrid step is a few thousand cells: one launch per phase would
 // spend far more time in launch latency and in a handful of busy SMs than in arithmetic.  Here one
