@@ -176,8 +176,9 @@ stokes_status stokes_sizes(const stokes_handle* h, int* N, size_t* n_vel, size_t
  * step: float64 residual, params.inner_cycles float32 cycles on the correction, float64 update; it keeps
  * the float32 order of operations of one launch per phase or step (and of the one-CTA cycle below N = 64),
  * whose rounding its result carries, where the steps of a solve run the faster cluster cycle.  On the L with
- * levels >= tma_level it works on compact float32 levels of its own, allocated by the first such call (as do
- * stokes_smooth_f32 and stokes_residual_restrict_f32). */
+ * levels >= tma_level it works on compact float32 levels of its own (as do stokes_smooth_f32 and
+ * stokes_residual_restrict_f32), which the setup allocates; without the memory for both the handle keeps compact
+ * levels alone. */
 stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double* f, const double* g);
 
 /* Iterates stokes_cycle from the given (u, p) until ||F - A x||_2 <= tol ||F||_2 or max_cycles.

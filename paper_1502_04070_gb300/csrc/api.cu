@@ -156,7 +156,7 @@ struct stokes_handle_t {
     int L = 0;                              // number of levels
     std::vector<Level<double>> h64;         // FP64: all levels; MIXED: finest only
     std::vector<Level<float>> h32;          // MIXED: all levels
-    std::vector<Level<float>> cyc32;        // MIXED on the L: compact ones (make_cycle_levels)
+    std::vector<Level<float>> cyc32;        // MIXED on the L: compact ones (alloc_cycle_levels)
     double* inv = nullptr;                  // level-0 bordered inverse (27 x 27)
     int dom = kDomSquare;                   // the domain: kDomSquare, or kDomL (common.cuh)
     int clev = 0;                           // coarsest level of the iteration (exact solve there)
@@ -688,8 +688,17 @@ stokes_status upload_cluster_tables(stokes_handle* h, const std::vector<Level<T>
 }
 
 // stokes_cycle of a MIXED handle on the L runs the compact layout on every level (see build_plain_graph), and so do the
-// float32 step and restriction on a caller's arrays: the first such call gives levels that are planar in h32 a compact
-// twin, the others are h32's own.
+// float32 step and restriction on a caller's arrays: levels that are planar in h32 have a compact twin, the others are
+// h32's own.
+stokes_status alloc_cycle_levels(stokes_handle* h) {
+    h->cyc32.resize(h->h32.size());
+    for (size_t k = 0; k < h->h32.size(); ++k) {
+        if (!h->h32[k].planar) continue;
+        const stokes_status s = alloc_level(h->cyc32[k], (int)k, h->mem);
+        if (s != STOKES_OK) return s;
+    }
+    return STOKES_OK;
+}
 void fill_cycle_levels(stokes_handle* h) {
     for (size_t k = 0; k < h->cyc32.size(); ++k) {
         Level<float>& lv = h->cyc32[k];
@@ -700,22 +709,6 @@ void fill_cycle_levels(stokes_handle* h) {
         lv.c = h->h32[k].c;
         launch_schur_diag<float>(h->st, lv.n, make_coef<double>(lv.n, h->prm.beta), lv.sinv, h->dom, 0);
     }
-}
-stokes_status make_cycle_levels(stokes_handle* h) {
-    if (h->dom != kDomL || !h->has_planar || !h->cyc32.empty()) return STOKES_OK;
-    std::vector<Level<float>> H(h->h32.size());
-    for (size_t k = 0; k < H.size(); ++k) {
-        if (!h->h32[k].planar) continue;
-        const stokes_status s = alloc_level(H[k], (int)k, h->mem);
-        if (s != STOKES_OK) {
-            for (auto& lv : H) h->mem.put(lv.slab);
-            return s;
-        }
-    }
-    h->cyc32.swap(H);
-    fill_cycle_levels(h);
-    CK(cudaGetLastError());
-    return STOKES_OK;
 }
 
 stokes_status rebuild_beta(stokes_handle* h) {
@@ -869,11 +862,9 @@ void stokes_destroy(stokes_handle* h) {
     delete h;
 }
 
-stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle** out) {
-    ApiRange nvtx_range("stokes_setup");
-    if (!prm || !out) return STOKES_ERR_BAD_ARG;
-    *out = nullptr;
-    const stokes_params& P = *prm;
+// planar: float32 levels from tma_level up take the planar layout; cycles: the handle also serves the calls that run
+// the compact layout on the L
+static stokes_status setup_handle(const stokes_params& P, void* stream, bool planar, bool cycles, stokes_handle** out) {
     if (P.levels < 1 || P.levels > 13 || !(P.beta >= 0.0) || !std::isfinite(P.beta) || P.nu_pre < 0 ||
         P.nu_post < 0 || !(P.tau > 0.0) || !(P.sigma > 0.0) || (P.gamma != 1 && P.gamma != 2) ||
         (P.smoother != STOKES_UZAWA && P.smoother != STOKES_NORMAL_EQ) ||
@@ -921,10 +912,11 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
         if ((s = alloc_level(h->h64[0], kfin, h->mem)) != STOKES_OK) return bail(s);
         h->h32.resize(P.levels);
         const int tlev = P.tma_level > 0 ? P.tma_level : kDefaultTmaLevel;
-        const bool tma = P.smoother == STOKES_UZAWA && uzawa_tma_available();
+        const bool tma = planar && P.smoother == STOKES_UZAWA && uzawa_tma_available();
         for (int k = 0; k < P.levels; ++k)
             if ((s = alloc_level(h->h32[k], k, h->mem, tma && k >= tlev)) != STOKES_OK) return bail(s);
         h->has_planar = tma && tlev < P.levels;
+        if (h->has_planar && h->dom == kDomL && cycles && (s = alloc_cycle_levels(h)) != STOKES_OK) return bail(s);
         h->fuse_prolong = h->has_planar && fuse_prolong_enabled() && uzawa_tma_embed_available();
         // the cooperative small-level cycle: compact float32 levels up to coop_level, above the coarsest
         if (P.coop_level > 0 && P.smoother == STOKES_UZAWA && P.domain == STOKES_UNIT_SQUARE) {
@@ -980,6 +972,21 @@ stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle
     if ((s = rebuild_beta(h)) != STOKES_OK) return bail(s);
     *out = h;
     return STOKES_OK;
+}
+
+// A mixed-precision handle on the L that does not fit with planar levels and their compact twins runs the compact
+// levels alone, which take half the float32 memory.
+static stokes_status setup_any(const stokes_params* prm, void* stream, bool cycles, stokes_handle** out) {
+    if (!prm || !out) return STOKES_ERR_BAD_ARG;
+    *out = nullptr;
+    const stokes_status s = setup_handle(*prm, stream, true, cycles, out);
+    if (s != STOKES_ERR_OOM || prm->domain != STOKES_L_SHAPE || prm->precision != STOKES_MIXED) return s;
+    return setup_handle(*prm, stream, false, cycles, out);
+}
+
+stokes_status stokes_setup(const stokes_params* prm, void* stream, stokes_handle** out) {
+    ApiRange nvtx_range("stokes_setup");
+    return setup_any(prm, stream, true, out);
 }
 
 static stokes_status autotune_levels(stokes_handle* h, cudaStream_t st);
@@ -1039,7 +1046,6 @@ stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double*
     stokes_status s;
     if ((s = copy_in(h, u, p, f, g)) != STOKES_OK) return s;
     if (h->mixed()) {
-        if ((s = make_cycle_levels(h)) != STOKES_OK) return s;
         const bool own = !h->cyc32.empty();
         if (own) h->h32.swap(h->cyc32);
         residual_norm_fin(h);   // float64 residual and the float32 right-hand side of the correction
@@ -1214,9 +1220,7 @@ stokes_status stokes_smooth(stokes_handle* h, double* u, double* p, const double
 stokes_status stokes_smooth_f32(stokes_handle* h, float* u, float* p, const float* f, const float* g, int nu) {
     ApiRange nvtx_range("stokes_smooth_f32");
     if (!h || !u || !p || !f || !g || nu < 0 || !h->mixed()) return STOKES_ERR_BAD_ARG;
-    const stokes_status sc = make_cycle_levels(h);   // the L: on the caller's compact arrays
-    if (sc != STOKES_OK) return sc;
-    // coefficients, diagonals and ping-pong partners of the finest level
+    // coefficients, diagonals and ping-pong partners of the finest level (the L: on the caller's compact arrays)
     Level<float> lv = h->cyc32.empty() ? h->h32.back() : h->cyc32.back();
     if (lv.planar) {
         // the caller's compact arrays into the level's own planar buffers, and the result back
@@ -1246,8 +1250,6 @@ stokes_status stokes_residual_restrict_f32(stokes_handle* h, const float* u, con
                                            const float* g, float* fc, float* gc) {
     ApiRange nvtx_range("stokes_residual_restrict_f32");
     if (!h || !u || !p || !f || !g || !fc || !gc || !h->mixed() || h->L < 2) return STOKES_ERR_BAD_ARG;
-    const stokes_status sc = make_cycle_levels(h);
-    if (sc != STOKES_OK) return sc;
     std::vector<Level<float>>& H = h->cyc32.empty() ? h->h32 : h->cyc32;
     Level<float>& lv = H.back();
     Level<float>& cl = H[h->L - 2];
@@ -1509,7 +1511,7 @@ stokes_status stokes_batch_setup(int count, const int* levels, const double* bet
         prm.levels = levels[i];
         prm.beta = betas[i];
         stokes_handle* h = nullptr;
-        if ((s = stokes_setup(&prm, b->st, &h)) != STOKES_OK) {
+        if ((s = setup_any(&prm, b->st, false, &h)) != STOKES_OK) {   // instances only solve
             stokes_batch_destroy(b);
             return s;
         }
