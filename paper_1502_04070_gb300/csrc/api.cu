@@ -233,13 +233,14 @@ void ev_end(stokes_handle* h, int k) {
 
 // The status a call reports once its work is done: STOKES_ERR_CUDA if a step variant refused to
 // launch (recorded while launching or capturing), STOKES_ERR_TIMEOUT if a CTA of the planar levels'
-// step gave up waiting for its tiles (a device-wide flag, cleared by the read), else st.
-stokes_status take_launch_failure(stokes_handle* h, stokes_status st = STOKES_OK) {
+// step gave up waiting for its tiles (a device-wide flag, cleared by the read), else st.  planar: the call ran
+// planar levels; only then does it wait for the stream.
+stokes_status take_launch_failure(stokes_handle* h, stokes_status st, bool planar) {
     if (h->launch_failed) {
         h->launch_failed = false;
         return STOKES_ERR_CUDA;
     }
-    if (h->has_planar) {
+    if (planar) {
         CK(cudaStreamSynchronize(h->st));
         if (uzawa_tma_timeouts()) return STOKES_ERR_TIMEOUT;
     }
@@ -1058,7 +1059,7 @@ stokes_status stokes_cycle(stokes_handle* h, double* u, double* p, const double*
     } else {
         if ((s = build_graph(h)) != STOKES_OK || (s = launch_step(h)) != STOKES_OK) return s;
     }
-    return take_launch_failure(h, copy_out(h, u, p));
+    return take_launch_failure(h, copy_out(h, u, p), h->has_planar && h->cyc32.empty());
 }
 
 stokes_status stokes_solve(stokes_handle* h, double* u, double* p, const double* f, const double* g,
@@ -1177,7 +1178,7 @@ stokes_status stokes_solve(stokes_handle* h, double* u, double* p, const double*
         rep->rel_residual = nF > 0 ? r / nF : r;
         rep->mean_rate = cycles > 0 && r0 > 0 ? std::pow(r / r0, 1.0 / cycles) : 0.0;
     }
-    return take_launch_failure(h, result);
+    return take_launch_failure(h, result, h->has_planar);
 }
 
 stokes_status stokes_residual(stokes_handle* h, const double* u, const double* p, const double* f,
@@ -1230,7 +1231,7 @@ stokes_status stokes_smooth_f32(stokes_handle* h, float* u, float* p, const floa
         launch_from_planar(h->st, lv.n, sw ? lv.tu : lv.u, sw ? lv.tp : lv.p, u, p);
         h->launches += (unsigned long long)nu + 3;
         CK(cudaGetLastError());
-        return take_launch_failure(h);
+        return take_launch_failure(h, STOKES_OK, true);
     }
     lv.u = u;
     lv.p = p;
@@ -1243,7 +1244,7 @@ stokes_status stokes_smooth_f32(stokes_handle* h, float* u, float* p, const floa
     }
     h->launches += (unsigned long long)nu;
     CK(cudaGetLastError());
-    return take_launch_failure(h);
+    return take_launch_failure(h, STOKES_OK, false);
 }
 
 stokes_status stokes_residual_restrict_f32(stokes_handle* h, const float* u, const float* p, const float* f,
@@ -1271,7 +1272,7 @@ stokes_status stokes_residual_restrict_f32(stokes_handle* h, const float* u, con
         h->launches += 2;
     }
     CK(cudaGetLastError());
-    return take_launch_failure(h);
+    return take_launch_failure(h, STOKES_OK, lv.planar);
 }
 
 stokes_status stokes_restrict(stokes_handle* h, const double* fu, const double* fp, double* fc, double* gc) {
@@ -1666,7 +1667,7 @@ stokes_status stokes_batch_solve(stokes_batch* b, double* const* u, double* cons
         if (cycles) cycles[i] = total;
         if (rel_residual) rel_residual[i] = nF > 0 ? r / nF : r;
     }
-    for (int i = 0; i < b->count; ++i) result = take_launch_failure(b->inst[i], result);
+    for (int i = 0; i < b->count; ++i) result = take_launch_failure(b->inst[i], result, b->inst[i]->has_planar);
     return result;
 }
 
@@ -1835,7 +1836,7 @@ stokes_status stokes_euler_run(stokes_handle* h, double* u, double* p, const dou
     unsigned long long total = 0;
     const stokes_status out = euler_results(res, steps, tol, cycles, rel_residual, &total);
     h->launches += (unsigned long long)h->euler_kernels + total * (unsigned long long)h->euler_body;
-    return take_launch_failure(h, out);
+    return take_launch_failure(h, out, h->has_planar);
 }
 
 stokes_status stokes_batch_euler_run(stokes_batch* b, double* const* u, double* const* p,
@@ -1894,7 +1895,7 @@ stokes_status stokes_batch_euler_run(stokes_batch* b, double* const* u, double* 
         b->mem.put(dres[i]);
     }
     if (e != cudaSuccess) return fail(e);
-    for (int i = 0; i < count; ++i) out = take_launch_failure(b->inst[i], out);
+    for (int i = 0; i < count; ++i) out = take_launch_failure(b->inst[i], out, b->inst[i]->has_planar);
     return out;
 }
 
