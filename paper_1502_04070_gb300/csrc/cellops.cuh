@@ -316,7 +316,9 @@ __device__ __forceinline__ void mb_row(const OpCoef<T>& c, const T (&wx)[25], co
 }
 
 // SUB false: a.au = A u, a.bt = B^T p, a.bu = B u.  SUB true: a.au, a.bu come in as f, g and go out as f - A u - B^T p and
-// g - B u (a.bt is not used): no separate subtractions.
+// g - B u (a.bt is not used): no separate subtractions.  B^T p first: its terms and f are of order h where those of A u
+// are of order one, so their sum rounds less (a residual's relative error 1.29e-16; 1.50e-16 with A u first, 1.43e-16 with
+// the two products summed apart; the time is the same).
 template <bool DA, bool DBT, bool DB, bool DD, bool MASK, int C, bool SUB, typename T, typename VU, typename VP>
 __device__ __forceinline__ void cell_apply_merged(int i, int j, int n, const OpCoef<T>& c, const VU& ux, const VU& uy,
                                                   const VP& p, Acc<T>& a) {
@@ -330,18 +332,18 @@ __device__ __forceinline__ void cell_apply_merged(int i, int j, int n, const OpC
         for (int s = 0; s < 4; ++s) a.au[0][s] = a.au[1][s] = a.bt[0][s] = a.bt[1][s] = a.idg[s] = T(0);
         a.bu = T(0);
     }
-    if constexpr (DA) {
-        ma_row<SUB, C, 0>(c.MA, wx, wy, a.au[0][0], a.au[1][0], K25);
-        ma_row<SUB, C, 1>(c.MA, wx, wy, a.au[0][1], a.au[1][1], K25);
-        ma_row<SUB, C, 2>(c.MA, wx, wy, a.au[0][2], a.au[1][2], K25);
-        ma_row<SUB, C, 3>(c.MA, wx, wy, a.au[0][3], a.au[1][3], K25);
-    }
     if constexpr (DBT) {
         auto& r = SUB ? a.au : a.bt;
         mbt_row<SUB, C, 0>(c, pw, r[0][0], r[1][0], V9);
         mbt_row<SUB, C, 1>(c, pw, r[0][1], r[1][1], V9);
         mbt_row<SUB, C, 2>(c, pw, r[0][2], r[1][2], V9);
         mbt_row<SUB, C, 3>(c, pw, r[0][3], r[1][3], V9);
+    }
+    if constexpr (DA) {
+        ma_row<SUB, C, 0>(c.MA, wx, wy, a.au[0][0], a.au[1][0], K25);
+        ma_row<SUB, C, 1>(c.MA, wx, wy, a.au[0][1], a.au[1][1], K25);
+        ma_row<SUB, C, 2>(c.MA, wx, wy, a.au[0][2], a.au[1][2], K25);
+        ma_row<SUB, C, 3>(c.MA, wx, wy, a.au[0][3], a.au[1][3], K25);
     }
     if constexpr (DD) {
 #pragma unroll
