@@ -46,7 +46,7 @@ MassCoef<T> make_mass(int n) {
         for (int q = 0; q < 4; ++q)
             for (int r = 0; r < 4; ++r) m.MP[o][q][r] = (T)(h * h * S.MP[o][q][r]);
     }
-    fill_merged(m);
+    fill_merged(m, n);
     return m;
 }
 

@@ -47,3 +47,26 @@ def test_residual_rounds_no_more_than_separate_products():
     want = b[:d.nu].astype(np.longdouble) - au - _times(B, x[d.nu:])
     err = got.astype(np.longdouble) - want
     assert float(np.sqrt((err * err).sum() / (want * want).sum())) <= 1.43e-16
+
+
+def test_load_vectors_have_exact_coefficients():
+    """The load vector of a basis function is a column of the mass matrix: every entry is its multiple of h^2/360 (velocity,
+    at the unknowns) and h^2/24 (pressure, off the boundary), rounded once.  N = 8; basis functions in every orientation
+    class, their neighbours included."""
+    from paper_1502_04070_gb300.solver import Solver
+    k = 2
+    n = 2 ** (k + 1)
+    d = fem.discretizations(k + 1)[-1]
+    S = Solver(k + 1, 1.0)
+    for y in range(1, 2 * n):
+        for x in range(1, 2 * n):
+            fn, gn = np.zeros((2, 2 * n + 1, 2 * n + 1)), np.zeros((n + 1, n + 1))
+            fn[0, y, x] = fn[1, y, x] = 1.0
+            if x <= n and y <= n:
+                gn[y, x] = 1.0
+            f, g = [host(t) for t in S.load_vectors(dev(fn), dev(gn), project_g=False)]
+            F = d.load(fn, gn)
+            wf, wg = d.from_vec(F)
+            for got, want, unit in ((f, wf, 360.0 * n * n), (g[1:-1, 1:-1], wg[1:-1, 1:-1], 24.0 * n * n)):
+                assert np.abs(want * unit - np.rint(want * unit)).max() < 1e-9
+                assert np.array_equal(got, np.rint(want * unit) / unit), (x, y)
