@@ -948,6 +948,7 @@ static stokes_status setup_handle(const stokes_params& P, void* stream, bool pla
         }
     }
     h->mass = make_mass<double>(h->fin().n);
+    if (!stencil_masks_cover(h->mass)) return bail(STOKES_ERR_BAD_ARG);   // no level does
     h->npartial = 2 * cells_blocks(h->fin().n);   // two sets of per-block partial sums (refinement update)
     if (h->mem.get(&h->inv, 27 * 27 * sizeof(double)) != cudaSuccess ||
         h->mem.get(&h->partial, (size_t)h->npartial * sizeof(double)) != cudaSuccess ||
@@ -1325,9 +1326,10 @@ stokes_status stokes_stencil_rows(int levels, double beta, int cls, double* ma, 
 
 stokes_status stokes_step_tables_match(int levels, double beta) {
     if (levels < 1 || levels > 13 || !(beta >= 0.0) || !std::isfinite(beta)) return STOKES_ERR_BAD_ARG;
-    return reg_tables_match(make_coef<float>(1 << levels, beta)) && stencil_masks_cover(make_coef<double>(1 << levels, beta))
-               ? STOKES_OK
-               : STOKES_ERR_BAD_ARG;
+    const int n = 1 << levels;
+    const bool ok = reg_tables_match(make_coef<float>(n, beta)) && stencil_masks_cover(make_coef<double>(n, beta)) &&
+                    stencil_masks_cover(make_mass<double>(n));
+    return ok ? STOKES_OK : STOKES_ERR_BAD_ARG;
 }
 
 stokes_status stokes_transfer_weights(double* w) {

@@ -154,6 +154,15 @@ inline bool stencil_masks_cover(const OpCoef<T>& c) {
     }
     return amax > 0.0 && bmax > 0.0 && a <= tol * amax && b <= tol * bmax;
 }
+// host: the same of the mass rows, which the operator's coefficients hide at small beta h^2 (exact: fill_merged)
+template <typename T>
+inline bool stencil_masks_cover(const MassCoef<T>& m) {
+    for (int k = 0; k < kStencilClasses; ++k)
+        for (int s = 0; s < 4; ++s)
+            for (int w = 0; w < 25; ++w)
+                if (!nz_MA(k, s, w) && m.MM[k][s][w] != T(0)) return false;
+    return true;
+}
 
 // host: merged stencils from the square-local matrices (sums over the squares that share a node)
 template <typename T>
@@ -351,11 +360,6 @@ __device__ __forceinline__ int vertex_triangles_dom(int i, int j, int n, int dom
         cnt += ((tri_mask(o, 0) >> node) & 1u) + ((tri_mask(o, 1) >> node) & 1u);
     }
     return cnt;
-}
-// w_i = int_Omega psi_i for the square or the L
-__device__ __forceinline__ double vertex_weight_dom(int i, int j, int n, int dom) {
-    const double h = 1.0 / n;
-    return vertex_triangles_dom(i, j, n, dom) * h * h / 6.0;
 }
 
 // Planar float32 layout of the large float32 levels (the velocity arrays of the refinement's inner

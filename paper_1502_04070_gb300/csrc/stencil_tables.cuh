@@ -1,6 +1,7 @@
-// stencil_tables.cuh -- compile-time structure of the merged stencils of the orientation classes 0 and
-// 1, the values that a level fills it with, and the weights of the canonical embedding: what the
-// kernels that keep the operator's coefficients in registers share (uzawa_reg.cu, cluster_cycle.cu).
+// stencil_tables.cuh -- the merged stencils as their kernels use them: the compile-time structure of the orientation
+// classes 0 and 1 and the values that a level fills it with (uzawa_reg.cu, coefficients in registers), the weights of
+// the canonical embedding (uzawa_reg.cu, kernels.cu), and the entries of every class as lists (cluster_cycle.cu and the
+// mid-line tiles of uzawa_reg.cu).
 #pragma once
 #include <algorithm>
 #include <cmath>
@@ -50,20 +51,18 @@ __host__ __device__ constexpr bool bt_vwin(int C, int v) {
     return false;
 }
 
-// Values of the structure above for one level, in the level's own precision (T)
-template <typename T>
+// Values of the structure above for one level
 struct RegVals {
-    T a[2][kGroups];   // A group values, per class
-    T ti[2][2];        // tau / diag A: [class][0 = V row, 1 = H, E, C rows]
-    T b;               // B = (b / 2) x (the integer tables)
+    float a[2][kGroups];   // A group values, per class
+    float ti[2][2];        // tau / diag A: [class][0 = V row, 1 = H, E, C rows]
+    float b;               // B = (b / 2) x (the integer tables)
 };
 
 // Fills q from the level's merged stencils and checks that they have exactly the compile-time
 // structure (zeros, equal groups, B entries +-b, +-b/2) up to rounding; false if not (the caller then
 // uses kernels that take the stencils as they are).
-template <typename T>
-inline bool make_reg_vals(const OpCoef<T>& c, T tau, RegVals<T>& q) {
-    const double tol = sizeof(T) == 4 ? 1e-6 : 1e-14;
+inline bool make_reg_vals(const OpCoef<float>& c, float tau, RegVals& q) {
+    constexpr double tol = 1e-6;
     double amax = 0.0, bmax = 0.0;
     for (int C = 0; C < 2; ++C) {
         for (int s = 0; s < 4; ++s)
@@ -83,7 +82,7 @@ inline bool make_reg_vals(const OpCoef<T>& c, T tau, RegVals<T>& q) {
                     continue;
                 }
                 if (!set[gid]) {
-                    q.a[C][gid] = (T)v;
+                    q.a[C][gid] = (float)v;
                     set[gid] = true;
                 } else if (std::fabs(v - (double)q.a[C][gid]) > tol * std::fabs(v) + 0.1 * tol * amax) {
                     return false;
@@ -107,17 +106,17 @@ inline bool make_reg_vals(const OpCoef<T>& c, T tau, RegVals<T>& q) {
         q.ti[C][0] = tau * c.MIdg[C][0];
         q.ti[C][1] = tau * c.MIdg[C][1];
     }
-    q.b = (T)b;
+    q.b = (float)b;
     return true;
 }
 
 // acc += (k / 2) v with a compile-time k in {0, +-1, +-2}
-template <int K, typename T>
-__device__ __forceinline__ void addk(T& acc, T v) {
+template <int K>
+__device__ __forceinline__ void addk(float& acc, float v) {
     if constexpr (K == 2) acc += v;
     else if constexpr (K == -2) acc -= v;
-    else if constexpr (K == 1) acc = fma(T(0.5), v, acc);
-    else if constexpr (K == -1) acc = fma(T(-0.5), v, acc);
+    else if constexpr (K == 1) acc = fmaf(0.5f, v, acc);
+    else if constexpr (K == -1) acc = fmaf(-0.5f, v, acc);
 }
 
 // ---- the canonical embedding (Sec. 3)

@@ -46,7 +46,7 @@ struct RegCoef {
 
 // false if the level's stencils lack the structure (the caller then uses another step variant)
 static bool make_reg_coef(const OpCoef<float>& c, float tau, RegCoef& q) {
-    RegVals<float> v;
+    RegVals v;
     if (!make_reg_vals(c, tau, v)) return false;
     for (int C = 0; C < 2; ++C) {
         for (int g = 0; g < kGroups; ++g) q.a[C][g] = make_float2(v.a[C][g], v.a[C][g]);
