@@ -708,7 +708,9 @@ void fill_cycle_levels(stokes_handle* h) {
             continue;
         }
         lv.c = h->h32[k].c;
-        launch_schur_diag<float>(h->st, lv.n, make_coef<double>(lv.n, h->prm.beta), lv.sinv, h->dom, 0);
+        const size_t row = (lv.n + 1) * sizeof(float);
+        cudaMemcpy2DAsync(lv.sinv, row, h->h32[k].sinv, pl_vpitch(lv.n) * sizeof(float), row, lv.n + 1,
+                          cudaMemcpyDeviceToDevice, h->st);
     }
 }
 
