@@ -676,15 +676,20 @@ void collect_timing(stokes_handle* h) {
     }
 }
 
-// The cluster cycle's lists for the levels' current operators.
+// The cluster cycle's lists: the transfers' at set-up, the levels' for their current operators.
 template <typename T>
-stokes_status upload_cluster_tables(stokes_handle* h, const std::vector<Level<T>>& H, ClusterTables<T>* dst) {
-    std::vector<ClusterTables<T>> t(1);   // on the heap
-    bool ok = fill_cluster_xfer(t[0].x);
-    for (int k = 1; k <= h->cl_top && ok; ++k) ok = fill_cluster_level(t[0].L[k], H[k].n, H[k].c, (T)h->prm.tau);
-    if (!ok) return STOKES_ERR_BAD_ARG;
-    CK(cudaMemcpyAsync(dst, t.data(), sizeof(ClusterTables<T>), cudaMemcpyHostToDevice, h->st));
-    CK(cudaStreamSynchronize(h->st));
+stokes_status upload_cluster_xfer(stokes_handle* h, ClusterTables<T>* dst) {
+    XferLists<T> x;
+    if (!fill_cluster_xfer(x)) return STOKES_ERR_BAD_ARG;
+    CK(cudaMemcpyAsync(&dst->x, &x, sizeof x, cudaMemcpyHostToDevice, h->st));   // pageable: copied on return
+    return STOKES_OK;
+}
+template <typename T>
+stokes_status upload_cluster_levels(stokes_handle* h, const std::vector<Level<T>>& H, ClusterTables<T>* dst) {
+    std::vector<LevelLists<T>> t(h->cl_top);
+    for (int k = 1; k <= h->cl_top; ++k)
+        if (!fill_cluster_level(t[k - 1], H[k].n, H[k].c, (T)h->prm.tau)) return STOKES_ERR_BAD_ARG;
+    CK(cudaMemcpyAsync(&dst->L[1], t.data(), sizeof t[0] * t.size(), cudaMemcpyHostToDevice, h->st));   // likewise
     return STOKES_OK;
 }
 
@@ -718,7 +723,6 @@ stokes_status rebuild_beta(stokes_handle* h) {
     const double beta = h->prm.beta;
     for (auto& lv : h->h64) {
         lv.c = make_coef<double>(lv.n, beta);
-        if (!stencil_masks_cover(lv.c)) return STOKES_ERR_BAD_ARG;   // no beta does
         launch_schur_diag<double>(h->st, lv.n, lv.c, lv.sinv, h->dom);
     }
     for (auto& lv : h->h32) {
@@ -737,8 +741,8 @@ stokes_status rebuild_beta(stokes_handle* h) {
     }
     fill_cycle_levels(h);
     if (h->cl_top > 0) {
-        const stokes_status s = h->mixed() ? upload_cluster_tables(h, h->h32, h->cl_tab32)
-                                           : upload_cluster_tables(h, h->h64, h->cl_tab64);
+        const stokes_status s = h->mixed() ? upload_cluster_levels(h, h->h32, h->cl_tab32)
+                                           : upload_cluster_levels(h, h->h64, h->cl_tab64);
         if (s != STOKES_OK) return s;
     }
     if (h->mixed()) {
@@ -947,10 +951,11 @@ static stokes_status setup_handle(const stokes_params& P, void* stream, bool pla
                 cudaGetLastError();
                 return bail(STOKES_ERR_OOM);
             }
+            s = f32 ? upload_cluster_xfer(h, h->cl_tab32) : upload_cluster_xfer(h, h->cl_tab64);
+            if (s != STOKES_OK) return bail(s);
         }
     }
     h->mass = make_mass<double>(h->fin().n);
-    if (!stencil_masks_cover(h->mass)) return bail(STOKES_ERR_BAD_ARG);   // no level does
     h->npartial = 2 * cells_blocks(h->fin().n);   // two sets of per-block partial sums (refinement update)
     if (h->mem.get(&h->inv, 27 * 27 * sizeof(double)) != cudaSuccess ||
         h->mem.get(&h->partial, (size_t)h->npartial * sizeof(double)) != cudaSuccess ||
@@ -974,6 +979,8 @@ static stokes_status setup_handle(const stokes_params& P, void* stream, bool pla
         }
     }
     if ((s = rebuild_beta(h)) != STOKES_OK) return bail(s);
+    // the masks hold for A = K + beta M and for M, so for every beta (and alike on every level)
+    if (!stencil_masks_cover(h->fin().c) || !stencil_masks_cover(h->mass)) return bail(STOKES_ERR_BAD_ARG);
     *out = h;
     return STOKES_OK;
 }
