@@ -98,8 +98,8 @@ typedef struct stokes_params {
                           and the zero-mean pressure is over the L.  It needs the Uzawa smoother,
                           coarse_level = 1 (the L's level 0) and levels >= 2; with STOKES_MIXED its
                           float32 levels follow tma_level as the square's do, the levels below it that no
-                          cluster takes run the per-phase step; load vectors, Euler right-hand sides and mass products are square-only (they return
-                          STOKES_ERR_BAD_ARG on an L handle) */
+                          cluster takes run the per-phase step; load vectors, Euler right-hand sides and
+                          mass products are square-only (they return STOKES_ERR_BAD_ARG on an L handle) */
     int tma_level;     /* STOKES_MIXED with the Uzawa smoother: the float32 levels
                           k >= tma_level are held in a padded layout whose rows start on 16-byte
                           boundaries and smoothed by a one-kernel step whose tiles arrive by
@@ -343,8 +343,8 @@ stokes_status stokes_residual_norm2_noalloc(int levels, double beta, const doubl
 /* Chooses, for every level of a STOKES_MIXED handle whose size has not been tuned in this process,
  * the fastest float32 Uzawa step variant (one-kernel tiles of several kinds and shapes, or the
  * three-kernel step with several block shapes; on planar levels the planar step variants) by timing
- * each on the handle's buffers; the choice is kept process-wide per level size.  Untuned levels use the three-kernel step below N = 128 and
- * the 32 x 16 fused tile above.  Synchronises the stream. */
+ * each on the handle's buffers; the choice is kept process-wide per level size.  Untuned levels use
+ * the three-kernel step below N = 128 and the 32 x 16 fused tile above.  Synchronises the stream. */
 stokes_status stokes_autotune(stokes_handle* h);
 /* The step variant currently used for a float32 level with `levels` levels (N = 2^levels), -1 if
  * out of range: 0-3 fused tiles 32x16, 32x8, 64x8, 16x16; 4-6 three-kernel step, blocks 32x8, 16x8, 8x8;

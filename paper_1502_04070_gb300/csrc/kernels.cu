@@ -376,10 +376,10 @@ __device__ __forceinline__ T ldv(const T* p) {
     else return *p;
 }
 
-// Strides of the arrays a transfer reads and writes, each pointer at the array's (0, 0) entry: the dense
-// level arrays (dense_layout), the padded shared-memory arrays of the coarse cycle, or float32 levels in the planar layout (template flags PF / PC of the
-// fine / coarse level; there the row stride is in floats, the component stride is 1 and psf / psc is the
-// parity-plane stride).
+// Strides of the arrays a transfer reads and writes, each pointer at the array's (0, 0) entry: the dense level arrays
+// (dense_layout), the padded shared-memory arrays of the coarse cycle, or float32 levels in the planar layout (template
+// flags PF / PC of the fine / coarse level; there the row stride is in floats, the component stride is 1 and psf / psc
+// is the parity-plane stride).
 struct XferLayout {
     int ldf, n2f;   // fine velocity: row stride, component stride
     int ldpf;       // fine vertex array: row stride
@@ -853,7 +853,8 @@ __device__ __forceinline__ void mp_row(int i, int j, int n, const MassCoef<T>& m
 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_load(int n, const __grid_constant__ MassCoef<T> m, const T* __restrict__ fn,
-                                             const T* __restrict__ gn, T* __restrict__ f, T* __restrict__ g, double* __restrict__ partial) {
+                                             const T* __restrict__ gn, T* __restrict__ f, T* __restrict__ g,
+                                             double* __restrict__ partial) {
     CELL_INDEX
     const size_t n2 = (size_t)(2 * n + 1) * (2 * n + 1);
     double wg = 0.0;

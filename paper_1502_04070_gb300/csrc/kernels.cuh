@@ -122,10 +122,11 @@ bool launch_uzawa_tma_variant(int variant, cudaStream_t s, int n, const OpCoef<f
                               float* u_out, float* p_out, const CoarseCorrection& cc = CoarseCorrection{});
 // r = F - A x on a planar level (N = n) and its restriction (fc, gc) = I^T r to the coarse level
 // (planar or not: pc_planar), with the coarse iterate (uc, pc) set to zero, in one kernel on the
-// tiles of the planar step (uc, pc null: the coarse iterate is left alone); the fine defect stays in shared memory.  False (nothing launched) as
-// for launch_uzawa_tma.
+// tiles of the planar step (uc, pc null: the coarse iterate is left alone); the fine defect stays in
+// shared memory.  False (nothing launched) as for launch_uzawa_tma.
 bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& ml,
-                         const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc, float* pc);
+                         const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc,
+                         float* pc);
 // The float32 V- or W-cycle from level `top` (compact layout, top <= kSmallCycleTop) down to the
 // coarsest level clev of the iteration, with its exact solve, in ONE cooperative launch (uzawa_reg.cu):
 // every CTA resident, phases separated by grid barriers whose waits are bounded (about a second; a
@@ -154,7 +155,8 @@ bool tma_tuned(int n);
 bool set_tma_choice(int n, int v);
 // times every planar variant on these planar buffers (contents overwritten) and keeps the fastest
 cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& ml, float tau,
-                               float sigma, float* u, float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out);
+                               float sigma, float* u, float* p, const float* f, const float* g, const float* sinv,
+                               float* u_out, float* p_out);
 unsigned uzawa_tma_timeouts();
 // Does the compile-time structure of the register tile match these coefficients?
 bool reg_tables_match(const OpCoef<float>& c);

@@ -702,18 +702,20 @@ __device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const 
                                            float* __restrict__ u_out, float* __restrict__ p_out) {
     const int UPL = G::upl(TY), FPL = G::fpl(TY), lane = threadIdx.x & 31, h = n >> 1;
     const bool col = h >= i0 - 2 && h < i0 + G::TX + 2, right = i0 >= h;
-    if (zero) zero_phase1<G, NW>(n, TY, i0, j0, q, &ml, sF);
-    else
-    mid_cover(col, right, h, j0 - 2, TY + 4, NW,
-              [&](int cls, int r, int end, int step) {
-                  if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n, mf);
-                  else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n, mf);
-              },
-              [&](int r) {
-                  const int k = mid_class(i0 - 2 + lane, j0 - 2 + r, n);
+    if (zero) {
+        zero_phase1<G, NW>(n, TY, i0, j0, q, &ml, sF);
+    } else {
+        mid_cover(col, right, h, j0 - 2, TY + 4, NW,
+                  [&](int cls, int r, int end, int step) {
+                      if (cls == 0) phase1_fast<G, 0, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n, mf);
+                      else phase1_fast<G, 1, false>(q, sU, UPL, sP, sF, FPL, r, end, step, lane, i0, j0, n, mf);
+                  },
+                  [&](int r) {
+                      const int k = mid_class(i0 - 2 + lane, j0 - 2 + r, n);
 #pragma unroll
-                  for (int s = 0; s < 4; ++s) mid_node<G, true>(ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n, mf);
-              });
+                      for (int s = 0; s < 4; ++s) mid_node<G, true>(ml, k, s, sU, UPL, sP, sF, FPL, r, lane, i0, j0, n, mf);
+                  });
+    }
     __syncthreads();
     mid_cover(col, right, h, j0 - 1, TY + 2, NW,
               [&](int cls, int r, int end, int step) {
@@ -740,9 +742,9 @@ __device__ __forceinline__ void mid_phases(int n, int TY, int i0, int j0, const 
 // the new state of the CTA's cells to (u_out, p_out).
 template <class G, bool PLO, int NW, bool PAIR = false, bool LISTS = false, class MF = NoMask>
 __device__ __forceinline__ void reg_phases(int n, int TY, int i0, int j0, const OpCoef<float>* c, const RegCoef& q,
-                                           const MidLists* ml, bool zero, MF mf, float tau, float sigma, const float2* sU, float2* sF, const float* sP,
-                                           float* sG, const float* sS, float* __restrict__ u_out,
-                                           float* __restrict__ p_out) {
+                                           const MidLists* ml, bool zero, MF mf, float tau, float sigma,
+                                           const float2* sU, float2* sF, const float* sP, float* sG, const float* sS,
+                                           float* __restrict__ u_out, float* __restrict__ p_out) {
     constexpr int TX = G::TX;
     const int UPL = G::upl(TY), FPL = G::fpl(TY);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1202,7 +1204,8 @@ __device__ __forceinline__ void embed_apply(const EmbedJob& jb, int n, int TY, i
     }
     // P1: injection at the coarse vertex, averages halfway along the coarse edges from it
     auto addp = [&](int x, int y, float v) {
-        if (x < pxlo || x >= pxlo + G::PW || y < pylo || y >= pylo + TY + 6 || x > n || y > n || masked(2 * x - 1, 2 * y - 1, mf)) return;
+        if (x < pxlo || x >= pxlo + G::PW || y < pylo || y >= pylo + TY + 6 || x > n || y > n) return;
+        if (masked(2 * x - 1, 2 * y - 1, mf)) return;
         sP[(y - pylo) * G::PW + (x - pxlo)] += v;
     };
     addp(2 * I, 2 * J, jb.p00);
@@ -1514,7 +1517,8 @@ __device__ __forceinline__ void defect_restrict(int n, int TY, int i0, int j0, c
 
 template <int NW, int MINB, bool PC, bool LISTS, class MF>
 __global__ void __launch_bounds__(32 * NW, MINB)
-    k_restrict_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t, const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
+    k_restrict_tma(int n, int TY, TileOrder ord, const __grid_constant__ RowTables<LISTS> t,
+                   const __grid_constant__ RegCoef q, const __grid_constant__ RestrictWeights wt,
                    const __grid_constant__ TmaMaps maps, float* __restrict__ fc, float* __restrict__ gc,
                    float* __restrict__ uc, float* __restrict__ pc, MF mf) {
     using G = TmaTile;
@@ -1818,8 +1822,8 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
             const int i0 = (t % cols) * G::TX, j0 = (t / cols) * TY;
             stage_compact(n, TY, i0, j0, j0 - 1, xu, xp, L.f, L.g, L.sinv, sU, sF, sP, sG, sS);
             __syncthreads();
-            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, false, NoMask{}, A.tau, A.sigma, sU, sF, sP, sG,
-                                           sS, ou, op);
+            reg_phases<G, false, kSmallNW>(n, TY, i0, j0, &sc[lv - A.clev - 1], A.q[lv], nullptr, false, NoMask{}, A.tau,
+                                           A.sigma, sU, sF, sP, sG, sS, ou, op);
             __syncthreads();
         }
         sw[lv] = !sw[lv];
@@ -1847,8 +1851,8 @@ __global__ void __launch_bounds__(32 * kSmallNW, 1) k_small_cycle(const __grid_c
                     stage_compact(n, TY, i0, j0, j0 - 2, sw[l] ? L.tu : L.u, sw[l] ? L.tp : L.p, L.f, L.g, nullptr, sU,
                                   sF, sP, sG, sS);
                     __syncthreads();
-                    defect_restrict<G, kSmallNW, false>(n, TY, i0, j0, &sc[l - A.clev - 1], A.q[l], nullptr, NoMask{}, A.wt, sU, sF, sP, sG,
-                                                        C.f, C.g, C.u, C.p);
+                    defect_restrict<G, kSmallNW, false>(n, TY, i0, j0, &sc[l - A.clev - 1], A.q[l], nullptr, NoMask{},
+                                                        A.wt, sU, sF, sP, sG, C.f, C.g, C.u, C.p);
                     __syncthreads();
                 }
                 sw[l - 1] = false;
@@ -2041,9 +2045,9 @@ bool make_tma_maps(int n, int ty, const float* u, const float* p, const float* f
 }
 
 template <int NW, int MINB, bool PAIR = false>
-bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau, float sigma, const float* u, const float* p,
-                  const float* f, const float* g, const float* sinv, float* u_out, float* p_out, bool prefetch,
-                  const CoarseCorrection& cc) {
+bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau, float sigma,
+                  const float* u, const float* p, const float* f, const float* g, const float* sinv, float* u_out,
+                  float* p_out, bool prefetch, const CoarseCorrection& cc) {
     RegCoef q;
     if (!make_reg_coef(c, tau, q)) return false;
     int ty = tma_rows<NW, MINB, PAIR>(n, pl);
@@ -2075,11 +2079,11 @@ bool launch_tma_v(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLev
         launch_pdl(k_uzawa_tma<8, 3, false, true, QuadrantMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord,
                    RowTables<true>{pl.lists}, q, tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, QuadrantMask{n});
     else if (pl.lists)
-        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, true, NoMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
-                   tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, NoMask{});
+        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, true, NoMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<true>{pl.lists}, q, tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, NoMask{});
     else
-        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, false, NoMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q, tau,
-                   sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, NoMask{});
+        launch_pdl(k_uzawa_tma<NW, MINB, PAIR, false, NoMask>, grid, block, TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<false>{c}, q, tau, sigma, m, u_out, p_out, pf, cc.u, cc.p, cc.planar ? 1 : 0, NoMask{});
     return true;
 }
 
@@ -2124,11 +2128,11 @@ bool launch_rt(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel&
         launch_pdl(k_restrict_tma<8, 3, PC, true, QuadrantMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord,
                    RowTables<true>{pl.lists}, q, restrict_weights(), m, fc, gc, uc, pc, QuadrantMask{n});
     else if (pl.lists)
-        launch_pdl(k_restrict_tma<8, 3, PC, true, NoMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<true>{pl.lists}, q,
-                   restrict_weights(), m, fc, gc, uc, pc, NoMask{});
+        launch_pdl(k_restrict_tma<8, 3, PC, true, NoMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<true>{pl.lists}, q, restrict_weights(), m, fc, gc, uc, pc, NoMask{});
     else
-        launch_pdl(k_restrict_tma<8, 3, PC, false, NoMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord, RowTables<false>{c}, q,
-                   restrict_weights(), m, fc, gc, uc, pc, NoMask{});
+        launch_pdl(k_restrict_tma<8, 3, PC, false, NoMask>, grid, dim3(256), TmaTile::bytes(ty), s, n, ty, ord,
+                   RowTables<false>{c}, q, restrict_weights(), m, fc, gc, uc, pc, NoMask{});
     return true;
 }
 
@@ -2182,7 +2186,8 @@ cudaError_t launch_small_cycle(cudaStream_t s, const SmallCycleHost& h) {
 }
 
 bool launch_restrict_tma(cudaStream_t s, int n, bool pc_planar, const OpCoef<float>& c, const PlanarLevel& pl,
-                         const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc, float* pc) {
+                         const float* u, const float* p, const float* f, const float* g, float* fc, float* gc, float* uc,
+                         float* pc) {
     return pc_planar ? launch_rt<true>(s, n, c, pl, u, p, f, g, fc, gc, uc, pc)
                      : launch_rt<false>(s, n, c, pl, u, p, f, g, fc, gc, uc, pc);
 }
@@ -2241,7 +2246,8 @@ bool launch_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const Plana
                       const float* u, const float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out,
                       const CoarseCorrection& cc) {
     // the L has one variant, and so have steps from zero
-    return launch_uzawa_tma_variant(pl.dom == kDomL ? 0 : pl.zero ? 1 : g_tma_choice[pl.lists == nullptr][lvl(n)], s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
+    const int variant = pl.dom == kDomL ? 0 : pl.zero ? 1 : g_tma_choice[pl.lists == nullptr][lvl(n)];
+    return launch_uzawa_tma_variant(variant, s, n, c, pl, tau, sigma, u, p, f, g, sinv, u_out, p_out, cc);
 }
 
 bool uzawa_tma_embed_available() { return uzawa_tma_available() && embed_table_matches(); }
@@ -2263,7 +2269,8 @@ bool set_tma_choice(int n, int v) {
 }
 
 cudaError_t autotune_uzawa_tma(cudaStream_t s, int n, const OpCoef<float>& c, const PlanarLevel& pl, float tau,
-                               float sigma, float* u, float* p, const float* f, const float* g, const float* sinv, float* u_out, float* p_out) {
+                               float sigma, float* u, float* p, const float* f, const float* g, const float* sinv,
+                               float* u_out, float* p_out) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return cudaErrorUnknown;
     if (cudaEventCreate(&e1) != cudaSuccess) {
