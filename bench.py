@@ -80,7 +80,7 @@ def parse():
                     help="kernel modes: lowest planar float32 level (0: the library default; 14: none)")
     ap.add_argument("--planar-variant", type=int, default=None, help="kernel modes: force this planar step variant")
     ap.add_argument("--coop-level", type=int, default=0,
-                    help="kernel modes: highest level of the cooperative small-level cycle (0: off)")
+                    help="kernel modes: highest level of the cooperative small-level cycle (0: the cluster, -1: launches)")
     ap.add_argument("--batch-count", type=int, default=256)
     ap.add_argument("--reps", type=int, default=5)
     ap.add_argument("--host-loop", action="store_true",

@@ -141,7 +141,7 @@ typedef struct stokes_report {
  * `stream` (the handle's cudaStream_t), or NULL on failure (the setup then returns STOKES_ERR_OOM);
  * release frees a block that alloc returned, with the same bytes and stream.  ctx is passed through.
  * The callbacks are called only inside stokes_setup, stokes_batch_setup, stokes_euler_rhs (its first
- * call) and the destroy calls, on the calling thread. */
+ * call), stokes_euler_run, stokes_batch_euler_run and the destroy calls, on the calling thread. */
 typedef void* (*stokes_alloc_fn)(size_t bytes, void* stream, void* ctx);
 typedef void (*stokes_free_fn)(void* ptr, size_t bytes, void* stream, void* ctx);
 

@@ -22,10 +22,11 @@
 // float64 a warp instruction occupies its pipe for 64 clocks, so the work has to be spread over many
 // warps.  Items are ordered node by node: the warps of a phase have the same number of entries.
 //
-// Measured (GB300, whole calls): a float64 V(3,3) cycle at h = 1/32 264 us against 1752 us with a launch per
-// phase, a mixed-precision solve with W-cycles at h = 1/512 37.6 against 64.0 ms, an implicit Euler step there 10.9
-// against 17.1 ms with levels 0-4 in one CTA and level 5 by launches; the float32 levels 1-5 take 91 us a
-// V-cycle (105 phases; before, 283 us for levels 1-4 alone), the float64 levels 1-4 176 us (float64 pipe).
+// Measured (GB300, whole calls) against a launch per phase, or levels 0-4 in one CTA where that served: by this kernel
+// alone a float64 V(3,3) cycle at h = 1/32 264 us against 1752 us and a mixed-precision solve with W-cycles at h = 1/512
+// 37.6 against 64.0 ms; with what changed since 231 us and 34.2 ms, three implicit Euler steps there 25.7 against 51.6 ms.
+// The float32 levels 1-5 take 91 us a V-cycle (105 phases; before, 283 us for levels 1-4 alone), the float64 levels 1-4
+// 176 us (float64 pipe).
 //
 // A launch executes a list of operations that the host recursion writes: V- or W-cycle,
 // coarsest level 0 (27 x 27 inverse), 1 or 2 (dense inverse, rows over the cluster).  With coarsest level
